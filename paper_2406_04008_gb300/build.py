@@ -29,7 +29,7 @@ def _nvcc():
 
 def _deps():
     return [os.path.join(CSRC, s) for s in SOURCES] + [
-        os.path.join(CSRC, "internal.h"), os.path.join(INCLUDE, "collage.h")]
+        os.path.join(CSRC, "edt.h"), os.path.join(CSRC, "internal.h"), os.path.join(INCLUDE, "collage.h")]
 
 
 def _fresh(lib):

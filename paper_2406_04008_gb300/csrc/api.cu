@@ -94,7 +94,7 @@ struct collage_s {
   int sched_start = -1;
   // quality-metric scratch (allocated by collage_metrics)
   uint8_t* met_obj = nullptr;
-  int* met_gcol = nullptr;
+  unsigned short* met_gcol = nullptr;
   unsigned long long* met_cnt = nullptr;  // [5 * P]: 4 counts, then the distance sums
   // skeleton-based initialisation scratch (allocated by collage_mat_init)
   unsigned char* mat_buf = nullptr;
@@ -1699,7 +1699,7 @@ extern "C" collage_status collage_metrics(collage_t h, void* stream, double* h_m
     h->met_gcol = nullptr;
     h->met_pix = 0;
     CK(h, cudaMalloc(&h->met_obj, np));
-    CK(h, cudaMalloc(&h->met_gcol, sizeof(int) * np));
+    CK(h, cudaMalloc(&h->met_gcol, sizeof(unsigned short) * np));
     h->met_pix = np;
   }
   if (!h->met_cnt) CK(h, cudaMalloc(&h->met_cnt, sizeof(unsigned long long) * 5 * h->P));

@@ -304,7 +304,7 @@ struct RasterOcc {
 };
 void raster_occupancy(int tile, int emit_threads, RasterOcc* o);
 // quality metrics after a render pass: counts [4 * n_probs] and squared-distance sums [n_probs]
-cudaError_t launch_metrics(const Dev& d, cudaStream_t s, uint8_t* obj, int* gcol,
+cudaError_t launch_metrics(const Dev& d, cudaStream_t s, uint8_t* obj, unsigned short* gcol,
                            unsigned long long* cnt, unsigned long long* sums, int max_res);
 
 }  // namespace collage

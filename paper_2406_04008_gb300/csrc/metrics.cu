@@ -9,12 +9,17 @@
 // distance (unit coordinates) from the pixel centre to the nearest object pixel centre.  All
 // counts and squared distances are integers, summed exactly.
 #include "collage.h"
+#include "edt.h"
 #include "internal.h"
 
 namespace collage {
 
 constexpr int kMetWarps = 4;
-constexpr int kMetFar = 1 << 20;  // "no object pixel in this column" (rows)
+
+struct ObjectSite {
+  const uint8_t* obj;
+  __device__ __forceinline__ bool operator()(long long pix) const { return obj[pix] != 0; }
+};
 
 // Counts per problem: cnt[4p + 0] object in shape, [1] shape, [2] overlap, [3] object outside the
 // shape; obj[pix] = 1 for an object pixel.  One tile per warp.
@@ -69,64 +74,43 @@ __global__ void __launch_bounds__(kMetWarps * 32) k_metric_counts(Dev d, uint8_t
   }
 }
 
-// Column pass of the distance transform: rows to the nearest object pixel of the same column.
-__global__ void k_metric_cols(Dev d, const uint8_t* obj, int* gcol, int max_res) {
-  const int p = blockIdx.y, k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int res = d.prob_res[p];
-  if (k >= res || k >= max_res) return;
-  const long long pb = d.prob_pix_base[p];
-  int last = -kMetFar;
-  for (int i = 0; i < res; ++i) {
-    const long long pix = pb + (long long)i * res + k;
-    if (obj[pix]) last = i;
-    gcol[pix] = last > -kMetFar ? i - last : kMetFar;
-  }
-  last = kMetFar + res;
-  for (int i = res - 1; i >= 0; --i) {
-    const long long pix = pb + (long long)i * res + k;
-    if (obj[pix]) last = i;
-    if (last - i < gcol[pix]) gcol[pix] = last - i;
-  }
-}
-
-// Row pass, one row per warp: for each non-object shape pixel the squared distance to the nearest
-// object pixel is the minimum over the columns k of (j - k)^2 + gcol(i, k)^2; the sum over the
-// row goes to sums[p] (exact 64-bit integers).
-__global__ void __launch_bounds__(kMetWarps * 32) k_metric_rows(Dev d, const uint8_t* obj, const int* gcol,
-                                                              unsigned long long* sums, int max_res) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int p = blockIdx.y, i = blockIdx.x * kMetWarps + wid;
-  const int res = d.prob_res[p];
-  if (i >= res || i >= max_res) return;
+// Row pass, one row per block: for each non-object shape pixel the squared distance to the nearest
+// object pixel; the row's sum goes to sums[p] (exact 64-bit integers).
+__global__ void __launch_bounds__(kEdtRowThreads) k_metric_rows(Dev d, const unsigned short* g, unsigned long long* sums) {
+  extern __shared__ unsigned s_g2[];
+  const int p = blockIdx.y, i = blockIdx.x, res = d.prob_res[p];
+  if (i >= res) return;
   const long long rowb = d.prob_pix_base[p] + (long long)i * res;
+  edt_stage_row(g + rowb, res, s_g2);
+  __syncthreads();
   unsigned long long acc = 0;
-  for (int j = lane; j < res; j += 32) {
-    if (obj[rowb + j] || !(d.covc[rowb + j] >= 0.5f)) continue;
-    long long best = (long long)kMetFar * kMetFar;
-    for (int k = 0; k < res; ++k) {
-      const long long g = gcol[rowb + k];
-      const long long dj = j - k;
-      const long long d2 = dj * dj + g * g;
-      best = d2 < best ? d2 : best;
-    }
-    if (best < (long long)kMetFar * kMetFar) acc += (unsigned long long)best;
+  for (int j = threadIdx.x; j < res; j += kEdtRowThreads) {
+    // (an object pixel is its column's own site)
+    if (s_g2[j] == 0u || !(d.covc[rowb + j] >= 0.5f)) continue;
+    const unsigned best = edt_search(s_g2, res, j, kEdtFar2);
+    if (best < kEdtFar2) acc += best;
   }
   for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0 && acc) atomicAdd(&sums[p], acc);
+  if ((threadIdx.x & 31) == 0 && acc) atomicAdd(&sums[p], acc);
 }
 
-cudaError_t launch_metrics(const Dev& d, cudaStream_t s, uint8_t* obj, int* gcol,
+cudaError_t launch_metrics(const Dev& d, cudaStream_t s, uint8_t* obj, unsigned short* gcol,
                            unsigned long long* cnt, unsigned long long* sums, int max_res) {
   cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 4 * d.n_probs, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * d.n_probs, s);
+  const size_t cs = edt_col_smem(max_res), rs = edt_row_smem(max_res);
+  if (e == cudaSuccess && cs > 48 * 1024)
+    e = cudaFuncSetAttribute(k_edt_cols<ObjectSite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+  if (e == cudaSuccess && rs > 48 * 1024)
+    e = cudaFuncSetAttribute(k_metric_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
   if (e != cudaSuccess) return e;
   const int tgrid = (d.total_tiles + kMetWarps - 1) / kMetWarps;
   if (d.tile == 8) k_metric_counts<8><<<tgrid, kMetWarps * 32, 0, s>>>(d, obj, cnt);
   else if (d.tile == 16) k_metric_counts<16><<<tgrid, kMetWarps * 32, 0, s>>>(d, obj, cnt);
   else return cudaErrorInvalidValue;
-  k_metric_cols<<<dim3((max_res + 127) / 128, d.n_probs), 128, 0, s>>>(d, obj, gcol, max_res);
-  k_metric_rows<<<dim3((max_res + kMetWarps - 1) / kMetWarps, d.n_probs), kMetWarps * 32, 0, s>>>(
-      d, obj, gcol, sums, max_res);
+  k_edt_cols<<<dim3((max_res + kEdtCols - 1) / kEdtCols, d.n_probs), kEdtThreads, cs, s>>>(
+      d, ObjectSite{obj}, gcol, 0);
+  k_metric_rows<<<dim3(max_res, d.n_probs), kEdtRowThreads, rs, s>>>(d, gcol, sums);
   return cudaGetLastError();
 }
 
