@@ -1663,7 +1663,8 @@ extern "C" collage_status collage_mat_init(collage_t h, void* stream, int* d_axi
   cudaStream_t s = (cudaStream_t)stream;
   const size_t np = (size_t)h->d.total_pix, al = 256;
   auto up = [&](size_t b) { return (b + al - 1) / al * al; };
-  // gcol, D2, candidates, clearances (4 B per pixel each), placement order, candidate counts
+  // column distances (then the candidates' coordinates), D2, candidates, clearances (4 B per pixel
+  // each), the elements' placed marks, candidate counts
   const size_t need = 4 * up(4 * np) + up(sizeof(int) * (size_t)h->N) + up(sizeof(int) * (size_t)h->P);
   if (need > h->mat_bytes) {
     CK(h, cudaDeviceSynchronize());
@@ -1674,16 +1675,16 @@ extern "C" collage_status collage_mat_init(collage_t h, void* stream, int* d_axi
     h->mat_bytes = need;
   }
   unsigned char* b = h->mat_buf;
-  int* gcol = reinterpret_cast<int*>(b);
+  unsigned* gcol = reinterpret_cast<unsigned*>(b);
   unsigned* d2 = reinterpret_cast<unsigned*>(b + up(4 * np));
-  int* cand = reinterpret_cast<int*>(b + 2 * up(4 * np));
+  unsigned* cand = reinterpret_cast<unsigned*>(b + 2 * up(4 * np));
   float* clear = reinterpret_cast<float*>(b + 3 * up(4 * np));
-  int* order = reinterpret_cast<int*>(b + 4 * up(4 * np));
+  int* placed = reinterpret_cast<int*>(b + 4 * up(4 * np));
   int* n_cand = reinterpret_cast<int*>(b + 4 * up(4 * np) + up(sizeof(int) * (size_t)h->N));
   CK(h, launch_adam_flush(h->d, s));  // a pending step belongs to the old params
   int max_res = 1;
   for (int p = 0; p < h->P; ++p) max_res = std::max(max_res, h->res[p]);
-  CK(h, launch_mat_init(h->d, s, max_res, gcol, d2, cand, n_cand, clear, order, d_axis, d_width));
+  CK(h, launch_mat_init(h->d, s, max_res, gcol, d2, cand, n_cand, clear, placed, d_axis, d_width));
   return COLLAGE_OK;
 }
 

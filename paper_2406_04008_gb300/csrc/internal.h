@@ -288,8 +288,8 @@ cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out = nullptr
 // only flattens
 cudaError_t launch_ctrl_step(const Dev& d, cudaStream_t s, int mode);
 // skeleton-based initialisation: distance transform, medial axis, greedy placement into d.q
-cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, int* gcol, unsigned* d2,
-                            int* cand, int* n_cand, float* clear, int* order, int* axis_out,
+cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
+                            unsigned* cand, int* n_cand, float* clear, int* placed, int* axis_out,
                             float* width_out);
 cudaError_t launch_loss(const Dev& d, cudaStream_t s);
 // the captured level schedule: records the step count at the start of a run; sets a level's loop

@@ -17,363 +17,410 @@
 //    so every decision is reproducible.  The element's translation becomes its pixel centre;
 //    rotation and scale are kept.
 #include <cfloat>
-#include <cooperative_groups.h>
 
 #include "collage.h"
+#include "edt.h"
 #include "internal.h"
 
 namespace collage {
 
-namespace cg = cooperative_groups;
+struct OutsideSite {  // outside pixels of the container raster
+  const float* covc;
+  __device__ __forceinline__ bool operator()(long long pix) const { return !(covc[pix] >= 0.5f); }
+};
 
-constexpr int kMatWarps = 4;
-constexpr int kPlaceThreads = 512;
-constexpr int kPlaceCluster = 8;  // blocks (one thread-block cluster) per problem
-
-__device__ __forceinline__ bool inside_px(const Dev& d, long long pix) { return d.covc[pix] >= 0.5f; }
-
-// Column pass: rows to the nearest outside pixel of the same column (rows -1 and res are outside).
-__global__ void k_mat_cols(Dev d, int* gcol, int max_res) {
-  const int p = blockIdx.y, k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int res = d.prob_res[p];
-  if (k >= res || k >= max_res) return;
-  const long long pb = d.prob_pix_base[p];
-  // rows in groups of 8 whose coverages are read together (the loads are independent; only the
-  // running index of the last outside pixel carries from row to row)
-  constexpr int G = 8;
-  int last = -1;
-  for (int i0 = 0; i0 < res; i0 += G) {
-    bool out[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) out[u] = i0 + u < res && !inside_px(d, pb + (long long)(i0 + u) * res + k);
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-      if (i0 + u >= res) break;
-      if (out[u]) last = i0 + u;
-      gcol[pb + (long long)(i0 + u) * res + k] = i0 + u - last;
-    }
-  }
-  last = res;
-  for (int i1 = res - 1; i1 >= 0; i1 -= G) {
-    bool out[G];
-    int g[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-      const int i = i1 - u;
-      out[u] = i >= 0 && !inside_px(d, pb + (long long)i * res + k);
-      g[u] = i >= 0 ? gcol[pb + (long long)i * res + k] : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-      const int i = i1 - u;
-      if (i < 0) break;
-      if (out[u]) last = i;
-      if (last - i < g[u]) gcol[pb + (long long)i * res + k] = last - i;
-    }
-  }
-}
-
-// Row pass, one row per warp: D2 = min over the columns k in [-1, res] of (j - k)^2 + g(k)^2, with
+// Row pass, one row per block: D2 = min over the columns k in [-1, res] of (j - k)^2 + g(k)^2, with
 // g = 0 in the two columns beyond the image; 0 for outside pixels.
-__global__ void __launch_bounds__(kMatWarps * 32) k_mat_rows(Dev d, const int* gcol, unsigned* d2,
-                                                             int max_res) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int p = blockIdx.y, i = blockIdx.x * kMatWarps + wid;
-  const int res = d.prob_res[p];
-  if (i >= res || i >= max_res) return;
+__global__ void __launch_bounds__(kEdtRowThreads) k_mat_rows(Dev d, const unsigned short* g, unsigned* d2) {
+  extern __shared__ unsigned s_g2[];
+  const int p = blockIdx.y, i = blockIdx.x, res = d.prob_res[p];
+  if (i >= res) return;
   const long long rowb = d.prob_pix_base[p] + (long long)i * res;
-  for (int j = lane; j < res; j += 32) {
-    if (!inside_px(d, rowb + j)) {
-      d2[rowb + j] = 0u;
-      continue;
+  edt_stage_row(g + rowb, res, s_g2);
+  __syncthreads();
+  for (int j = threadIdx.x; j < res; j += kEdtRowThreads) {
+    unsigned v = 0u;
+    if (s_g2[j] != 0u) {  // an inside pixel (g = 0 is an outside pixel itself)
+      const unsigned left = (unsigned)(j + 1) * (unsigned)(j + 1), right = (unsigned)(res - j) * (unsigned)(res - j);
+      v = edt_search(s_g2, res, j, min(left, right));
     }
-    long long best = (long long)(j + 1) * (j + 1);
-    const long long right = (long long)(res - j) * (res - j);
-    if (right < best) best = right;
-    for (int k = 0; k < res; ++k) {
-      const long long g = gcol[rowb + k], dj = j - k;
-      const long long v = dj * dj + g * g;
-      best = v < best ? v : best;
-    }
-    d2[rowb + j] = (unsigned)best;
+    d2[rowb + j] = v;
   }
 }
 
-// Medial axis test per pixel; the axis pixels are appended to their problem's candidate list
-// (in no particular order: the placement orders them by key).
-__global__ void k_mat_axis(Dev d, const unsigned* d2, int* cand, int* n_cand, int* axis_out,
-                           float* width_out) {
-  const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= d.total_pix) return;
-  int p = 0, lo = 0, hi = d.n_probs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (d.prob_pix_base[mid] <= pix) lo = mid;
-    else hi = mid - 1;
-  }
-  p = lo;
+// Medial axis test per pixel, one warp per 32 columns of a row; the axis pixels are appended to their
+// problem's candidate list, packed x | y << 16, with one atomic per warp (in no particular order: the
+// placement orders them by key).
+constexpr int kAxisThreads = 128;
+__global__ void __launch_bounds__(kAxisThreads) k_mat_axis(Dev d, const unsigned* d2, unsigned* cand, int* n_cand,
+                                                           int* axis_out, float* width_out) {
+  const int p = blockIdx.z, y = blockIdx.y, res = d.prob_res[p];
+  const int x = blockIdx.x * kAxisThreads + threadIdx.x, lane = threadIdx.x & 31;
+  if (y >= res || x - lane >= res) return;  // warp-uniform
   const long long pb = d.prob_pix_base[p];
-  const int res = d.prob_res[p];
-  const int local = (int)(pix - pb), y = local / res, x = local % res;
-  const unsigned a = d2[pix];
   auto at = [&](int xx, int yy) -> unsigned {
     return xx < 0 || yy < 0 || xx >= res || yy >= res ? 0u : d2[pb + (long long)yy * res + xx];
   };
+  const unsigned a = at(x, y);
   bool axis = false;
   if (a > 0) {
     const int dirs[4][2] = {{1, 0}, {0, 1}, {1, 1}, {1, -1}};
-    for (int k = 0; k < 4 && !axis; ++k) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
       const unsigned u = at(x + dirs[k][0], y + dirs[k][1]), v = at(x - dirs[k][0], y - dirs[k][1]);
-      axis = a >= u && a >= v && (a > u || a > v);
+      axis |= a >= u && a >= v && (a > u || a > v);
     }
   }
-  if (axis) cand[pb + atomicAdd(&n_cand[p], 1)] = local;
+  const unsigned bal = __ballot_sync(0xffffffffu, axis);
+  if (bal != 0u) {
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&n_cand[p], __popc(bal));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (axis) cand[pb + base + __popc(bal & ((1u << lane) - 1u))] = (unsigned)x | (unsigned)y << 16;
+  }
+  if (x >= res) return;
+  const long long pix = pb + (long long)y * res + x;
   if (axis_out) axis_out[pix] = axis ? 1 : 0;
   if (width_out) width_out[pix] = a > 0 ? sqrtf((float)a) : 0.0f;
-}
-
-__device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* s) {
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = w > v ? w : v;
-  }
-  __syncthreads();  // the previous reduction's readers are done
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    v = threadIdx.x < (blockDim.x >> 5) ? s[threadIdx.x] : 0ull;
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-      v = w > v ? w : v;
-    }
-    if (threadIdx.x == 0) s[0] = v;
-  }
-  __syncthreads();
-  return s[0];
-}
-
-// The block's maxima of two keys in one reduction.
-__device__ __forceinline__ void block_max2(unsigned long long& a, unsigned long long& b, unsigned long long (*s)[2]) {
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long wa = __shfl_xor_sync(0xffffffffu, a, o);
-    const unsigned long long wb = __shfl_xor_sync(0xffffffffu, b, o);
-    a = wa > a ? wa : a;
-    b = wb > b ? wb : b;
-  }
-  __syncthreads();  // the previous reduction's readers are done
-  if ((threadIdx.x & 31) == 0) {
-    s[threadIdx.x >> 5][0] = a;
-    s[threadIdx.x >> 5][1] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const bool in = threadIdx.x < (blockDim.x >> 5);
-    a = in ? s[threadIdx.x][0] : 0ull;
-    b = in ? s[threadIdx.x][1] : 0ull;
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long wa = __shfl_xor_sync(0xffffffffu, a, o);
-      const unsigned long long wb = __shfl_xor_sync(0xffffffffu, b, o);
-      a = wa > a ? wa : a;
-      b = wb > b ? wb : b;
-    }
-  }
 }
 
 // A float's bits as an unsigned key with the float's order (negative values included).
 __device__ __forceinline__ unsigned ordered(float f) {
   const unsigned u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return u ^ ((unsigned)((int)u >> 31) | 0x80000000u);
 }
 
-// Greedy placement, one thread-block cluster of kPlaceCluster blocks per problem.  Block 0 first
-// ranks the elements by radius (ties: lower index) into order[]; every block then gathers its
-// share of the axis pixels (D2, packed coordinates, clearance) into dynamic shared memory (else
-// into cand, gxy and clear); each step is one pass of every block over its share: the clearances
-// take the previous element's disk into account and the block reduces its two candidates (the
-// widest pixel with room, the pixel of largest clearance); after one cluster barrier every block
-// reads the cluster's partials from the blocks' shared memory (double-buffered by step parity, so
-// one barrier a step suffices) and takes the same choice; block 0 writes the translation.  Every
-// block runs the same steps and barriers, and a last barrier keeps each block's shared memory
-// alive until the others have read it.
-constexpr int kPlaceRankMax = 4096;                // elements ranked in shared memory (more: a
-                                                   // reduction per step)
-constexpr int kPlaceSmemCandBytes = 160 * 1024;    // candidates of a placement block (D2,
-constexpr int kPlaceSmemCands = kPlaceSmemCandBytes / 12;  // coordinates, clearance)
-// then, for the ranked elements, each step's element and radius
-constexpr int kPlaceSmem = kPlaceSmemCandBytes + kPlaceRankMax * 8;
-static_assert(kPlaceSmemCandBytes >= kPlaceRankMax * 8, "the ranking keys share the candidates' space");
+// The warp's largest value (no NaN).
+__device__ __forceinline__ float warp_maxf(float v) {
+  float m;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+  return m;
+}
+
+// The warp's largest (hi, lo) pair.
+__device__ __forceinline__ void warp_max2(unsigned& hi, unsigned& lo) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, hi);
+  lo = __reduce_max_sync(0xffffffffu, hi == m ? lo : 0u);
+  hi = m;
+}
+
+// Greedy placement, one block per problem.  The elements' order is fixed before the first step
+// (sorted by radius), and each step chooses one axis pixel (a candidate), so the steps are a serial
+// chain: what bounds this kernel is the latency of one step, not the candidates' arithmetic.
+//
+// The candidates are sorted by cell of the raster and taken in groups of 32, each owned by one lane of
+// one warp for the whole run.  A lane keeps its group's box, largest clearance, widest pixel with
+// room, and the largest clearance among the wider ones without room.  A step then touches only the
+// groups whose choice can have changed (12 of 500 on average for 1000 elements in the annulus at
+// 1024^2):
+//  - those the previous element's disk can reach: the distance from the disk's centre to the group's
+//    box is below the group's largest clearance plus the disk's radius;
+//  - those where a wider pixel gains room because the radius has shrunk.
+// In a group the pixels are in order of their key (D2, then the lower pixel), so the widest with room
+// is the first set bit of a ballot.  The warps' choices meet in one double-buffered exchange and one
+// barrier a step, and every warp reduces them by itself.  1000 elements on 16 k candidates: 0.05 ms to
+// sort and 0.7 us a step, 0.55 us once the first disks are placed (eight clustered blocks that scanned
+// every candidate at each step, with 64-bit shuffle reductions and a cluster barrier: 2.2 us a step).
+// Sixteen warps: with 32 the barrier and the shared issue slots cost more than the fewer groups a
+// warp looks at save.
+constexpr int kPlaceThreads = 512;
+constexpr int kPlaceWarps = kPlaceThreads / 32;
+constexpr int kPlaceRankMax = 4096;        // elements sorted in shared memory (more: a reduction per step)
+constexpr int kPlaceCells = 32;            // cells a side of the candidates' spatial order
+constexpr int kPlaceFast = kPlaceThreads;  // groups kept one per lane, their pixels in shared memory
+constexpr int kPlaceSmem = 221 * 1024;     // keys and candidates (else in global memory)
 
 __device__ __forceinline__ unsigned long long elem_key(const Dev& d, int e, float fres) {
   const float r = __fmul_rn(__fmul_rn(d.elem_rbin[e], d.q[e].w), fres);
   return ((unsigned long long)__float_as_uint(r) << 32) | (0xffffffffu - (unsigned)e);
 }
 
-__global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, int* cand, const int* n_cand,
-                                                             const unsigned* d2, float* clear, int* gxy,
-                                                             int* order) {
-  extern __shared__ __align__(16) unsigned char s_dyn[];
-  __shared__ unsigned long long s_red[kPlaceThreads / 32];
-  __shared__ unsigned long long s_red2[kPlaceThreads / 32][2];
-  __shared__ unsigned long long s_part[2][2];  // per step parity: (widest with room, largest clearance)
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int p = blockIdx.x / kPlaceCluster;
-  const int res = d.prob_res[p], nc = n_cand[p];
-  const long long pb = d.prob_pix_base[p];
-  const int e0 = d.prob_elem_base[p], e1 = d.prob_elem_base[p + 1], ne = e1 - e0;
-  if (nc == 0) return;  // no inside pixel: the params stay (every block of the cluster leaves here)
-  const float fres = (float)res;
-  // the elements in placement order: decreasing key (radius bits, then the lower index)
-  const bool ranked = ne <= kPlaceRankMax;
-  if (rank == 0) {
-    if (ranked) {
-      unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_dyn);
-      for (int i = threadIdx.x; i < ne; i += kPlaceThreads) s_key[i] = elem_key(d, e0 + i, fres);
-      __syncthreads();
-      for (int i = threadIdx.x; i < ne; i += kPlaceThreads) {
-        const unsigned long long k = s_key[i];
-        int rnk = 0;
-        for (int j = 0; j < ne; ++j) rnk += s_key[j] > k ? 1 : 0;
-        order[e0 + rnk] = e0 + i;
-      }
-    } else {
-      for (int i = threadIdx.x; i < ne; i += kPlaceThreads) order[e0 + i] = 0;  // 0: not placed yet
-    }
-    __threadfence();
-  }
-  cluster.sync();  // order[] is complete (and block 0's keys' space is free)
-  int* s_ord = reinterpret_cast<int*>(s_dyn + kPlaceSmemCandBytes);
-  float* s_rad = reinterpret_cast<float*>(s_dyn + kPlaceSmemCandBytes + 4 * kPlaceRankMax);
-  if (ranked)
-    for (int i = threadIdx.x; i < ne; i += kPlaceThreads) {
-      const int e = order[e0 + i];
-      s_ord[i] = e;
-      s_rad[i] = __fmul_rn(__fmul_rn(d.elem_rbin[e], d.q[e].w), fres);
-    }
-  // this block's share of the candidates: D2, x | y << 16, the clearance
-  const int c_lo = (int)((long long)nc * rank / kPlaceCluster);
-  const int mc = (int)((long long)nc * (rank + 1) / kPlaceCluster) - c_lo;
-  const bool in_smem = mc <= kPlaceSmemCands;
-  unsigned* cd2 = in_smem ? reinterpret_cast<unsigned*>(s_dyn) : reinterpret_cast<unsigned*>(cand + pb + c_lo);
-  int* cxy = in_smem ? reinterpret_cast<int*>(s_dyn + 4 * kPlaceSmemCands) : gxy + pb + c_lo;
-  float* ccl = in_smem ? reinterpret_cast<float*>(s_dyn + 8 * kPlaceSmemCands) : clear + pb + c_lo;
-  for (int c = threadIdx.x; c < mc; c += kPlaceThreads) {
-    const int idx = cand[pb + c_lo + c];
-    const unsigned w = d2[pb + idx];
-    cd2[c] = w;
-    cxy[c] = (idx % res) | ((idx / res) << 16);
-    ccl[c] = FLT_MAX;
-  }
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* s) {
+  unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+  warp_max2(hi, lo);
+  __syncthreads();  // the previous reduction's readers are done
+  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = ((unsigned long long)hi << 32) | lo;
   __syncthreads();
+  v = s[threadIdx.x % kPlaceWarps];
+  hi = (unsigned)(v >> 32);
+  lo = (unsigned)v;
+  warp_max2(hi, lo);
+  return ((unsigned long long)hi << 32) | lo;
+}
+
+// What a lane keeps of a group.  Its best pixel's key puts those with room before the others: 0xd0000000
+// + D2 (below 2^28 for a side of at most 32768) with room, else the clearance's ordered bits, which are
+// below 0xc8000000 for any distance on the raster (FLT_MAX, before the first disk, is held down to
+// 0xcfffffff); the lower pixel wins ties (its complement is the larger).
+struct PlaceGroup {
+  float x0, x1, y0, y1;  // the box of its pixels
+  float cl;              // the largest clearance
+  float nx;              // the largest clearance among the pixels wider than the widest with room
+  unsigned key, pix;     // the best pixel's key and its complement
+};
+constexpr unsigned kRoomKey = 0xd0000000u;
+
+// FAST: the candidates in shared memory and at most one group per lane; else both in global memory.
+template <bool FAST>
+__device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, unsigned long long* s_key,
+                            unsigned* cxy, float* ccl, const unsigned* cd2, PlaceGroup* groups, const unsigned* d2,
+                            int* placed) {
+  __shared__ unsigned long long s_red[kPlaceWarps];
+  __shared__ uint2 s_part[2][kPlaceWarps];  // per step parity: each warp's best (key, pixel)
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, ng = (nc + 31) / 32;
+  const int res = d.prob_res[p], e0 = d.prob_elem_base[p];
+  const long long pb = d.prob_pix_base[p];
+  const float fres = (float)res;
+  PlaceGroup own{};  // FAST: the lane's group (key 0 when it has none)
+  const bool has_own = FAST && lane * kPlaceWarps + wid < ng;
+  if (has_own) own = groups[lane * kPlaceWarps + wid];
+  uint2 best = make_uint2(0u, 0u);  // the warp's best
+  unsigned* s_key32 = reinterpret_cast<unsigned*>(s_key);  // (element, radius bits) of each step
+  unsigned r_bits = ranked ? s_key32[1] : 0u;
   int px = 0, py = 0;  // the previous element's pixel and radius (none before the first step)
-  float pr = -1.0f;
+  float pr = -1.0f, r_last = 0.0f;
   for (int step = 0; step < ne; ++step) {
-    int e;
-    float r;
-    if (ranked) {
-      e = s_ord[step];
-      r = s_rad[step];
-    } else {  // the largest element not yet placed, by a reduction (the same in every block)
+    unsigned e_inv = 0u;
+    if (!ranked) {  // the largest element not yet placed, by a reduction
       unsigned long long ek = 0;
-      for (int i = threadIdx.x; i < ne; i += kPlaceThreads) {
-        if (order[e0 + i]) continue;
+      for (int i = tid; i < ne; i += kPlaceThreads) {
+        if (placed[e0 + i]) continue;
         const unsigned long long k = elem_key(d, e0 + i, fres);
         ek = k > ek ? k : ek;
       }
       ek = block_max(ek, s_red);
-      e = (int)(0xffffffffu - (unsigned)(ek & 0xffffffffu));
-      r = __fmul_rn(__fmul_rn(d.elem_rbin[e], d.q[e].w), fres);
+      r_bits = (unsigned)(ek >> 32);
+      e_inv = (unsigned)ek;
     }
-    // one pass: the previous element's disk into the clearances, then the widest axis pixel with
-    // clearance >= r (key: D2, then the lower pixel index), and the largest clearance as fallback
-    unsigned long long ck = 0, fk = 0;
-    for (int c = threadIdx.x; c < mc; c += kPlaceThreads) {
-      const int xy = cxy[c], x = xy & 0xffff, y = xy >> 16;
-      float cl = ccl[c];
-      if (pr >= 0.0f) {
-        const int dx = x - px, dy = y - py;
-        const float dist = __fsub_rn(sqrtf(__int2float_rn(dx * dx + dy * dy)), pr);
-        if (dist < cl) {
-          cl = dist;
-          ccl[c] = cl;
+    const float r = __uint_as_float(r_bits);
+    // the groups' choices hold for radii that do not grow (the keys order the radii by their bits,
+    // so a negative one precedes the positive ones)
+    const bool all = (step == 0) | !(r <= r_last);
+    r_last = r;
+    const bool disk = pr >= 0.0f;
+    const float fpx = (float)px, fpy = (float)py;
+    // whether the previous disk reaches a group, or a wider pixel may have gained room (with a margin
+    // for the rounding of the distances; the offsets are exact)
+    auto changed = [&](const PlaceGroup& G) {
+      const float dx = fmaxf(fmaxf(G.x0 - fpx, fpx - G.x1), 0.0f), dy = fmaxf(fmaxf(G.y0 - fpy, fpy - G.y1), 0.0f);
+      const float t = fmaxf(G.cl + pr, 0.0f);
+      const bool reach = fmaf(dx, dx, dy * dy) <= fmaf(t * t, 1.0001f, 1.0f);
+      return (disk & reach) | all | !(r > G.nx);
+    };
+    // one group, by the whole warp: the disk into the clearances, then the group's choice, kept by the
+    // lane whose group it is (`mine`); selects rather than branches, as a step is a chain of latencies
+    auto look = [&](int gi, PlaceGroup& G, bool mine) {
+      const int c = gi * 32 + lane;
+      const bool in = FAST || c < nc;  // (in shared memory the last group is padded)
+      const unsigned xy = in ? cxy[c] : 0xffffffffu;
+      float v = in ? ccl[c] : -INFINITY;
+      const int dx = (int)(xy & 0xffffu) - px, dy = (int)(xy >> 16) - py;
+      const float dist = __fsub_rn(sqrtf(__int2float_rn(dx * dx + dy * dy)), pr);
+      v = disk && dist < v ? dist : v;
+      if (in) ccl[c] = v;
+      const float top = warp_maxf(v);
+      const unsigned fits = __ballot_sync(0xffffffffu, v >= r);
+      unsigned key, pix;
+      float nx = top;
+      if (fits == 0u) {  // none has room: the largest clearance, the lowest pixel that has it
+        pix = __reduce_max_sync(0xffffffffu, v == top ? ~xy : 0u);
+        key = min(ordered(top), kRoomKey - 1u);
+      } else {
+        const int first = __ffs((int)fits) - 1;
+        const unsigned fxy = __shfl_sync(0xffffffffu, xy, first);
+        key = kRoomKey + (FAST ? cd2[gi * 32 + first] : d2[pb + (long long)(fxy >> 16) * res + (fxy & 0xffffu)]);
+        pix = ~fxy;
+        nx = warp_maxf(lane < first ? v : -INFINITY);  // (-inf, none wider: no radius asks for another look)
+      }
+      G.cl = mine ? top : G.cl;
+      G.nx = mine ? nx : G.nx;
+      G.key = mine ? key : G.key;
+      G.pix = mine ? pix : G.pix;
+    };
+    if (FAST) {
+      const unsigned todo0 = __ballot_sync(0xffffffffu, has_own & changed(own));
+      for (unsigned todo = todo0; todo; todo &= todo - 1u) {
+        const int b = __ffs((int)todo) - 1;
+        look(b * kPlaceWarps + wid, own, lane == b);
+      }
+      if (todo0) {  // (else the warp's best stands)
+        best = make_uint2(own.key, own.pix);
+        warp_max2(best.x, best.y);
+      }
+    } else {
+      best = make_uint2(0u, 0u);
+      for (int g0 = wid; g0 < ng; g0 += kPlaceThreads) {
+        const int gi = g0 + lane * kPlaceWarps;
+        PlaceGroup G{};
+        if (gi < ng) G = groups[gi];
+        for (unsigned todo = __ballot_sync(0xffffffffu, gi < ng && changed(G)); todo; todo &= todo - 1u) {
+          const int b = __ffs((int)todo) - 1;
+          look(g0 + b * kPlaceWarps, G, lane == b);
+          if (lane == b) groups[gi] = G;
         }
+        if (gi < ng && (G.key > best.x || (G.key == best.x && G.pix > best.y))) best = make_uint2(G.key, G.pix);
       }
-      const unsigned long long low = 0xffffffffu - (unsigned)(y * res + x);
-      if (cl >= r) {
-        const unsigned long long k = ((unsigned long long)cd2[c] << 32) | low;
-        ck = k > ck ? k : ck;
-      }
-      const unsigned long long kf = ((unsigned long long)ordered(cl) << 32) | low;
-      fk = kf > fk ? kf : fk;
+      warp_max2(best.x, best.y);
     }
-    block_max2(ck, fk, s_red2);
-    if (threadIdx.x == 0) {
-      s_part[step & 1][0] = ck;
-      s_part[step & 1][1] = fk;
-    }
-    cluster.sync();  // every block's partials of this step are written
-    // every warp reduces the cluster's partials itself (lane k reads block k's)
-    unsigned long long a = 0, b = 0;
-    const int lane = threadIdx.x & 31;
-    if (lane < kPlaceCluster) {
-      const unsigned long long* part = cluster.map_shared_rank(&s_part[step & 1][0], (unsigned)lane);
-      a = part[0];
-      b = part[1];
-    }
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long wa = __shfl_xor_sync(0xffffffffu, a, o);
-      const unsigned long long wb = __shfl_xor_sync(0xffffffffu, b, o);
-      a = wa > a ? wa : a;
-      b = wb > b ? wb : b;
-    }
-    const unsigned long long best = a != 0 ? a : b;  // none has room: the largest clearance
-    const int idx = (int)(0xffffffffu - (unsigned)(best & 0xffffffffu));
-    px = idx % res;
-    py = idx / res;
+    if (lane == 0) s_part[step & 1][wid] = best;
+    if (ranked) r_bits = s_key32[2 * min(step + 1, ne - 1) + 1];  // the next step's radius
+    __syncthreads();  // (the buffer is written again two steps on, after the next step's barrier)
+    uint2 win = s_part[step & 1][lane % kPlaceWarps];
+    warp_max2(win.x, win.y);
+    px = (int)(~win.y & 0xffffu);
+    py = (int)(~win.y >> 16);
     pr = r;
-    if (threadIdx.x == 0) {
-      if (!ranked) order[e] = 1;  // (every block marks it: its own next reduction reads it)
-      if (rank == 0) {
-        float4 q = d.q[e];
-        q.x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
-        q.y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
-        d.q[e] = q;
+    if (tid == 0) {
+      if (ranked) {
+        s_key32[2 * step + 1] = ~win.y;  // the pixel, beside the element
+      } else {
+        const int e = (int)(0xffffffffu - e_inv);
+        placed[e] = 1;
+        d.q[e].x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
+        d.q[e].y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
       }
     }
-    // the unranked flags are visible to the next reduction (the partials' buffer of this step is
-    // not written again before the next step's cluster barrier, which every thread passes)
-    if (!ranked) __syncthreads();
+    if (!ranked) __syncthreads();  // the mark is visible to the next step's reduction
   }
-  cluster.sync();  // no block leaves while another may still read its partials
 }
 
-cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, int* gcol, unsigned* d2,
-                            int* cand, int* n_cand, float* clear, int* order, int* axis_out,
+__global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* cand, const int* n_cand,
+                                                             const unsigned* d2, unsigned* gxy, float* clear,
+                                                             int* placed) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  __shared__ int s_cell[kPlaceCells * kPlaceCells];
+  __shared__ int s_wsum[kPlaceWarps];
+  static_assert(kPlaceCells * kPlaceCells == 2 * kPlaceThreads, "two cells per thread in the scan");
+  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int res = d.prob_res[p], nc = n_cand[p];
+  const long long pb = d.prob_pix_base[p];
+  const int e0 = d.prob_elem_base[p], ne = d.prob_elem_base[p + 1] - e0;
+  if (nc == 0) return;  // no inside pixel: the params stay
+  const float fres = (float)res;
+  // ---- the elements in placement order: decreasing key (radius bits, then the lower index) ----
+  const bool ranked = ne <= kPlaceRankMax;
+  unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_dyn);
+  int nk = 0;  // keys, padded to a power of two
+  if (ranked) {
+    for (nk = 1; nk < ne;) nk <<= 1;
+    for (int i = tid; i < nk; i += kPlaceThreads) s_key[i] = i < ne ? elem_key(d, e0 + i, fres) : 0ull;
+    for (int k = 2; k <= nk; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        __syncthreads();
+        for (int i = tid; i < nk / 2; i += kPlaceThreads) {
+          const int a = (i / j) * 2 * j + i % j, b = a + j;
+          const unsigned long long x = s_key[a], y = s_key[b];
+          if ((a & k) == 0 ? x < y : x > y) {
+            s_key[a] = y;
+            s_key[b] = x;
+          }
+        }
+      }
+  } else {
+    for (int i = tid; i < ne; i += kPlaceThreads) placed[e0 + i] = 0;
+  }
+  // ---- the candidates by cell, and the groups ----
+  const int ng = (nc + 31) / 32;
+  unsigned char* s_cand = s_dyn + sizeof(unsigned long long) * nk;
+  const bool fast = ng <= kPlaceFast && 8 * nk + ng * (32 * 12 + (int)sizeof(PlaceGroup)) <= kPlaceSmem;
+  unsigned* cxy = fast ? reinterpret_cast<unsigned*>(s_cand) : gxy + pb;
+  float* ccl = fast ? reinterpret_cast<float*>(s_cand) + 32 * ng : clear + pb;
+  unsigned* cd2 = reinterpret_cast<unsigned*>(s_cand) + 64 * ng;  // in shared memory only
+  // (the unsorted list is spent once the candidates are sorted: when they stay in global memory, which
+  // takes thousands of them, its space then holds the groups, 8 words for 32 candidates)
+  PlaceGroup* groups = fast ? reinterpret_cast<PlaceGroup*>(s_cand + 32 * 12 * ng)
+                            : reinterpret_cast<PlaceGroup*>(cand + pb);
+  int shift = 0;
+  while (((res - 1) >> shift) >= kPlaceCells) ++shift;
+  auto cell = [&](unsigned xy) {
+    return (int)((xy >> 16) >> shift) * kPlaceCells + (int)((xy & 0xffffu) >> shift);
+  };
+  s_cell[2 * tid] = s_cell[2 * tid + 1] = 0;
+  __syncthreads();
+  for (int c = tid; c < nc; c += kPlaceThreads) atomicAdd(&s_cell[cell(cand[pb + c])], 1);
+  __syncthreads();
+  {  // exclusive scan of the cells' counts
+    const int v0 = s_cell[2 * tid], v = v0 + s_cell[2 * tid + 1];
+    int incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) s_wsum[wid] = incl;
+    __syncthreads();
+    int before = incl - v;
+    for (int w = 0; w < wid; ++w) before += s_wsum[w];
+    s_cell[2 * tid] = before;
+    s_cell[2 * tid + 1] = before + v0;
+  }
+  __syncthreads();
+  for (int c = tid; c < nc; c += kPlaceThreads) {
+    const unsigned xy = cand[pb + c];
+    cxy[atomicAdd(&s_cell[cell(xy)], 1)] = xy;
+  }
+  __syncthreads();
+  for (int gi = wid; gi < ng; gi += kPlaceWarps) {
+    const int c = gi * 32 + lane;
+    unsigned xy = c < nc ? cxy[c] : 0xffffffffu;
+    unsigned w = c < nc ? d2[pb + (long long)(xy >> 16) * res + (xy & 0xffffu)] : 0u;
+    const unsigned x = xy & 0xffffu, y = xy >> 16;
+    const unsigned x0 = __reduce_min_sync(0xffffffffu, x), x1 = __reduce_max_sync(0xffffffffu, c < nc ? x : 0u);
+    const unsigned y0 = __reduce_min_sync(0xffffffffu, y), y1 = __reduce_max_sync(0xffffffffu, c < nc ? y : 0u);
+    // bitonic sort of the lanes, decreasing D2, then increasing pixel (beyond the list: D2 = 0, last)
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        const unsigned wo = __shfl_xor_sync(0xffffffffu, w, j), xo = __shfl_xor_sync(0xffffffffu, xy, j);
+        const bool before = w > wo || (w == wo && xy < xo);  // this lane's goes first
+        const bool first = ((lane & j) == 0) == ((lane & k) == 0);
+        if (first != before && (w != wo || xy != xo)) {
+          w = wo;
+          xy = xo;
+        }
+      }
+    if (c < nc || fast) {  // (the padding of the last group: no pixel, never the best)
+      cxy[c] = xy;
+      ccl[c] = c < nc ? FLT_MAX : -INFINITY;
+      if (fast) cd2[c] = w;
+    }
+    if (lane == 0) groups[gi] = PlaceGroup{(float)x0, (float)x1, (float)y0, (float)y1, FLT_MAX, FLT_MAX, 0u, 0u};
+  }
+  __syncthreads();
+  if (fast) place_steps<true>(d, p, nc, ne, ranked, s_key, reinterpret_cast<unsigned*>(s_cand),
+                              reinterpret_cast<float*>(s_cand) + 32 * ng, cd2, groups, d2, placed);
+  else place_steps<false>(d, p, nc, ne, ranked, s_key, gxy + pb, clear + pb, nullptr, groups, d2, placed);
+  if (!ranked) return;
+  __syncthreads();
+  for (int i = tid; i < ne; i += kPlaceThreads) {
+    const unsigned xy = (unsigned)(s_key[i] >> 32);
+    const int e = (int)(0xffffffffu - (unsigned)s_key[i]);
+    d.q[e].x = __fdiv_rn(__fadd_rn((float)(xy & 0xffffu), 0.5f), fres);
+    d.q[e].y = __fdiv_rn(__fadd_rn((float)(xy >> 16), 0.5f), fres);
+  }
+}
+
+cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
+                            unsigned* cand, int* n_cand, float* clear, int* placed, int* axis_out,
                             float* width_out) {
   cudaError_t e = cudaMemsetAsync(n_cand, 0, sizeof(int) * d.n_probs, s);
+  const size_t cs = edt_col_smem(max_res), rs = edt_row_smem(max_res);
+  if (e == cudaSuccess && cs > 48 * 1024)
+    e = cudaFuncSetAttribute(k_edt_cols<OutsideSite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+  if (e == cudaSuccess && rs > 48 * 1024)
+    e = cudaFuncSetAttribute(k_mat_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlaceSmem);
   if (e != cudaSuccess) return e;
-  k_mat_cols<<<dim3((max_res + 127) / 128, d.n_probs), 128, 0, s>>>(d, gcol, max_res);
-  k_mat_rows<<<dim3((max_res + kMatWarps - 1) / kMatWarps, d.n_probs), kMatWarps * 32, 0, s>>>(
-      d, gcol, d2, max_res);
-  const long long np = d.total_pix;
-  k_mat_axis<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(d, d2, cand, n_cand, axis_out, width_out);
-  // gcol is free after the row pass: it holds the candidates' coordinates when they do not fit in
+  unsigned short* gcol = reinterpret_cast<unsigned short*>(g);
+  k_edt_cols<<<dim3((max_res + kEdtCols - 1) / kEdtCols, d.n_probs), kEdtThreads, cs, s>>>(
+      d, OutsideSite{d.covc}, gcol, 1);
+  k_mat_rows<<<dim3(max_res, d.n_probs), kEdtRowThreads, rs, s>>>(d, gcol, d2);
+  k_mat_axis<<<dim3((max_res + kAxisThreads - 1) / kAxisThreads, max_res, d.n_probs), kAxisThreads, 0, s>>>(
+      d, d2, cand, n_cand, axis_out, width_out);
+  // g is free after the row pass: it holds the candidates' coordinates when they do not fit in
   // shared memory
-  e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlaceSmem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(d.n_probs * kPlaceCluster);
-  cfg.blockDim = dim3(kPlaceThreads);
-  cfg.dynamicSmemBytes = kPlaceSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kPlaceCluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_mat_place, d, cand, n_cand, d2, clear, gcol, order);
+  k_mat_place<<<d.n_probs, kPlaceThreads, kPlaceSmem, s>>>(d, cand, n_cand, d2, g, clear, placed);
+  return cudaGetLastError();
 }
 
 }  // namespace collage
