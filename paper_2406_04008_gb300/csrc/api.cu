@@ -523,7 +523,7 @@ static collage_status probe_pairs(collage_t h, cudaStream_t s, size_t* need) {
   Dev probe = d;
   probe.cap = 0x7fffffff;
   probe.list_cap = 0;  // no chunk is listed
-  CK(h, launch_transform(probe, s, false));
+  CK(h, launch_transform(probe, s, false, false));
   CK(h, cudaMemcpyAsync(h->h_ctl + 2, d.pair_need, sizeof(int), cudaMemcpyDeviceToHost, s));
   // the probe allocated slots and counted chunks without an emission: reset both, and the pending
   // Adam step it applied
@@ -582,7 +582,7 @@ struct LaunchRange {
 };
 
 static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* out_bw, float* out_tau,
-                                cudaEvent_t* ev = nullptr) {
+                                cudaEvent_t* ev = nullptr, bool follows = false) {
   const Dev& d = h->d;
   const bool bwd = mode != kRender;
   const bool dil = bwd && d.L.gamma != 0.0f && d.L.n_dil > 0;
@@ -597,7 +597,7 @@ static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* ou
 #define MARK_(i) \
   if (ev) STEP_(cudaEventRecord(ev[i], s));
   MARK_(0);
-  LAUNCH_("k_transform", launch_transform(d, s, bwd && !d.deterministic));
+  LAUNCH_("k_transform", launch_transform(d, s, bwd && !d.deterministic, follows));
   MARK_(1);
   MARK_(2);
   LAUNCH_("k_raster_chunks", launch_raster_fwd(d, s, h->pair_grid, h->tile_grid, out_bw, out_tau, 1));
@@ -911,6 +911,13 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
       CKC(cudaMemset(d.dv, 0, sizeof(float2) * h->V));
     }
   }
+  {
+    std::vector<float4> trig(kTrigSteps);
+    trig_table(trig.data());
+    float4* p_trig;
+    CKC(upload(h->owned, p_trig, trig));
+    d.trig = p_trig;
+  }
   CKC(upload(h->owned, d.q, q));
   CKC(dmalloc(h->owned, d.m, h->N));
   CKC(dmalloc(h->owned, d.v, h->N));
@@ -1014,7 +1021,7 @@ static collage_status enqueue_steps(collage_t h, cudaStream_t s, int n) {
     if (st) return st;
     for (int i = 0; i < n; ++i) CK(h, cudaGraphLaunch(h->graph, s));
   } else {
-    for (int i = 0; i < n; ++i) CK(h, enqueue_iter(h, s, kStep, nullptr, nullptr));
+    for (int i = 0; i < n; ++i) CK(h, enqueue_iter(h, s, kStep, nullptr, nullptr, nullptr, i > 0));
   }
   return COLLAGE_OK;
 }
@@ -1098,7 +1105,7 @@ static cudaError_t capture_schedule(collage_t h, int start, cudaStream_t s) {
                                       cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) break;
     cudaError_t eb = cudaSuccess;
-    for (int u = 0; u < U && eb == cudaSuccess; ++u) eb = enqueue_iter(h, b, kStep, nullptr, nullptr);
+    for (int u = 0; u < U && eb == cudaSuccess; ++u) eb = enqueue_iter(h, b, kStep, nullptr, nullptr, nullptr, u > 0);
     if (eb == cudaSuccess) eb = launch_sched_cond(d, b, cond, target);
     cudaGraph_t body = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(b, &body);

@@ -74,77 +74,185 @@ __device__ __forceinline__ float2 vertex_px(const float2 v, const RotFF& M) {
   return make_float2(dot2_ff(M.m[0], M.m[1], v.x, v.y), dot2_ff(M.m[2], M.m[3], v.x, v.y));
 }
 
-// One block per element: the pending Adam step of the previous iteration, then segment records
+// Float pairs (hi + lo).  FP64 runs at 1/64 of the FP32 rate on this part, and one element's sine and
+// cosine in double were a dependent chain of about a hundred such instructions: 2 us of the
+// transform's 12 at 1000 elements, and most of its 100 at 26 k.  The pairs below carry 46
+// bits (|error| <= 2^-46 over |angle| <= 8192, measured), past the 2^-24 to which a vertex is rounded.
+// Sum a + b as hi + lo, exactly (Knuth); the second form needs |a| >= |b| or a = 0 (Dekker).
+__device__ __forceinline__ float two_sum(float a, float b, float& lo) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  lo = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+__device__ __forceinline__ float fast_two_sum(float a, float b, float& lo) {
+  const float s = __fadd_rn(a, b);
+  lo = __fsub_rn(b, __fsub_rn(s, a));
+  return s;
+}
+// Product a b as hi + lo, exactly (FMA).
+__device__ __forceinline__ float two_prod(float a, float b, float& lo) {
+  const float p = __fmul_rn(a, b);
+  lo = __fmaf_rn(a, b, -p);
+  return p;
+}
+
+// Sine and cosine of an angle |z| <= kTrigMax as unevaluated float pairs.  z = k (2 pi / 1024) + x with
+// the step in three floats (Cody & Waite 1980) and the products and differences carried exactly, then
+// the angle sum of the tabled sin, cos of k (2 pi / 1024) with sin x = x - x^3/6 + x^5/120 and
+// cos x - 1 = -x^2/2 + x^4/24, |x| <= 0.0031, of which only the leading terms need the low part.
+constexpr float kTrigMax = 8192.0f;
+constexpr double kTrigStep = 6.283185307179586 / kTrigSteps;                // 2 pi / 1024
+constexpr double kTrigStepLow = 2.4492935982947064e-16 / kTrigSteps;  // ... beyond a double
+constexpr float kTrigC1 = (float)kTrigStep;
+constexpr float kTrigC2 = (float)(kTrigStep - (double)kTrigC1);
+constexpr float kTrigC3 = (float)(kTrigStep - (double)kTrigC1 - (double)kTrigC2 + kTrigStepLow);
+
+// One of the pair: T + A x' + B y', with T, A the tabled values (hi, lo), x' = sin x (xh + xl) and
+// y = cos x - 1 (yh + yl) multiplying T: sin(k + x) = S + C sin x + S (cos x - 1), and so on.
+__device__ __forceinline__ float trig_sum(float th, float tl, float ah, float al, float xh, float xl, float yh,
+                                          float yl, float& lo) {
+  float e1, e2, f1, f2;
+  const float p1 = two_prod(ah, xh, e1), p2 = two_prod(th, yh, e2);
+  const float s1 = two_sum(th, p1, f1);
+  const float s2 = two_sum(s1, p2, f2);
+  const float rest = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(f1, f2)),
+                               __fmaf_rn(ah, xl, __fmaf_rn(al, xh, __fmaf_rn(th, yl, __fmaf_rn(tl, yh, tl)))));
+  return fast_two_sum(s2, rest, lo);
+}
+
+__device__ __forceinline__ void sincos_ff(float z, const float4* table, float (&s)[2], float (&c)[2]) {
+  const float k = rintf(__fmul_rn(z, 1.0f / kTrigC1));
+  const float4 t = table[(int)k & (kTrigSteps - 1)];  // sin hi, lo, cos hi, lo
+  float e, q, b, dd;
+  const float p = two_prod(k, kTrigC1, e);
+  const float u = two_prod(k, kTrigC2, q);
+  const float a1 = two_sum(__fsub_rn(z, p), -e, b);  // z - p is exact: p is within a factor 2 of z
+  const float a2 = two_sum(a1, -u, dd);
+  float xl;
+  const float xh = fast_two_sum(a2, __fsub_rn(__fadd_rn(b, dd), __fmaf_rn(k, kTrigC3, q)), xl);
+  float y2l;
+  const float y2 = two_prod(xh, xh, y2l);
+  y2l = __fmaf_rn(2.0f * xh, xl, y2l);
+  // sin x beyond its leading term x, cos x - 1 beyond -x^2/2
+  const float sl = __fmaf_rn(__fmul_rn(xh, y2), __fmaf_rn(y2, 1.0f / 120.0f, -1.0f / 6.0f), xl);
+  const float yl = __fmaf_rn(__fmul_rn(y2, y2), 1.0f / 24.0f, -0.5f * y2l);
+  s[0] = trig_sum(t.x, t.y, t.z, t.w, xh, sl, -0.5f * y2, yl, s[1]);
+  c[0] = trig_sum(t.z, t.w, -t.x, -t.y, xh, sl, -0.5f * y2, yl, c[1]);
+}
+
+__device__ __noinline__ void sincos_wide(float z, float (&s)[2], float (&c)[2]) {  // any other angle
+  double sn, cs;
+  sincos((double)z, &sn, &cs);
+  s[0] = (float)sn;
+  s[1] = (float)(sn - (double)s[0]);
+  c[0] = (float)cs;
+  c[1] = (float)(cs - (double)c[0]);
+}
+
+// E = 1 or 4 elements per block: the pending Adam step of the previous iteration, then segment records
 // (start, direction, end y, 1/|e|^2) of the vertices relative to the translation, translation in
 // pixels as a float hi/lo pair, outline box grown by the coverage margin, tile rectangle, the
 // element's pair slots and its emission chunks.
-// Threads 0..3 each take the step in registers (the same arithmetic), write back one parameter and
-// form one entry of the rotation-scale matrix, so one barrier separates the step from the vertices.
-// Warps 0..2 then transform the vertices (lanes own consecutive vertices; a segment's end point is
-// the next lane's start point, shuffled, so each vertex is transformed once) while warp 3 files the
-// tile rectangle, the pair slots and the chunk list, which do not depend on the vertices.
+// In warp 0, eight lanes per element take the step (one parameter each of the first four, the two bias
+// powers on different lanes) and form the rotation-scale matrix; one barrier separates the step from
+// the vertices.  Lanes own consecutive vertices; a segment's end point is the next lane's start point,
+// shuffled, so each vertex is transformed once.
+// E = 1: warps 0..2 transform the vertices while warp 3 files the tile rectangle, the pair slots and
+// the chunk list, which do not depend on the vertices: the shortest chain for one element.
+// E = 4: each warp does both for one element, so that four elements share the step's instructions and
+// no block waits for a second barrier.  It is taken when the elements fill the device several times
+// over (launch_transform), where issue slots rather than latency bound the kernel.
 constexpr int kTfThreads = 128;
+constexpr int kTfWideElems = 4096;  // elements from which a block takes four: the two forms meet here
+                                    // (18 and 17.5 us; at 26 k elements four take 56 us, one 100)
 constexpr int kTfVertexWarps = 3;
-__global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad) {
-  pdl_enter();
-  __shared__ RotFF s_rot;
-  __shared__ float4 s_q;
+template <int E>
+__global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, int follows) {
+  static_assert(E == 1 || E == 4, "eight lanes per element in one warp, one warp per element or block");
+  __shared__ RotFF s_rot[E];
+  __shared__ float4 s_q[E];
   __shared__ float s_box[4][kTfVertexWarps];
-  const int g = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int g = E == 1 ? blockIdx.x : min((int)blockIdx.x * E + wid, d.n_elems - 1);
+  const bool live = E == 1 || (int)blockIdx.x * E + wid < d.n_elems;
+  // what is written once, at create or per level, is read before the predecessor has completed
   // (a single problem's resolution is read without waiting for the element's problem index)
   const int p = d.n_probs == 1 ? 0 : d.elem_prob[g];
   const int res = d.prob_res[p];
-  if (g == 0 && threadIdx.x == 0) {  // this iteration's live pairs and finished gradient blocks
-    d.work[1] = 0;
-    d.work[3] = 0;
-  }
-  // the outline and its first vertices do not depend on the step: read before the barrier
   const int v0 = d.elem_voff[g], nv = d.elem_voff[g + 1] - v0;
   const bool closed = d.elem_closed[g] != 0;
   const float hw = closed ? 0.0f : d.elem_hw[g];
-  const float rbin = wid == kTfVertexWarps ? d.elem_rbin[g] : 0.0f;
-  const int k_first = wid * 32 + lane;
+  const bool files = E == 4 || wid == kTfVertexWarps, verts = E == 4 || wid < kTfVertexWarps;
+  constexpr int kStride = E == 4 ? 32 : kTfVertexWarps * 32;
+  const int k_first = E == 4 ? lane : wid * 32 + lane;
+  float rbin = 0.0f;
   float2 va0 = make_float2(0.f, 0.f), vb0 = make_float2(0.f, 0.f);
-  if (wid < kTfVertexWarps && k_first < nv) {
-    va0 = d.vloc[v0 + k_first];
-    if (lane == 31 || k_first + 1 == nv) vb0 = d.vloc[v0 + (k_first + 1 == nv ? 0 : k_first + 1)];
+  auto first_vertices = [&]() {  // (written by calls that replace the outlines, and by each fitting iteration)
+    if (files) rbin = d.elem_rbin[g];
+    if (verts && k_first < nv) {
+      va0 = d.vloc[v0 + k_first];
+      if (lane == 31 || k_first + 1 == nv) vb0 = d.vloc[v0 + (k_first + 1 == nv ? 0 : k_first + 1)];
+    }
+  };
+  const bool early = follows && !d.fit;
+  if (early) first_vertices();
+  pdl_enter();
+  if (!early) first_vertices();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // this iteration's live pairs and finished gradient blocks
+    d.work[1] = 0;
+    d.work[3] = 0;
   }
-  if (threadIdx.x < 4) {
-    const int k = threadIdx.x;
-    float4 q = d.q[g], m, v;
+  if (wid == 0) {
+    const int e = E == 1 ? 0 : lane >> 3, k = lane & 3, ge = min((int)blockIdx.x * E + e, d.n_elems - 1);
+    const bool writer = (E == 1 ? lane < 4 : (lane & 7) < 4) && (int)blockIdx.x * E + e < d.n_elems;
+    const int re = E == 1 ? res : d.prob_res[d.n_probs == 1 ? 0 : d.elem_prob[ge]];
+    float x = reinterpret_cast<const float*>(d.q + ge)[k];
     // the previous iteration's step (when the outlines are fitted the transforms stay fixed)
     const bool step = *d.pending && !d.fit;
     if (step) {
-      m = d.m[g];
-      v = d.v[g];
-      const uchar4 tr = d.trainable ? d.trainable[g] : make_uchar4(1, 1, 1, 1);
-      adam_apply(d, *d.step, d.dq[g], tr, q, m, v);
+      float m = reinterpret_cast<const float*>(d.m + ge)[k], v = reinterpret_cast<const float*>(d.v + ge)[k];
+      const float gr = reinterpret_cast<const float*>(d.dq + ge)[k];
+      const bool tr = !d.trainable || reinterpret_cast<const unsigned char*>(d.trainable + ge)[k];
+      const float pw = powf((lane & 4) ? d.b2 : d.b1, (float)*d.step);
+      const AdamScale a = adam_scale(d, __shfl_sync(0xffffffffu, pw, 0), __shfl_sync(0xffffffffu, pw, 4));
+      if (tr) adam_entry(d, a, gr, x, m, v);
+      if (k == 3) x = fminf(fmaxf(x, d.s_min), d.s_max);
+      if (writer) {
+        reinterpret_cast<float*>(d.m + ge)[k] = m;
+        reinterpret_cast<float*>(d.v + ge)[k] = v;
+      }
     }
     // the host-buffer step: the caller's params replace the stepped ones (the moments keep the step)
-    if (d.q_in) q = d.q_in[g];
-    __syncwarp(0xfu);  // every reader of the old params is done
-    auto pick = [k](float4 x) { return k == 0 ? x.x : k == 1 ? x.y : k == 2 ? x.z : x.w; };
-    if (step) {
-      reinterpret_cast<float*>(d.m + g)[k] = pick(m);
-      reinterpret_cast<float*>(d.v + g)[k] = pick(v);
+    if (d.q_in) x = reinterpret_cast<const float*>(d.q_in + ge)[k];
+    if (writer && (step || d.q_in)) reinterpret_cast<float*>(d.q + ge)[k] = x;
+    const float z = __shfl_sync(0xffffffffu, x, 2, 4), sc = __shfl_sync(0xffffffffu, x, 3, 4);
+    if (writer) {
+      reinterpret_cast<float*>(&s_q[e])[k] = x;
+      float s[2], c[2];
+      if (fabsf(z) <= kTrigMax) sincos_ff(z, d.trig, s, c);
+      else sincos_wide(z, s, c);
+      // entry k of s res [cos, -sin; sin, cos]
+      float th = k == 0 || k == 3 ? c[0] : s[0], tl = k == 0 || k == 3 ? c[1] : s[1];
+      if (k == 1) {
+        th = -th;
+        tl = -tl;
+      }
+      float hl, pl, lo;
+      const float hh = two_prod(sc, (float)re, hl), pp = two_prod(hh, th, pl);
+      s_rot[e].m[k][0] = fast_two_sum(pp, __fadd_rn(pl, __fmaf_rn(hh, tl, __fmul_rn(hl, th))), lo);
+      s_rot[e].m[k][1] = lo;
     }
-    if (step || d.q_in) reinterpret_cast<float*>(d.q + g)[k] = pick(q);
-    if (k == 0) s_q = q;
-    double sn, c;
-    sincos((double)q.z, &sn, &c);
-    const double sc = (double)q.w * (double)res;
-    const double mk = k == 0 ? sc * c : k == 1 ? -sc * sn : k == 2 ? sc * sn : sc * c;
-    const float hi = (float)mk;
-    s_rot.m[k][0] = hi;
-    s_rot.m[k][1] = (float)(mk - (double)hi);
   }
   __syncthreads();
-  const float4 q = s_q;
-  if (wid == kTfVertexWarps) {
+  if (!live) return;
+  const int slot = E == 1 ? 0 : wid;
+  const float4 q = s_q[slot];
+  int4 r = make_int4(0, 0, -1, -1);
+  int nx = 0, ny = 0, cbase = 0;
+  bool heavy = false;
+  if (files) {
     // the tile rectangle, the pair slots and the emission's chunks (lane 0 takes the counts)
     const bool finite = isfinite(q.x) && isfinite(q.y) && isfinite(q.z) && isfinite(q.w) && q.w > 0.0f;
-    int4 r = make_int4(0, 0, -1, -1);
     if (finite) r = bin_rect(q, rbin, hw, res, d.tile, d.L.rho_px, d.L.pad_px);
     else if (lane == 0) atomicOr(d.status, kStatusBadParam);
     if (lane == 0) {
@@ -157,32 +265,39 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad) 
       // the emission's work: the rectangle in chunks of kChunkPx / T tiles a side; chunks whose
       // segments x tiles exceed kHeavyChunk are listed from the front, the others from the back,
       // so that the emission takes the costliest first and none trails at the end
-      const int cw = d.chunk_tiles, nx = (r.z - r.x) / cw + 1, ny = (r.w - r.y) / cw + 1;
+      const int cw = d.chunk_tiles;
+      nx = (r.z - r.x) / cw + 1;
+      ny = (r.w - r.y) / cw + 1;
       const int tiles = min(r.z - r.x + 1, cw) * min(r.w - r.y + 1, cw);
-      const bool heavy = nv * tiles > kHeavyChunk;
-      int pbase = 0, cbase = 0;
+      heavy = nv * tiles > kHeavyChunk;
       if (lane == 0) {  // both counts taken at once (neither waits for the other's result)
-        pbase = atomicAdd(d.pair_need, n);
+        const int pbase = atomicAdd(d.pair_need, n);
         cbase = atomicAdd(d.chunk_count + (heavy ? 0 : 1), nx * ny);
         if (pbase > d.cap - n) atomicOr(d.status, kStatusOverflow);
         d.elem_pbase[g] = pbase;
       }
-      cbase = __shfl_sync(0xffffffffu, cbase, 0);
-      // (heavy + light chunks beyond the list mean more pairs than the capacity too: the iteration
-      // overflows and the emission does not read the list; every write stays inside it)
-      if (cbase + nx * ny <= d.list_cap)
-        for (int c = lane; c < nx * ny; c += 32) {
-          const int at = heavy ? cbase + c : d.list_cap - 1 - (cbase + c);
-          d.near_list[at] = make_int4(g, (r.x + (c % nx) * cw) | ((r.y + (c / nx) * cw) << 16), p, 0);
-        }
     }
+  }
+  auto file_chunks = [&]() {
+    if (nx == 0) return;
+    const int at0 = __shfl_sync(0xffffffffu, cbase, 0), cw = d.chunk_tiles;
+    // (heavy + light chunks beyond the list mean more pairs than the capacity too: the iteration
+    // overflows and the emission does not read the list; every write stays inside it)
+    if (at0 + nx * ny <= d.list_cap)
+      for (int c = lane; c < nx * ny; c += 32) {
+        const int at = heavy ? at0 + c : d.list_cap - 1 - (at0 + c);
+        d.near_list[at] = make_int4(g, (r.x + (c % nx) * cw) | ((r.y + (c / nx) * cw) << 16), p, 0);
+      }
+  };
+  if (E == 1 && files) {
+    file_chunks();
     return;  // no barrier follows for this warp
   }
-  const RotFF rot = s_rot;
+  const RotFF rot = s_rot[slot];
   float xmin = FLT_MAX, ymin = FLT_MAX, xmax = -FLT_MAX, ymax = -FLT_MAX;
-  for (int k0 = wid * 32; k0 < nv; k0 += kTfVertexWarps * 32) {  // warp-uniform trip count
+  for (int k0 = E == 4 ? 0 : wid * 32; k0 < nv; k0 += kStride) {  // warp-uniform trip count
     const int k = k0 + lane;
-    const bool first = k0 == wid * 32;
+    const bool first = k0 < kStride;
     float2 a = make_float2(0.f, 0.f);
     if (k < nv) {
       a = vertex_px(first ? va0 : d.vloc[v0 + k], rot);
@@ -212,38 +327,49 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad) 
       d.segS[v0 + k] = slope;
     }
   }
+  if (E == 4) file_chunks();
   xmin = warp_min(xmin);
   ymin = warp_min(ymin);
   xmax = warp_max(xmax);
   ymax = warp_max(ymax);
-  if (lane == 0) {
-    s_box[0][wid] = xmin;
-    s_box[1][wid] = ymin;
-    s_box[2][wid] = xmax;
-    s_box[3][wid] = ymax;
+  if (E == 1) {
+    if (lane == 0) {
+      s_box[0][wid] = xmin;
+      s_box[1][wid] = ymin;
+      s_box[2][wid] = xmax;
+      s_box[3][wid] = ymax;
+    }
+    // the vertex warps only (warp 3 has left): named barrier 1 over their threads
+    asm volatile("bar.sync 1, %0;" ::"n"(kTfVertexWarps * 32) : "memory");
   }
-  // the vertex warps only (warp 3 has left): named barrier 1 over their threads
-  asm volatile("bar.sync 1, %0;" ::"n"(kTfVertexWarps * 32) : "memory");
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < kTfVertexWarps; ++w) {
+  if (E == 1 ? threadIdx.x == 0 : lane == 0) {
+    for (int w = 1; E == 1 && w < kTfVertexWarps; ++w) {
       xmin = fminf(xmin, s_box[0][w]);
       ymin = fminf(ymin, s_box[1][w]);
       xmax = fmaxf(xmax, s_box[2][w]);
       ymax = fmaxf(ymax, s_box[3][w]);
     }
-    const double tx = (double)q.x * res, ty = (double)q.y * res;
-    const float hx = (float)tx, hy = (float)ty;
-    d.tpx[g] = make_float4(hx, hy, (float)(tx - (double)hx), (float)(ty - (double)hy));
+    const float fres = (float)res;
+    float lx, ly;
+    const float hx = two_prod(q.x, fres, lx), hy = two_prod(q.y, fres, ly);
+    d.tpx[g] = make_float4(hx, hy, lx, ly);
     // outline box relative to the translation, grown by the coverage margin (+ rounding slack)
-    const float m = d.L.rho_px + d.L.pad_px + hw * (float)res + 0.01f;
+    const float m = d.L.rho_px + d.L.pad_px + hw * fres + 0.01f;
     d.bbox[g] = make_float4(xmin - m, ymin - m, xmax + m, ymax + m);
   }
 }
 
-cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad) {
-  return klaunch(d.pdl, k_transform, d.n_elems, kTfThreads, 0, s, d, zero_grad ? 1 : 0);
+void trig_table(float4* t) {
+  for (int k = 0; k < kTrigSteps; ++k) {
+    const double a = k * (6.283185307179586 / kTrigSteps), s = sin(a), c = cos(a);
+    t[k] = make_float4((float)s, (float)(s - (double)(float)s), (float)c, (float)(c - (double)(float)c));
+  }
 }
 
-
+cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad, bool follows) {
+  const int z = zero_grad ? 1 : 0, f = follows ? 1 : 0;
+  if (d.n_elems >= kTfWideElems) return klaunch(d.pdl, k_transform<4>, (d.n_elems + 3) / 4, kTfThreads, 0, s, d, z, f);
+  return klaunch(d.pdl, k_transform<1>, d.n_elems, kTfThreads, 0, s, d, z, f);
+}
 
 }  // namespace collage

@@ -19,6 +19,7 @@
 namespace collage {
 
 constexpr int kMaxDil = 8;
+constexpr int kTrigSteps = 1024;        // angles of the transform's table
 constexpr int kCtlWords = 24;           // device control words (status first, see Dev)
 constexpr int kChunkPx = 64;            // side, in pixels, of the emission's chunks of an element
 constexpr int kHeavyChunk = 1024;       // segments x tiles above which a chunk is taken first
@@ -81,6 +82,7 @@ struct Dev {
   const float4* q_in;           // [n] params the transform takes in place of q (the host-buffer
                                 //   step's mapped input), or null
   const uchar4* trainable;      // may be null
+  const float4* trig;           // [kTrigSteps] sin (hi, lo), cos (hi, lo) of k (2 pi / kTrigSteps)
   float lr, b1, b2, eps, s_min, s_max;
   // ---- per iteration ----
   float4* segA;                 // [V] segment k: start (px, relative to the translation), direction
@@ -190,29 +192,27 @@ __device__ __forceinline__ bool in_bounds(const Dev& d, bool ok) {
 // An iteration's step is applied lazily: the loss assembly marks it pending, and the next
 // iteration's transform kernel (one block per element, which reads the params first anyway)
 // applies it before forming the geometry; API calls that read or replace params flush it.
-__device__ __forceinline__ void adam_apply(const Dev& d, int t, float4 gr, uchar4 tr, float4& q, float4& m,
-                                           float4& v) {
-  const float bc1 = 1.0f - powf(d.b1, (float)t), bc2 = 1.0f - powf(d.b2, (float)t);
-  const float step_size = d.lr / bc1, bc2s = sqrtf(bc2);
-  float* qp = &q.x;
-  float* mp = &m.x;
-  float* vp = &v.x;
-  const float gg[4] = {gr.x, gr.y, gr.z, gr.w};
-  const unsigned char tt[4] = {tr.x, tr.y, tr.z, tr.w};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    if (!tt[k]) continue;
-    mp[k] = d.b1 * mp[k] + (1.0f - d.b1) * gg[k];
-    vp[k] = d.b2 * vp[k] + (1.0f - d.b2) * gg[k] * gg[k];
-    const float denom = sqrtf(vp[k]) / bc2s + d.eps;
-    qp[k] -= step_size * mp[k] / denom;
-  }
-  q.w = fminf(fmaxf(q.w, d.s_min), d.s_max);
+struct AdamScale {
+  float step, root2;  // lr / (1 - b1^t), sqrt(1 - b2^t)
+};
+__device__ __forceinline__ AdamScale adam_scale(const Dev& d, float b1_t, float b2_t) {
+  return {d.lr / (1.0f - b1_t), sqrtf(1.0f - b2_t)};
+}
+__device__ __forceinline__ void adam_entry(const Dev& d, AdamScale a, float g, float& q, float& m, float& v) {
+  m = d.b1 * m + (1.0f - d.b1) * g;
+  v = d.b2 * v + (1.0f - d.b2) * g * g;
+  const float denom = sqrtf(v) / a.root2 + d.eps;
+  q -= a.step * m / denom;
 }
 __device__ __forceinline__ void adam_update(const Dev& d, int g, int t, float4 gr) {
   float4 q = d.q[g], m = d.m[g], v = d.v[g];
   const uchar4 tr = d.trainable ? d.trainable[g] : make_uchar4(1, 1, 1, 1);
-  adam_apply(d, t, gr, tr, q, m, v);
+  const AdamScale a = adam_scale(d, powf(d.b1, (float)t), powf(d.b2, (float)t));
+  if (tr.x) adam_entry(d, a, gr.x, q.x, m.x, v.x);
+  if (tr.y) adam_entry(d, a, gr.y, q.y, m.y, v.y);
+  if (tr.z) adam_entry(d, a, gr.z, q.z, m.z, v.z);
+  if (tr.w) adam_entry(d, a, gr.w, q.w, m.w, v.w);
+  q.w = fminf(fmaxf(q.w, d.s_min), d.s_max);
   d.q[g] = q;
   d.m[g] = m;
   d.v[g] = v;
@@ -269,7 +269,10 @@ __device__ __forceinline__ void mark_step_if_last(const Dev& d) {
 }
 
 // ---- launchers (each enqueues on `s`, returns the launch error) ----
-cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad);
+void trig_table(float4* t);  // host: fills the table of Dev::trig
+// follows: the previous launch on `s` is another iteration's, so the outlines were written long before
+// and are read while it ends (never the first launch after a call that may replace them)
+cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad, bool follows);
 cudaError_t launch_container(const Dev& d, cudaStream_t s);
 // part 1: pair emission, classification and per-pixel signed distances (per element chunk);
 // part 2: per-tile composite and loss partials; 3: both
