@@ -69,7 +69,7 @@ struct collage_s {
   collage_tuning tuning{};
   // device memory
   Dev d{};
-  size_t pix_cap = 0, tile_cap = 0, dtile_cap = 0, pair_cap = 0, saved_tile = 0;
+  size_t pix_cap = 0, tile_cap = 0, unit_cap = 0, dtile_cap = 0, pair_cap = 0, saved_tile = 0;
   std::vector<void*> list_bufs;  // per-tile pair lists: tile_cap tiles x d.tile_cap entries
   int* ctl = nullptr;        // device: status, step, total_pairs, pending, 8 work counters,
                              //   schedule base step, 2 chunk counts, pairs allocated, 1 spare,
@@ -363,10 +363,8 @@ static collage_status ensure_pairs(collage_t h, size_t cap) {
   free_list(h->pair_bufs);
   h->pair_cap = 0;
   Dev& d = h->d;
-  CK(h, dmalloc(h->pair_bufs, d.pair_elem, cap));
   CK(h, dmalloc(h->pair_bufs, d.live_list, cap));
   CK(h, dmalloc(h->pair_bufs, d.near_list, cap));
-  CK(h, dmalloc(h->pair_bufs, d.pair_cls, cap));
   CK(h, dmalloc(h->pair_bufs, d.partial, cap));
   CK(h, dmalloc(h->pair_bufs, d.saved, cap * tt));
   h->pair_cap = cap;
@@ -396,18 +394,17 @@ static collage_status ensure_tile_lists(collage_t h, int per_tile) {
   const size_t n = h->tile_cap * (size_t)per_tile;
   CK(h, dmalloc(h->list_bufs, d.tile_list, n));
   CK(h, dmalloc(h->list_bufs, d.tile_sorted, n));
-  CK(h, dmalloc(h->list_bufs, d.tile_sorted_slot, n));
   d.tile_cap = per_tile;
   return COLLAGE_OK;
 }
 
-// Per-pixel, per-tile and per-dilation-tile buffers for the largest level (regrown if needed).
-static collage_status ensure_level_bufs(collage_t h, size_t np, size_t nt, size_t nd) {
-  if (np <= h->pix_cap && nt <= h->tile_cap && nd <= h->dtile_cap) return COLLAGE_OK;
+// Per-pixel, per-tile, per-unit and per-dilation-tile buffers for the largest level (regrown if needed).
+static collage_status ensure_level_bufs(collage_t h, size_t np, size_t nt, size_t nu, size_t nd) {
+  if (np <= h->pix_cap && nt <= h->tile_cap && nu <= h->unit_cap && nd <= h->dtile_cap) return COLLAGE_OK;
   drop_graph(h);
   CK(h, cudaDeviceSynchronize());
   free_list(h->level_bufs);
-  h->pix_cap = h->tile_cap = h->dtile_cap = 0;
+  h->pix_cap = h->tile_cap = h->unit_cap = h->dtile_cap = 0;
   Dev& d = h->d;
   CK(h, dmalloc(h->level_bufs, d.covc, np));
   CK(h, dmalloc(h->level_bufs, d.img_I, np));
@@ -418,13 +415,15 @@ static collage_status ensure_level_bufs(collage_t h, size_t np, size_t nt, size_
   CK(h, cudaMemset(d.tile_n, 0, sizeof(int) * nt));
   CK(h, dmalloc(h->level_bufs, d.tile_m, nt));
   CK(h, cudaMemset(d.tile_m, 0, sizeof(int) * nt));
-  CK(h, dmalloc(h->level_bufs, d.lossA, nt));
+  CK(h, dmalloc(h->level_bufs, d.lossA, nu));
+  CK(h, dmalloc(h->level_bufs, d.loss0, nu));
   CK(h, dmalloc(h->level_bufs, d.lossU, nd));
   CK(h, dmalloc(h->level_bufs, d.dtile_flags, nd));
   CK(h, dmalloc(h->level_bufs, d.dtile_list, 2 * nd));
   CK(h, dmalloc(h->level_bufs, d.dtile_n, 2));
   h->pix_cap = np;
   h->tile_cap = nt;
+  h->unit_cap = nu;
   h->dtile_cap = nd;
   return ensure_tile_lists(h, d.tile_cap);
 }
@@ -473,7 +472,7 @@ static collage_status build_levels(collage_t h) {
     CK(h, cudaMemcpy(t.d_pix_base, t.pix_base.data(), sizeof(long long) * (P + 1), cudaMemcpyHostToDevice));
   }
   drop_graph(h);
-  collage_status st = ensure_level_bufs(h, np, nt, nd);
+  collage_status st = ensure_level_bufs(h, np, nt, nt * (T * T / 64), nd);
   if (st) return st;
   h->lv_tile = T;
   return COLLAGE_OK;
@@ -602,7 +601,8 @@ static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* ou
   MARK_(2);
   LAUNCH_("k_raster_chunks", launch_raster_fwd(d, s, h->pair_grid, h->tile_grid, out_bw, out_tau, 1));
   MARK_(3);
-  LAUNCH_("k_composite", launch_raster_fwd(d, s, h->pair_grid, h->tile_grid, out_bw, out_tau, 2));
+  const int flags = bwd ? kCompLoss | (dil ? kCompAllI : 0) : out_bw ? 0 : kCompAllI;
+  LAUNCH_("k_composite", launch_raster_fwd(d, s, h->pair_grid, h->tile_grid, out_bw, out_tau, 2, flags));
   MARK_(4);
   // the loss assembly needs only the composite's and the distribution term's partials: it runs on
   // a side stream beside the distribution adjoint and the raster adjoint (joined at the end of
@@ -1374,16 +1374,20 @@ extern "C" collage_status collage_get_bins(collage_t h, void* stream, int* d_til
   if (!d_tile && !d_elem) return COLLAGE_OK;
   if (cap < n) return fail(h, COLLAGE_ERR_INVALID_ARG, "cap is smaller than the pair count");
   const size_t nt = (size_t)h->d.total_tiles, C = (size_t)h->d.tile_cap;
-  std::vector<int> tm(nt), ts(nt * C), te, ee;
+  std::vector<int> tm(nt), te, ee;
+  std::vector<uint2> ts(nt * C);
   CK(h, cudaMemcpy(tm.data(), h->d.tile_m, sizeof(int) * nt, cudaMemcpyDeviceToHost));
-  CK(h, cudaMemcpy(ts.data(), h->d.tile_sorted, sizeof(int) * nt * C, cudaMemcpyDeviceToHost));
+  CK(h, cudaMemcpy(ts.data(), h->d.tile_list, sizeof(uint2) * nt * C, cudaMemcpyDeviceToHost));
   te.reserve(n);
   ee.reserve(n);
-  for (size_t t = 0; t < nt; ++t)
+  for (size_t t = 0; t < nt; ++t) {
+    const size_t first = ee.size();
     for (int k = 0; k < tm[t] && k < (int)C; ++k) {
       te.push_back((int)t);
-      ee.push_back(ts[t * C + k]);
+      ee.push_back((int)ts[t * C + k].y);
     }
+    std::sort(ee.begin() + first, ee.end());  // the lists are in emission order
+  }
   if ((int)te.size() != n) return fail(h, COLLAGE_ERR_STATE, "tile lists disagree with the pair count");
   if (d_tile && n) CK(h, cudaMemcpy(d_tile, te.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
   if (d_elem && n) CK(h, cudaMemcpy(d_elem, ee.data(), sizeof(int) * n, cudaMemcpyHostToDevice));

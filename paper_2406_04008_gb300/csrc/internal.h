@@ -34,9 +34,15 @@ constexpr int kStatusVoid = kStatusNoBins | kStatusBadParam;      // the iterati
 // the coverage margin (rho + pad + stroke half-width) of some pixel centre of the tile; otherwise
 // the coverage and the padded coverage are the same saturated value (0 or 1) on every pixel of
 // the tile and the pair carries no gradient.
-constexpr uint8_t kPairOut = 0;   // not near, outside the outline: c = c^pad = 0
-constexpr uint8_t kPairIn = 1;    // not near, inside: c = c^pad = 1
-constexpr uint8_t kPairNear = 2;  // per-pixel signed distances (the distance kernel)
+constexpr unsigned kPairOut = 0;   // not near, outside the outline: c = c^pad = 0
+constexpr unsigned kPairIn = 1;    // not near, inside: c = c^pad = 1
+constexpr unsigned kPairNear = 2;  // per-pixel signed distances (the distance kernel)
+constexpr int kSlotBits = 30;      // a tile list's entry: slot | class << kSlotBits, element
+constexpr unsigned kSlotMask = (1u << kSlotBits) - 1u;
+
+// What a composite launch leaves.
+constexpr int kCompLoss = 1;  // loss partials, and the images where the adjoint reads them
+constexpr int kCompAllI = 2;  // img_I of every pixel (the distribution term or the metrics follow)
 
 struct LossParams {
   float alpha, beta, gamma, delta;
@@ -99,14 +105,13 @@ struct Dev {
   int* tile_n;                  // [total_tiles] pairs registered in each tile's list by the
                                 //   emission (the composite zeroes it)
   int* tile_m;                  // [total_tiles] pairs of each tile (the composite's count, kept)
-  int* tile_list;               // [total_tiles * tile_cap] pair slots of each tile, emission order
-  int* tile_sorted;             // [total_tiles * tile_cap] each tile's elements in increasing order
-  int* tile_sorted_slot;        //   and their pair slots (written by the composite)
+  uint2* tile_list;             // [total_tiles * tile_cap] each tile's pairs in emission order: (slot |
+                                //   class << kSlotBits, element)
+  unsigned* tile_sorted;        // [total_tiles * tile_cap] scratch of the composite: the first words of
+                                //   a very long list's covering pairs, in element order
   int tile_cap;                 // pair-list capacity of a tile
-  int* tile_max;                // [1] pairs of the fullest tile list of the iteration (the
-                                //   composite's maximum; the emission's block 0 zeroes it)
-  int* pair_elem;               // [cap] element of each pair slot (tile ranges, emission order)
-  uint8_t* pair_cls;            // [cap] kPairOut / kPairIn / kPairNear, set by the emission
+  int* tile_max;                // [1] pairs of the fullest tile list of the iteration where one passed 3/4
+                                //   of the capacity, else 0 (the emission's block 0 zeroes it)
   int4* near_list;              // [list_cap] the emission's work list: (element, chunk origin tile
                                 //   column | row << 16, problem, 0), one per kChunkPx-square chunk of
                                 //   every element's tile rectangle, appended by the transform: heavy
@@ -124,7 +129,9 @@ struct Dev {
   float* gOu;                   // [pix] dL_u/dO
   uint32_t* dil_g;              // [pix] the adjoint's staged word: round(M_C (1 - O) 2^Q) in bits
                                 // 0..23, bit 24 + k set where B_k < 1 (Q of the kernel count)
-  float4* lossA;                // [total_tiles] (sum W(I-Ic)^2, sum relu(A-tau), sum O(1-y), 0)
+  float4* lossA;                // per unit of 64 pixels of a tile (one of 8 x 8, four of 16 x 16), tile by
+                                //   tile: (sum W(I-Ic)^2, sum relu(A-tau), sum O(1-y), 0)
+  float* loss0;                 // per unit: the first of these where nothing covers it (level constant)
   float* lossU;                 // [total_dtiles] weighted uniform-loss partial
   uint8_t* dtile_flags;         // [total_dtiles] container coverage on the tile / its halo (or null)
   int* dtile_list;              // [2 total_dtiles] the tiles with kFlagOwn from 0, with kFlagHalo
@@ -275,9 +282,9 @@ void trig_table(float4* t);  // host: fills the table of Dev::trig
 cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad, bool follows);
 cudaError_t launch_container(const Dev& d, cudaStream_t s);
 // part 1: pair emission, classification and per-pixel signed distances (per element chunk);
-// part 2: per-tile composite and loss partials; 3: both
+// part 2: per-tile composite and loss partials (flags: kComp*)
 cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int tile_grid,
-                              float* out_bw, float* out_tau, int part = 3);
+                              float* out_bw, float* out_tau, int part, int flags = 0);
 cudaError_t prepare_dilate(int n_dil);  // sets dynamic shared memory limits (not capturable)
 cudaError_t launch_dilate(const Dev& d, cudaStream_t s, bool backward);
 cudaError_t launch_dtile_flags(const Dev& d, cudaStream_t s);  // once per level, after the container

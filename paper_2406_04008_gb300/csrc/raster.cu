@@ -75,15 +75,6 @@ constexpr int kRowCross = 16;   // crossings listed per pixel row of an emission
 constexpr int kPairWarps = 4;   // pairs per block of the per-pair adjoint (one per warp)
 constexpr float kFar = 1e30f;   // |sd| of a pixel farther than the coverage margin
 
-__device__ __forceinline__ void tile_coords(const Dev& d, int tile, int T, int& p, int& tx, int& ty,
-                                            int& res) {
-  p = find_prob(d.prob_tile_base, d.n_probs, tile);
-  const int lt = tile - d.prob_tile_base[p], ntx = d.prob_ntx[p];
-  res = d.prob_res[p];
-  tx = lt % ntx;
-  ty = lt / ntx;
-}
-
 // Winding number of a point (element frame) over every segment of an outline: the crossing test of
 // the per-row lists below applied to all segments (for rows that cross the outline too often).
 __device__ __noinline__ int winding_all(const Dev& d, int v0, int ns, float px, float py) {
@@ -200,7 +191,9 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
     const int ns = closed ? nv : nv - 1;
     const bool staged = ns <= kStageSegs;
     const int mw = staged ? (ns + 31) >> 5 : 0;
-    // 1. pair slots; cleared marks and row lists
+    // 1. pair slots and their places in the tiles' lists (the entries are written once the tiles are
+    // classified, when the counts taken here have long arrived); cleared marks and row lists
+    int place = -1;
     if (tid < NCT) {
       int slot = -1;
       const int t = tb + (ty0 + tid / ctw) * ntx + tx0 + tid % ctw;
@@ -208,10 +201,7 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
         const int u = d.elem_pbase[g] + (ty0 + tid / ctw - r.y) * (r.z - r.x + 1) + tx0 + tid % ctw - r.x;
         if (in_bounds(d, u >= 0 && u < d.cap)) {
           slot = u;
-          d.pair_elem[slot] = g;
-          const int k = atomicAdd(&d.tile_n[t], 1);
-          if (k < d.tile_cap) d.tile_list[(size_t)t * d.tile_cap + k] = slot;
-          else atomicOr(d.status, kStatusTileCap);
+          place = atomicAdd(&d.tile_n[t], 1);
         }
       }
       s_slot[tid] = slot;
@@ -273,7 +263,7 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
     // 3. classification; the near tiles in tile order
     if (tid < nct && s_slot[tid] >= 0) {
       const int slot = s_slot[tid];
-      uint8_t cls = kPairNear;
+      unsigned cls = kPairNear;
       if (!s_tn[tid]) {
         int w = 0;
         if (closed) {
@@ -294,7 +284,10 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
         cls = w != 0 ? kPairIn : kPairOut;
         if (d.deterministic) d.partial[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      d.pair_cls[slot] = cls;
+      const int t = tb + (ty0 + tid / ctw) * ntx + tx0 + tid % ctw;
+      const uint2 entry = make_uint2((unsigned)slot | cls << kSlotBits, (unsigned)g);
+      if (place < d.tile_cap) d.tile_list[(size_t)t * d.tile_cap + place] = entry;
+      else atomicOr(d.status, kStatusTileCap);
     }
     if (tid < 32) {  // warp 0: the near tiles, in tile order
       int n = 0;
@@ -437,177 +430,318 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
 }
 
 // ------------------------------------------------------------------------------------------------
-// Composite, one tile per warp: order the tile's pairs by element id (ids are unique in a tile, so
-// an id's rank is the number of smaller ids; for up to 32 pairs the lanes hold the ids and rank
-// them by shuffles), then per pixel Ihat = prod(1 - c_i) and prod(1 - tau c_i^pad) over the pairs
-// in that order, and the per-pixel loss terms (Eq. 5, Eq. 6 surrogate, force), summed over the
-// tile by a fixed shuffle tree.  No block-wide barrier: each warp owns its tile.
+// Composite, one unit of 64 pixels per warp: a tile of 8 x 8, or four rows of a tile of 16 x 16 (whose
+// four units are the four warps of a block).  The tile's pairs with some coverage are ordered by
+// element id (ids are unique in a tile, so an id's rank is the number of smaller ids; for up to 32
+// pairs the lanes hold the ids and rank them by shuffles), then per pixel Ihat = prod(1 - c_i) and
+// prod(1 - tau c_i^pad) over the pairs in that order, and the per-pixel loss terms (Eq. 5, Eq. 6
+// surrogate, force), summed over the unit by a fixed shuffle tree.
+//
+// Bound by instructions and by the round trips of one tile after another, not by bytes.  So a warp takes
+// a run of tiles at once, a tile per lane (C of them, launch_raster_fwd): the lanes find their tiles'
+// places and read the counts and first entries together, and settle the tiles without coverage by
+// themselves (their loss is a constant of the level); the others are taken one at a time, the next one's
+// entries in flight.  A list entry carries the slot, its class and its element (no gather per pair).
+// The images are written where a later kernel reads them: Ihat everywhere when the distribution term
+// (or the metrics) follows, both where a pair is near (the adjoint's pixels).  64 collages, 27.6 Mpx,
+// 431 k tiles, 170 k of them covered: 283 -> 172 us, of which 55 are the products, 43 the loss terms
+// and sums, 41 the tiles without coverage; 5000 elements at 2048^2: 78 -> 72 us; 64 outlines at 256^2:
+// 48 -> 34 us; 1000 elements at 1024^2: 18 us before and now, 8 of them the launch and the first reads.
 // ------------------------------------------------------------------------------------------------
 constexpr int kCompWarps = 4;
-constexpr int kCompGroup = 4;   // pairs whose records are read together
-constexpr int kCompWide = 256;  // lists up to this long are ranked from shared memory
+constexpr int kCompGroup = 2;   // pairs whose records are read together
+constexpr int kCompWide = 256;  // lists of up to this many covering pairs are ranked in shared memory
+
+// A tile's place: origin in pixels (x | y << 16), side and first pixel of its problem.
+struct TilePos {
+  unsigned xy;
+  int res;
+  long long pix;
+};
+// The places of tiles base + lane (a lane beyond `count` repeats the last): the problem of the first, by
+// one round of loads over the lanes for up to 1024 problems, then stepped to the lane's own.
+__device__ __forceinline__ TilePos locate_tiles(const Dev& d, int base, int count, int T) {
+  const int lane = threadIdx.x & 31, tile = base + min(lane, count - 1);
+  int p = 0;
+  if (d.n_probs > 1) {
+    if (d.n_probs <= 1024) {
+      p = -1;
+      for (int i = 0; i < d.n_probs; i += 32)
+        p += __popc(__ballot_sync(0xffffffffu, i + lane < d.n_probs && d.prob_tile_base[min(i + lane, d.n_probs)] <= base));
+    } else {
+      p = find_prob(d.prob_tile_base, d.n_probs, base);
+    }
+    while (p + 1 < d.n_probs && d.prob_tile_base[p + 1] <= tile) ++p;
+  }
+  const int lt = tile - d.prob_tile_base[p], ntx = d.prob_ntx[p];
+  // lt / ntx by a float reciprocal, off by at most one (lt <= 2^24 is exact)
+  int ty = (int)((float)lt * __frcp_rn((float)ntx));
+  int tx = lt - ty * ntx;
+  if (tx < 0) {
+    ty -= 1;
+    tx += ntx;
+  } else if (tx >= ntx) {
+    ty += 1;
+    tx -= ntx;
+  }
+  return {(unsigned)(tx * T) | (unsigned)(ty * T) << 16, d.prob_res[p], d.prob_pix_base[p]};
+}
+
 template <int T>
-__global__ void __launch_bounds__(kCompWarps * 32) k_composite(Dev d, float* out_bw, float* out_tau) {
+__global__ void __launch_bounds__(kCompWarps * 32, 9) k_composite(Dev d, float* out_bw, float* out_tau, int flags,
+                                                                  int C) {
+  constexpr int UNITS = T * T / 64, NP = T * T, DY = 32 / T;
+  __shared__ unsigned s_ord[kCompWarps][kCompWide];   // the covering pairs' slots and classes, in order
+  __shared__ unsigned s_elem[kCompWarps][kCompWide];  // a long list's element ids, in list order
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int stride = (UNITS == 1 ? gridDim.x * kCompWarps : gridDim.x) * C;
+  const int unit = UNITS == 1 ? 0 : wid;
+  int base = (UNITS == 1 ? blockIdx.x * kCompWarps + wid : blockIdx.x) * C;
+  // what the level switch wrote is read before the emission has completed
+  TilePos pos{};
+  float empty = 0.0f;
+  auto place = [&]() {
+    const int count = min(C, d.total_tiles - base);
+    pos = locate_tiles(d, base, count, T);
+    if ((flags & kCompLoss) && lane < count) empty = d.loss0[(base + lane) * UNITS + unit];
+  };
+  if (base < d.total_tiles) place();
   pdl_enter();
-  constexpr int NP = T * T, PPL = NP / 32;
-  __shared__ int s_slot[kCompWarps][32];
-  __shared__ uint8_t s_cls[kCompWarps][32];
-  __shared__ int s_wide[kCompWarps][kCompWide];  // a long list's element ids, in list order
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // the emission has completed: its work list is spent
     d.chunk_count[0] = d.chunk_count[1] = 0;
     d.work[0] = 0;
   }
   if (*d.status & kStatusNoBins) return;
   const float inv_rho = 1.0f / d.L.rho_px, pad = d.L.pad_px, tau = d.L.tau;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int* w_slot = s_slot[wid];
-  uint8_t* w_cls = s_cls[wid];
-  __shared__ int s_mmax;
-  if (threadIdx.x == 0) s_mmax = 0;
-  __syncthreads();
+  unsigned* w_ord = s_ord[wid];
+  unsigned* w_elem = s_elem[wid];
+  const int ux = lane % T, uy = unit * (64 / T) + lane / T;  // the lane's first pixel in a tile; the
+                                                             // second lies DY rows below
   int m_max = 0;  // the fullest list this warp saw (the host keeps the lists' capacity ahead of it)
-  for (int tile = blockIdx.x * kCompWarps + wid; tile < d.total_tiles; tile += gridDim.x * kCompWarps) {
-    int p, tx, ty, res;
-    tile_coords(d, tile, T, p, tx, ty, res);
-    const long long pixbase = d.prob_pix_base[p];
-    // the tile's pairs (emission order) and, for the next iteration, an empty list; the count and
-    // the first list entries are read together (an entry is used only below the count, and the
-    // slot it names is clamped into the buffer before its element and class are read)
-    const size_t lb = (size_t)tile * d.tile_cap;
-    int m = d.tile_n[tile];
-    const int sl0 = lane < d.tile_cap ? d.tile_list[lb + lane] : 0;
-    // the container coverage of the lane's pixels (independent of the pairs)
-    float cov[PPL];
-#pragma unroll
-    for (int k = 0; k < PPL; ++k) {
-      const int local = lane + 32 * k;
-      const int X = min(tx * T + local % T, res - 1), Y = min(ty * T + local / T, res - 1);
-      cov[k] = d.covc[pixbase + (long long)Y * res + X];
+  for (; base < d.total_tiles; base += stride) {
+    // ---- the run's tiles, one per lane ----
+    const bool mine = lane < C && base + lane < d.total_tiles;
+    int n = 0;
+    bool covered = false;
+    if (mine) {
+      n = d.tile_n[base + lane];
+      const unsigned first = d.tile_list[(size_t)(base + lane) * d.tile_cap].x;  // used when n = 1
+      if (!in_bounds(d, n >= 0 && n <= d.tile_cap)) n = 0;
+      covered = n > 1 || (n == 1 && first >> kSlotBits != kPairOut);
+      m_max = max(m_max, n);
     }
-    if (!in_bounds(d, m >= 0 && m <= d.tile_cap)) m = 0;
-    m_max = max(m_max, m);
-    __syncwarp();  // the previous tile's readers of this warp's lists and of tile_n are done
-    if (lane == 0) {
-      d.tile_n[tile] = 0;
-      d.tile_m[tile] = m;
+    if (UNITS > 1) __syncthreads();  // every unit has the tiles' counts
+    if (mine && unit == 0) {  // for the next iteration, empty lists
+      d.tile_n[base + lane] = 0;
+      d.tile_m[base + lane] = n;
     }
-    const bool small = m <= 32;
-    int* sorted = d.tile_sorted + lb;
-    int* sorted_slot = d.tile_sorted_slot + lb;
-    if (small) {
-      const int sl = (unsigned)sl0 < (unsigned)d.cap ? sl0 : 0;
-      const int v0 = d.pair_elem[sl];
-      const uint8_t c0 = d.pair_cls[sl];
-      const int v = lane < m ? v0 : 0;
-      int r = 0;
-      for (int j = 0; j < m; ++j) r += __shfl_sync(0xffffffffu, v, j) < v ? 1 : 0;
-      if (lane < m) {
-        w_slot[r] = sl;
-        w_cls[r] = c0;
-        sorted[r] = v;
-        sorted_slot[r] = sl;
-      }
-    } else if (m <= kCompWide) {
-      // the element ids read once (independent loads), then each entry ranked against them all
-      if (lane == 0 && d.paths) atomicAdd(&d.paths[2], 1ull);
-      int* wv = s_wide[wid];
-      for (int i = lane; i < m; i += 32) wv[i] = d.pair_elem[d.tile_list[lb + i]];
-      __syncwarp();
-      for (int i = lane; i < m; i += 32) {
-        const int vi = wv[i];
+    const unsigned todo0 = __ballot_sync(0xffffffffu, covered);
+    auto tile_at = [&](int b) -> TilePos {
+      return {__shfl_sync(0xffffffffu, pos.xy, b), __shfl_sync(0xffffffffu, pos.res, b),
+              __shfl_sync(0xffffffffu, pos.pix, b)};
+    };
+    auto no_coverage = [&](const TilePos& at) {  // Ihat = 1, A_tau = 0
+      const int X = (int)(at.xy & 0xffffu) + ux, Y = (int)(at.xy >> 16) + uy, off = Y * at.res + X;
+      const bool in0 = X < at.res && Y < at.res, in1 = X < at.res && Y + DY < at.res;
+      auto fill = [&](float* img, float v) {
+        if (in0) img[at.pix + off] = v;
+        if (in1) img[at.pix + off + DY * at.res] = v;
+      };
+      if (flags & kCompAllI) fill(d.img_I, 1.0f);
+      if (out_bw) fill(out_bw, 1.0f);
+      if (out_tau) fill(out_tau, 0.0f);
+    };
+    if ((flags & kCompLoss) && mine && !covered)
+      d.lossA[(base + lane) * UNITS + unit] = make_float4(empty, 0.0f, 0.0f, 0.0f);
+    if ((flags & kCompAllI) || out_bw || out_tau)
+      for (unsigned b = __ballot_sync(0xffffffffu, mine) & ~todo0; b; b &= b - 1u) no_coverage(tile_at(__ffs((int)b) - 1));
+    // ---- the covered ones, one at a time ----
+    uint2 ent = make_uint2(0u, 0u);
+    auto fetch = [&](int b) {  // for lane l, entry l of tile base + b (used only below the count)
+      if (lane < d.tile_cap) ent = d.tile_list[(size_t)(base + b) * d.tile_cap + lane];
+    };
+    if (todo0) fetch(__ffs((int)todo0) - 1);
+    for (unsigned todo = todo0; todo;) {
+      const int b = __ffs((int)todo) - 1, cur = base + b;
+      todo &= todo - 1u;
+      const int m = __shfl_sync(0xffffffffu, n, b);
+      const TilePos at = tile_at(b);
+      const uint2 e0 = ent;
+      if (todo) fetch(__ffs((int)todo) - 1);
+      const int X = (int)(at.xy & 0xffffu) + ux, Y = (int)(at.xy >> 16) + uy, off = Y * at.res + X;
+      const bool in0 = X < at.res && Y < at.res, in1 = X < at.res && Y + DY < at.res;
+      // the covering pairs in element order: w_ord[0..na)
+      const size_t lb = (size_t)cur * d.tile_cap;
+      int na = 0;
+      bool near = false, wide = false;
+      __syncwarp();  // the previous tile's readers of this warp's lists are done
+      if (m <= 32) {
+        const unsigned cls = e0.x >> kSlotBits;
+        const bool act = lane < m && cls != kPairOut;
+        const unsigned bal = __ballot_sync(0xffffffffu, act);
+        near = __any_sync(0xffffffffu, act && cls == kPairNear);
+        na = __popc(bal);
         int r = 0;
-        for (int j = 0; j < m; ++j) r += wv[j] < vi ? 1 : 0;  // one address for every lane
-        sorted[r] = vi;
-        sorted_slot[r] = d.tile_list[lb + i];
-      }
-    } else {
-      if (lane == 0 && d.paths) atomicAdd(&d.paths[2], 1ull);
-      for (int i = lane; i < m; i += 32) {
-        const int si = d.tile_list[lb + i], vi = d.pair_elem[si];
-        int r = 0;
-        for (int j = 0; j < m; ++j) r += d.pair_elem[d.tile_list[lb + j]] < vi ? 1 : 0;
-        sorted[r] = vi;
-        sorted_slot[r] = si;
-      }
-    }
-    __syncwarp();  // the ordered list is visible to the whole warp
-    // products over the pairs in element order; the pair loop is outermost so that a lane's loads
-    // of its PPL pixels are independent and in flight together
-    float keep[PPL], keept[PPL];
-    int zc[PPL], nfull[PPL];
-    bool partial[PPL];
-#pragma unroll
-    for (int k = 0; k < PPL; ++k) {
-      keep[k] = 1.0f;
-      keept[k] = 1.0f;
-      zc[k] = 0;
-      nfull[k] = 0;
-      partial[k] = false;
-    }
-    // in groups of kCompGroup pairs whose signed distances are read before any is used
-    for (int i0 = 0; i0 < m; i0 += kCompGroup) {
-      float sd[kCompGroup][PPL];
-      uint8_t cls[kCompGroup];
-#pragma unroll
-      for (int u = 0; u < kCompGroup; ++u) {
-        const int i = i0 + u;
-        cls[u] = kPairOut;
-        if (i < m) {
-          const int slot = small ? w_slot[i] : sorted_slot[i];
-          cls[u] = small ? w_cls[i] : d.pair_cls[slot];
-#pragma unroll
-          for (int k = 0; k < PPL; ++k)  // an inside pair has c = c^pad = 1: sd = +1e30 gives that
-            sd[u][k] = cls[u] == kPairNear ? d.saved[(size_t)slot * NP + lane + 32 * k].x : kFar;
+        if (na > 1)
+          for (unsigned q = bal; q; q &= q - 1u) r += __shfl_sync(0xffffffffu, e0.y, __ffs((int)q) - 1) < e0.y ? 1 : 0;
+        if (act) w_ord[r] = e0.x;
+      } else {
+        if (lane == 0 && unit == 0 && d.paths) atomicAdd(&d.paths[2], 1ull);
+        // the covering pairs' ids compacted into shared memory, then ranked against one another there
+        // (one address for every lane); beyond kCompWide of them, ranked in global memory
+        for (int i0 = 0; i0 < m; i0 += 32) {
+          const uint2 e = i0 + lane < m ? d.tile_list[lb + i0 + lane] : make_uint2(0u, 0u);
+          const unsigned cls = e.x >> kSlotBits;
+          const bool act = i0 + lane < m && cls != kPairOut;
+          const unsigned bal = __ballot_sync(0xffffffffu, act);
+          near |= __any_sync(0xffffffffu, act && cls == kPairNear);
+          const int k = na + __popc(bal & ((1u << lane) - 1u));
+          if (act && k < kCompWide) w_elem[k] = e.y;
+          na += __popc(bal);
+        }
+        __syncwarp();
+        wide = na > kCompWide;
+        unsigned* out = wide ? d.tile_sorted + lb : w_ord;
+        for (int i = lane; i < m; i += 32) {
+          const uint2 e = d.tile_list[lb + i];
+          if (e.x >> kSlotBits == kPairOut) continue;
+          int r = 0;
+          if (!wide)
+            for (int j = 0; j < na; ++j) r += w_elem[j] < e.y ? 1 : 0;
+          else
+            for (int j = 0; j < m; ++j) {
+              const uint2 f = d.tile_list[lb + j];
+              r += f.x >> kSlotBits != kPairOut && f.y < e.y ? 1 : 0;
+            }
+          out[r] = e.x;  // (the units of a tile write the same values to the global list)
         }
       }
+      __syncwarp();  // the ordered list is visible to the whole warp
+      if (na == 0) {  // every listed pair is outside
+        no_coverage(at);
+        if ((flags & kCompLoss) && lane == b) d.lossA[cur * UNITS + unit] = make_float4(empty, 0.0f, 0.0f, 0.0f);
+        continue;
+      }
+      float cov[2] = {0.0f, 0.0f};
+      if (flags & kCompLoss) {
+        if (in0) cov[0] = d.covc[at.pix + off];
+        if (in1) cov[1] = d.covc[at.pix + off + DY * at.res];
+      }
+      // products over the pairs in element order, in groups of kCompGroup pairs whose signed
+      // distances are read before any is used
+      float keep[2] = {1.0f, 1.0f}, keept[2] = {1.0f, 1.0f};
+      int nfull[2] = {0, 0}, npos[2] = {0, 0};  // pairs with c^pad = 1, with c^pad > 0
+      const float2* sv = d.saved + unit * 64 + lane;
+      for (int i0 = 0; i0 < na; i0 += kCompGroup) {
+        if (wide && i0 % kCompWide == 0) {  // the next stretch of a very long list
+          __syncwarp();
+          for (int i = lane; i < min(kCompWide, na - i0); i += 32) w_ord[i] = d.tile_sorted[lb + i0 + i];
+          __syncwarp();
+        }
+        float sd[kCompGroup][2];
+        unsigned ent_u[kCompGroup];
 #pragma unroll
-      for (int u = 0; u < kCompGroup; ++u) {
-        if (cls[u] == kPairOut) continue;  // c = c^pad = 0: factors of 1
+        for (int u = 0; u < kCompGroup; ++u) {
+          ent_u[u] = i0 + u < na ? w_ord[(i0 + u) % kCompWide] : kPairOut << kSlotBits;
+          if (ent_u[u] >> kSlotBits == kPairNear) {
+            const float2* rec = sv + (size_t)(ent_u[u] & kSlotMask) * NP;
+            sd[u][0] = rec[0].x;
+            sd[u][1] = rec[32].x;
+          }
+        }
 #pragma unroll
-        for (int k = 0; k < PPL; ++k) {
-          const float x = sd[u][k] * inv_rho;
-          const float omc = Sfun(-x), cp = Sfun((sd[u][k] + pad) * inv_rho);
-          if (omc == 0.0f) zc[k] += 1;
-          else keep[k] *= omc;
-          keept[k] *= 1.0f - tau * cp;
-          nfull[k] += cp == 1.0f;
-          partial[k] |= cp > 0.0f && cp < 1.0f;
+        for (int u = 0; u < kCompGroup; ++u) {
+          const unsigned cls = ent_u[u] >> kSlotBits;  // (the same in every lane)
+          if (cls == kPairNear) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const float omc = Sfun(-sd[u][k] * inv_rho), cp = Sfun((sd[u][k] + pad) * inv_rho);
+              keep[k] *= omc;
+              keept[k] *= 1.0f - tau * cp;
+              nfull[k] += cp == 1.0f;
+              npos[k] += cp > 0.0f;
+            }
+          } else if (cls == kPairIn) {  // c = c^pad = 1
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              keep[k] = 0.0f;
+              keept[k] *= 1.0f - tau;
+              nfull[k] += 1;
+              npos[k] += 1;
+            }
+          }
         }
       }
-    }
-    float lc = 0.0f, lo = 0.0f, ld = 0.0f;
+      const bool grad = (flags & kCompLoss) && near;  // the adjoint reads this unit's images
+      float lc = 0.0f, lo = 0.0f, ld = 0.0f;
 #pragma unroll
-    for (int k = 0; k < PPL; ++k) {
-      const int local = lane + 32 * k;
-      const int X = tx * T + local % T, Y = ty * T + local / T;
-      if (X >= res || Y >= res) continue;
-      const long long pix = pixbase + (long long)Y * res + X;
-      const float ihat = zc[k] ? 0.0f : keep[k];
-      const float W = cov[k] >= 0.5f ? d.L.w_in : d.L.w_out;
-      const float df = ihat - (1.0f - cov[k]);
-      lc += W * df * df;
-      const float A = 1.0f - keept[k];
-      // the kink of max(0, A - tau): one fully covering element gives A = tau exactly and any
-      // other element with c^pad > 0 lifts A above it, by less than float can resolve when that
-      // c^pad is tiny; so the side of the kink is taken from the counts in that case (exact)
-      const bool over = nfull[k] >= 2 || (nfull[k] == 1 ? partial[k] : A > tau);
-      lo += over ? fmaxf(A - tau, 0.0f) : 0.0f;
-      ld += (1.0f - ihat) * force_potential(d.L, ((float)X + 0.5f) / (float)res, ((float)Y + 0.5f) / (float)res);
-      d.img_I[pix] = ihat;
-      d.img_Pt[pix] = over ? -keept[k] : keept[k];  // the sign carries the side of the kink
-      if (out_bw) out_bw[pix] = ihat;
-      if (out_tau) out_tau[pix] = A;
+      for (int k = 0; k < 2; ++k) {
+        if (!(k ? in1 : in0)) continue;
+        const int o = off + k * DY * at.res;
+        const float ihat = keep[k];
+        const float A = 1.0f - keept[k];
+        if (flags & kCompLoss) {
+          const float W = cov[k] >= 0.5f ? d.L.w_in : d.L.w_out;
+          const float df = ihat - (1.0f - cov[k]);
+          lc += W * df * df;
+          // the kink of max(0, A - tau): one fully covering element gives A = tau exactly and any
+          // other element with c^pad > 0 lifts A above it, by less than float can resolve when that
+          // c^pad is tiny; so the side of the kink is taken from the counts in that case (exact)
+          const bool over = nfull[k] >= 2 || (nfull[k] == 1 ? npos[k] > 1 : A > tau);
+          lo += over ? fmaxf(A - tau, 0.0f) : 0.0f;
+          // the downward potential 1 - y in pixels (exact), divided by the side once per unit
+          const float fy = (float)(Y + k * DY) + 0.5f;
+          ld += (1.0f - ihat) * (d.L.force_kind == 0
+                                     ? (float)at.res - fy
+                                     : force_potential(d.L, ((float)X + 0.5f) / (float)at.res, fy / (float)at.res));
+          if (grad) d.img_Pt[at.pix + o] = over ? -keept[k] : keept[k];  // the sign: the side of the kink
+        }
+        if (grad || (flags & kCompAllI)) d.img_I[at.pix + o] = ihat;
+        if (out_bw) out_bw[at.pix + o] = ihat;
+        if (out_tau) out_tau[at.pix + o] = A;
+      }
+      if (flags & kCompLoss) {
+        // fixed-order sums of the three partials, in one tree: after two steps lane l carries value
+        // l / 8 (lc, lo, ld, none)
+        const bool h = lane & 16, q = lane & 8;
+        const float a = (h ? ld : lc) + __shfl_xor_sync(0xffffffffu, h ? lc : ld, 16);
+        const float b2 = (h ? 0.0f : lo) + __shfl_xor_sync(0xffffffffu, h ? lo : 0.0f, 16);
+        float v = (q ? b2 : a) + __shfl_xor_sync(0xffffffffu, q ? a : b2, 8);
+        for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 16 && d.L.force_kind == 0) v /= (float)at.res;
+        if ((lane & 7) == 0) reinterpret_cast<float*>(d.lossA + cur * UNITS + unit)[lane >> 3] = v;
+      }
     }
-    for (int o = 16; o; o >>= 1) {  // fixed-order sums of the three partials
-      lc += __shfl_xor_sync(0xffffffffu, lc, o);
-      lo += __shfl_xor_sync(0xffffffffu, lo, o);
-      ld += __shfl_xor_sync(0xffffffffu, ld, o);
+    if (base + stride < d.total_tiles) {
+      base += stride;
+      place();
+      base -= stride;
     }
-    if (lane == 0) d.lossA[tile] = make_float4(lc, lo, ld, 0.0f);
   }
-  if (lane == 0) atomicMax(&s_mmax, m_max);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_mmax > 0) atomicMax(d.tile_max, s_mmax);
+  // (the host asks only whether a list passed 3/4 of the capacity)
+  if (m_max * 4 > d.tile_cap * 3) atomicMax(d.tile_max, m_max);
+}
+
+// Per level: the containment loss of a unit that no element covers (Ihat = 1), summed as above.
+template <int T>
+__global__ void __launch_bounds__(kCompWarps * 32) k_empty_loss(Dev d) {
+  constexpr int UNITS = T * T / 64, DY = 32 / T;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int u = blockIdx.x * kCompWarps + wid;
+  if (u >= d.total_tiles * UNITS) return;
+  const TilePos at = locate_tiles(d, u / UNITS, 1, T);
+  const int X = (int)(at.xy & 0xffffu) + lane % T, Y = (int)(at.xy >> 16) + (u % UNITS) * (64 / T) + lane / T;
+  float lc = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (X >= at.res || Y + k * DY >= at.res) continue;
+    const float cov = d.covc[at.pix + (long long)(Y + k * DY) * at.res + X];
+    const float W = cov >= 0.5f ? d.L.w_in : d.L.w_out;
+    const float df = 1.0f - (1.0f - cov);
+    lc += W * df * df;
+  }
+  for (int o = 16; o; o >>= 1) lc += __shfl_xor_sync(0xffffffffu, lc, o);
+  if (lane == 0) d.loss0[u] = lc;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -849,21 +983,28 @@ struct TileCfg<16> {
 
 template <int T>
 static cudaError_t fwd_t(const Dev& d, cudaStream_t s, int pair_grid, int tile_grid, float* bw,
-                         float* tau, int part) {
+                         float* tau, int part, int flags) {
   cudaError_t e = cudaSuccess;
   if (part & 1)
     e = d.emit_threads == 256 ? klaunch(d.pdl, k_raster_chunks<T, 256>, pair_grid, 256, 0, s, d)
                               : klaunch(d.pdl, k_raster_chunks<T, 128>, pair_grid, 128, 0, s, d);
-  if (e == cudaSuccess && (part & 2))
-    e = klaunch(d.pdl, k_composite<T>, tile_grid, kCompWarps * 32, 0, s, d, bw, tau);
+  if (e == cudaSuccess && (part & 2)) {
+    // tiles a warp takes at once: a power of two that leaves four resident waves of blocks, so that dense
+    // and empty stretches even out; then one run per warp
+    const int per_block = T == 8 ? kCompWarps : 1;
+    int C = 1;
+    while (C < 32 && 2ll * C * 4 * tile_grid * per_block <= d.total_tiles) C *= 2;
+    const int grid = C > 1 ? (d.total_tiles + C * per_block - 1) / (C * per_block) : tile_grid;
+    e = klaunch(d.pdl, k_composite<T>, grid, kCompWarps * 32, 0, s, d, bw, tau, flags, C);
+  }
   return e;
 }
 
 cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int tile_grid,
-                              float* out_bw, float* out_tau, int part) {
+                              float* out_bw, float* out_tau, int part, int flags) {
   switch (d.tile) {
-    case 8: return fwd_t<8>(d, s, pair_grid, tile_grid, out_bw, out_tau, part);
-    case 16: return fwd_t<16>(d, s, pair_grid, tile_grid, out_bw, out_tau, part);
+    case 8: return fwd_t<8>(d, s, pair_grid, tile_grid, out_bw, out_tau, part, flags);
+    case 16: return fwd_t<16>(d, s, pair_grid, tile_grid, out_bw, out_tau, part, flags);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -887,6 +1028,9 @@ cudaError_t launch_container(const Dev& d, cudaStream_t s) {
     case 16: k_container<16, TileCfg<16>::NT><<<d.total_tiles, TileCfg<16>::NT, 0, s>>>(d); break;
     default: return cudaErrorInvalidValue;
   }
+  const int units = d.total_tiles * (d.tile * d.tile / 64), grid = (units + kCompWarps - 1) / kCompWarps;
+  if (d.tile == 8) k_empty_loss<8><<<grid, kCompWarps * 32, 0, s>>>(d);
+  else k_empty_loss<16><<<grid, kCompWarps * 32, 0, s>>>(d);
   return cudaGetLastError();
 }
 
@@ -901,7 +1045,7 @@ static void per_sm_t(int emit_threads, RasterOcc* o) {
   o->bwd_per_sm = b > 0 ? b : 1;
   o->tile_per_sm = c > 0 ? c : 1;
   o->bwd_pairs_per_block = kPairWarps;
-  o->tiles_per_block = kCompWarps;
+  o->tiles_per_block = T == 8 ? kCompWarps : 1;
 }
 
 void raster_occupancy(int tile, int emit_threads, RasterOcc* o) {
