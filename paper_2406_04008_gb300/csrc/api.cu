@@ -876,6 +876,12 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(upload(h->owned, p_vloc, h->vloc));
   CKC(upload(h->owned, p_peb, h->prob_elem_base));
   CKC(upload(h->owned, p_ring, h->ring_pts));
+  std::vector<float2> ring_f(h->ring_pts.size() / 2);
+  for (size_t i = 0; i < ring_f.size(); ++i)
+    ring_f[i] = make_float2((float)h->ring_pts[2 * i], (float)h->ring_pts[2 * i + 1]);
+  float2* p_ring_f;
+  CKC(upload(h->owned, p_ring_f, ring_f));
+  d.ring_f = p_ring_f;
   CKC(upload(h->owned, p_roff, h->ring_off));
   CKC(upload(h->owned, p_prb, h->prob_ring_base));
   d.elem_prob = p_elem_prob;

@@ -67,6 +67,7 @@ struct Dev {
                                 //   k_ctrl_step when the outlines are fitted)
   const int* prob_elem_base;    // [P+1]
   const double* ring_pts;       // container rings, unit coords (double)
+  const float2* ring_f;         //   and as given
   const int* ring_off;          // [total rings + 1]
   const int* prob_ring_base;    // [P+1] into ring_off
   // ---- level ----

@@ -349,35 +349,27 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
 // Per dilation tile, once per level: whether the container coverage is nonzero on the tile, and
 // whether it is nonzero within the halo of the widest kernel; each flag also lists the tile for the
 // pass that visits it (the forward pass the first kind, the adjoint the second).
-__global__ void k_dtile_flags(Dev d, int h) {
-  __shared__ int s_own, s_halo;
+__global__ void __launch_bounds__(256) k_dtile_flags(Dev d, int h) {
   for (int dt = blockIdx.x; dt < d.total_dtiles; dt += gridDim.x) {
     const int p = find_prob_d(d.prob_dtile_base, d.n_probs, dt);
     const int res = d.prob_res[p], nd = (res + kDT - 1) / kDT, ld = dt - d.prob_dtile_base[p];
     const int x0 = (ld % nd) * kDT, y0 = (ld / nd) * kDT;
-    const long long pb = d.prob_pix_base[p];
-    if (threadIdx.x == 0) s_own = s_halo = 0;
-    __syncthreads();
-    const int S = kDT + 2 * h;
-    int own = 0, halo = 0;
-    for (int idx = threadIdx.x; idx < S * S; idx += blockDim.x) {
-      const int rr = idx / S, cc = idx % S;
-      const int Y = y0 + rr - h, X = x0 + cc - h;
-      if (X < 0 || Y < 0 || X >= res || Y >= res) continue;
-      if (d.covc[pb + (long long)Y * res + X] > 0.0f) {
-        halo = 1;
-        if (rr >= h && rr < h + kDT && cc >= h && cc < h + kDT) own = 1;
-      }
-    }
-    if (own) atomicOr(&s_own, 1);
-    if (halo) atomicOr(&s_halo, 1);
-    __syncthreads();
+    const float* cov = d.covc + d.prob_pix_base[p];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    bool own = false, halo = false;
+    for (int Y = max(y0 - h, 0) + wid; Y < min(y0 + kDT + h, res); Y += 8)
+      for (int X = max(x0 - h, 0) + lane; X < min(x0 + kDT + h, res); X += 32)
+        if (cov[Y * res + X] > 0.0f) {
+          halo = true;
+          own |= Y >= y0 && Y < y0 + kDT && X >= x0 && X < x0 + kDT;
+        }
+    own = __syncthreads_or(own);
+    halo = __syncthreads_or(halo);
     if (threadIdx.x == 0) {
-      d.dtile_flags[dt] = (uint8_t)((s_own ? kFlagOwn : 0) | (s_halo ? kFlagHalo : 0));
-      if (s_own) d.dtile_list[atomicAdd(&d.dtile_n[0], 1)] = dt;
-      if (s_halo) d.dtile_list[d.total_dtiles + atomicAdd(&d.dtile_n[1], 1)] = dt;
+      d.dtile_flags[dt] = (uint8_t)((own ? kFlagOwn : 0) | (halo ? kFlagHalo : 0));
+      if (own) d.dtile_list[atomicAdd(&d.dtile_n[0], 1)] = dt;
+      if (halo) d.dtile_list[d.total_dtiles + atomicAdd(&d.dtile_n[1], 1)] = dt;
     }
-    __syncthreads();
   }
 }
 

