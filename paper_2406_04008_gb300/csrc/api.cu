@@ -84,9 +84,7 @@ struct collage_s {
   bool ctl_current = false;  // h_ctl[1] (step count) and h_ctl[3] (pending) are the device's:
                              // no step was enqueued since the last read
   cudaStream_t cap_stream = nullptr;
-  cudaStream_t aux_stream = nullptr;  // side branch of an iteration (the loss assembly)
   cudaStream_t body_stream = nullptr;  // captures the loop bodies of the schedule graph
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaGraphExec_t graph = nullptr;  // one iteration at the current level
   cudaGraphExec_t host_graph = nullptr;  // one iteration taking its params from h_in, then the
                                          // gathering kernel writing h_stage (collage_step_host)
@@ -177,13 +175,10 @@ collage_s::~collage_s() {
   if (sched) cudaGraphExecDestroy(sched);
   if (cap_stream) cudaStreamDestroy(cap_stream);
   if (body_stream) cudaStreamDestroy(body_stream);
-  if (aux_stream) cudaStreamDestroy(aux_stream);
   if (met_obj) cudaFree(met_obj);
   if (met_gcol) cudaFree(met_gcol);
   if (met_cnt) cudaFree(met_cnt);
   if (mat_buf) cudaFree(mat_buf);
-  if (ev_fork) cudaEventDestroy(ev_fork);
-  if (ev_join) cudaEventDestroy(ev_join);
   if (h_ctl) cudaFreeHost(h_ctl);
   if (h_stage) cudaFreeHost(h_stage);
   free_list(pair_bufs);
@@ -363,9 +358,9 @@ static collage_status ensure_pairs(collage_t h, size_t cap) {
   free_list(h->pair_bufs);
   h->pair_cap = 0;
   Dev& d = h->d;
-  CK(h, dmalloc(h->pair_bufs, d.live_list, cap));
+  CK(h, dmalloc(h->pair_bufs, d.live_list, cap * (tt / 64)));
   CK(h, dmalloc(h->pair_bufs, d.near_list, cap));
-  CK(h, dmalloc(h->pair_bufs, d.partial, cap));
+  CK(h, dmalloc(h->pair_bufs, d.partial, cap * (tt / 64)));
   CK(h, dmalloc(h->pair_bufs, d.saved, cap * tt));
   h->pair_cap = cap;
   h->saved_tile = tt;
@@ -604,17 +599,7 @@ static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* ou
   const int flags = bwd ? kCompLoss | (dil ? kCompAllI : 0) : out_bw ? 0 : kCompAllI;
   LAUNCH_("k_composite", launch_raster_fwd(d, s, h->pair_grid, h->tile_grid, out_bw, out_tau, 2, flags));
   MARK_(4);
-  // the loss assembly needs only the composite's and the distribution term's partials: it runs on
-  // a side stream beside the distribution adjoint and the raster adjoint (joined at the end of
-  // the iteration); under stage timing it stays on the main stream
-  const bool side = bwd && !ev;
   if (dil) LAUNCH_("k_dilate_fwd", launch_dilate(d, s, false));
-  if (side) {
-    STEP_(cudaEventRecord(h->ev_fork, s));
-    STEP_(cudaStreamWaitEvent(h->aux_stream, h->ev_fork, 0));
-    LAUNCH_("k_loss", launch_loss(d, h->aux_stream));
-    STEP_(cudaEventRecord(h->ev_join, h->aux_stream));
-  }
   if (dil) LAUNCH_("k_dilate_bwd", launch_dilate(d, s, true));
   MARK_(5);
   // in step mode the last block of the last gradient kernel marks this iteration's Adam step
@@ -624,11 +609,9 @@ static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* ou
   MARK_(6);
   if (bwd && d.deterministic) LAUNCH_("k_grad_reduce", launch_grad_reduce(d, s, mark));
   MARK_(7);
-  if (bwd && !side) LAUNCH_("k_loss", launch_loss(d, s));
   MARK_(8);
   // outline fitting: the points' gradient, and in step mode their Adam step and new outlines
   if (bwd && d.fit) LAUNCH_("k_ctrl_step", launch_ctrl_step(d, s, mode == kStep ? 1 : 0));
-  if (side) STEP_(cudaStreamWaitEvent(s, h->ev_join, 0));
   MARK_(9);
 #undef STEP_
 #undef LAUNCH_
@@ -938,7 +921,6 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(dmalloc(h->owned, d.segB, h->V));
   CKC(dmalloc(h->owned, d.segS, h->V));
   CKC(dmalloc(h->owned, d.tpx, h->N));
-  CKC(dmalloc(h->owned, d.bbox, h->N));
   CKC(dmalloc(h->owned, d.rect, h->N));
   CKC(dmalloc(h->owned, d.dq, h->N));
   CKC(cudaMemset(d.dq, 0, sizeof(float4) * h->N));
@@ -973,10 +955,7 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
     cudaGetLastError();
   }
   CKC(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
-  CKC(cudaStreamCreateWithFlags(&h->aux_stream, cudaStreamNonBlocking));
   CKC(cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking));
-  CKC(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-  CKC(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
 #undef CKC
   st = build_levels(h);
   if (st) return bail(st);
@@ -1758,10 +1737,10 @@ extern "C" collage_status collage_get_info(collage_t h, collage_info* out) {
   out->pair_capacity = h->d.cap;
   out->last_pairs = h->h_ctl ? h->h_ctl[2] : 0;
   // transform (with the previous Adam step and the pair slots), emission with signed distances,
-  // composite, (2 dilation), raster bwd, (gradient reduce), loss
+  // composite, (2 dilation), raster bwd with the loss assembly, (gradient reduce)
   const bool dil = h->d.L.gamma != 0.0f && h->d.L.n_dil > 0;
   out->kernels_per_iter = 3 + (dil ? 2 : 0) + 1 +
-                         (h->d.deterministic ? 1 : 0) + 1 + (h->d.fit ? 1 : 0);
+                         (h->d.deterministic ? 1 : 0) + (h->d.fit ? 1 : 0);
   unsigned long long paths[4] = {0, 0, 0, 0};
   CK(h, cudaDeviceSynchronize());
   CK(h, cudaMemcpy(paths, h->d.paths, sizeof(paths), cudaMemcpyDeviceToHost));

@@ -7,20 +7,9 @@
 // its tile's list; the composite then orders each tile's short list by element id before using it,
 // so every tile lists its elements in increasing order whatever the order of the atomics.  The tile rectangle follows a fixed float formula
 // (bin_rect), so the bins are bit-exact against the oracle's rule.
-#include <cfloat>
-
 #include "internal.h"
 
 namespace collage {
-
-__device__ __forceinline__ float warp_min(float x) {
-  for (int o = 16; o; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
-__device__ __forceinline__ float warp_max(float x) {
-  for (int o = 16; o; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
 
 // Tile rectangle of one element, float arithmetic in a fixed order with explicit round-to-nearest
 // intrinsics (no contraction):
@@ -151,16 +140,14 @@ __device__ __noinline__ void sincos_wide(float z, float (&s)[2], float (&c)[2]) 
 
 // E = 1 or 4 elements per block: the pending Adam step of the previous iteration, then segment records
 // (start, direction, end y, 1/|e|^2) of the vertices relative to the translation, translation in
-// pixels as a float hi/lo pair, outline box grown by the coverage margin, tile rectangle, the
-// element's pair slots and its emission chunks.
+// pixels as a float hi/lo pair, tile rectangle, the element's pair slots and its emission chunks.
 // In warp 0, eight lanes per element take the step (one parameter each of the first four, the two bias
 // powers on different lanes) and form the rotation-scale matrix; one barrier separates the step from
 // the vertices.  Lanes own consecutive vertices; a segment's end point is the next lane's start point,
 // shuffled, so each vertex is transformed once.
 // E = 1: warps 0..2 transform the vertices while warp 3 files the tile rectangle, the pair slots and
 // the chunk list, which do not depend on the vertices: the shortest chain for one element.
-// E = 4: each warp does both for one element, so that four elements share the step's instructions and
-// no block waits for a second barrier.  It is taken when the elements fill the device several times
+// E = 4: each warp does both for one element, so that four elements share the step's instructions.  It is taken when the elements fill the device several times
 // over (launch_transform), where issue slots rather than latency bound the kernel.
 constexpr int kTfThreads = 128;
 constexpr int kTfWideElems = 4096;  // elements from which a block takes four: the two forms meet here
@@ -171,7 +158,6 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
   static_assert(E == 1 || E == 4, "eight lanes per element in one warp, one warp per element or block");
   __shared__ RotFF s_rot[E];
   __shared__ float4 s_q[E];
-  __shared__ float s_box[4][kTfVertexWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int g = E == 1 ? blockIdx.x : min((int)blockIdx.x * E + wid, d.n_elems - 1);
   const bool live = E == 1 || (int)blockIdx.x * E + wid < d.n_elems;
@@ -294,18 +280,11 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     return;  // no barrier follows for this warp
   }
   const RotFF rot = s_rot[slot];
-  float xmin = FLT_MAX, ymin = FLT_MAX, xmax = -FLT_MAX, ymax = -FLT_MAX;
   for (int k0 = E == 4 ? 0 : wid * 32; k0 < nv; k0 += kStride) {  // warp-uniform trip count
     const int k = k0 + lane;
     const bool first = k0 < kStride;
     float2 a = make_float2(0.f, 0.f);
-    if (k < nv) {
-      a = vertex_px(first ? va0 : d.vloc[v0 + k], rot);
-      xmin = fminf(xmin, a.x);
-      xmax = fmaxf(xmax, a.x);
-      ymin = fminf(ymin, a.y);
-      ymax = fmaxf(ymax, a.y);
-    }
+    if (k < nv) a = vertex_px(first ? va0 : d.vloc[v0 + k], rot);
     float2 b;
     b.x = __shfl_down_sync(0xffffffffu, a.x, 1);
     b.y = __shfl_down_sync(0xffffffffu, a.y, 1);
@@ -328,34 +307,10 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     }
   }
   if (E == 4) file_chunks();
-  xmin = warp_min(xmin);
-  ymin = warp_min(ymin);
-  xmax = warp_max(xmax);
-  ymax = warp_max(ymax);
-  if (E == 1) {
-    if (lane == 0) {
-      s_box[0][wid] = xmin;
-      s_box[1][wid] = ymin;
-      s_box[2][wid] = xmax;
-      s_box[3][wid] = ymax;
-    }
-    // the vertex warps only (warp 3 has left): named barrier 1 over their threads
-    asm volatile("bar.sync 1, %0;" ::"n"(kTfVertexWarps * 32) : "memory");
-  }
   if (E == 1 ? threadIdx.x == 0 : lane == 0) {
-    for (int w = 1; E == 1 && w < kTfVertexWarps; ++w) {
-      xmin = fminf(xmin, s_box[0][w]);
-      ymin = fminf(ymin, s_box[1][w]);
-      xmax = fmaxf(xmax, s_box[2][w]);
-      ymax = fmaxf(ymax, s_box[3][w]);
-    }
-    const float fres = (float)res;
     float lx, ly;
-    const float hx = two_prod(q.x, fres, lx), hy = two_prod(q.y, fres, ly);
+    const float hx = two_prod(q.x, (float)res, lx), hy = two_prod(q.y, (float)res, ly);
     d.tpx[g] = make_float4(hx, hy, lx, ly);
-    // outline box relative to the translation, grown by the coverage margin (+ rounding slack)
-    const float m = d.L.rho_px + d.L.pad_px + hw * fres + 0.01f;
-    d.bbox[g] = make_float4(xmin - m, ymin - m, xmax + m, ymax + m);
   }
 }
 

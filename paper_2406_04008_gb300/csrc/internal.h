@@ -96,7 +96,6 @@ struct Dev {
   float2* segB;                 // [V] segment k: end point y, 1 / |direction|^2
   float* segS;                  // [V] segment k: dx/dy of its direction (0 if horizontal)
   float4* tpx;                  // [n] translation in px: (hi.x, hi.y, lo.x, lo.y)
-  float4* bbox;                 // [n] outline box relative to the translation, grown by the margin
   int4* rect;                   // [n] tile rectangle (tx0, ty0, tx1, ty1), empty if tx1 < tx0
   int* elem_pbase;              // [n] first pair slot of each element: its tile rectangle's pairs
                                 //   take consecutive slots, row-major (the transform allocates them)
@@ -120,9 +119,9 @@ struct Dev {
   int list_cap;                 // entries near_list holds
   int* chunk_count;             // [2] heavy and light chunks appended by the transform (the
                                 //   composite's block 0 zeroes them)
-  int4* live_list;              // [cap] pairs with some non-saturated pixel: (slot, element, tile
-                                //   column | row << 16, problem), the adjoint's work list (order
-                                //   depends on atomics)
+  int4* live_list;              // [cap * units per tile] units with some non-saturated pixel: (slot | unit <<
+                                //   kSlotBits, element, tile column | row << 16, problem), the adjoint's
+                                //   work list (order depends on atomics)
   float2* saved;                // [cap * tile*tile] (sd px, closest segment as int bits)
   float* covc;                  // [pix] container coverage
   float* img_I;                 // [pix] Ihat = prod(1 - c)
@@ -139,10 +138,10 @@ struct Dev {
                                 //   from total_dtiles, in no particular order (or null: all tiles)
   int* dtile_n;                 // [2] lengths of the two lists
   float4* dq;                   // [n] gradient
-  float4* partial;              // [cap] deterministic gradient partials, at emit position
+  float4* partial;              // [cap * units per tile] deterministic gradient partials, by slot
   float* loss_terms;            // [P*5]
   int* status;                  // [1]
-  int* step;                    // [1] Adam step count (the loss assembly advances it)
+  int* step;                    // [1] Adam step count (the last gradient kernel advances it)
   int* pending;                 // [1] 1: the Adam step `step` is computed (dq) but not yet applied
   int* sched_base;              // [1] Adam step count when the running schedule graph began
   int* work;                    // [8] per-iteration counters: [0] chunks taken by the emission's
@@ -289,8 +288,9 @@ cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int t
 cudaError_t prepare_dilate(int n_dil);  // sets dynamic shared memory limits (not capturable)
 cudaError_t launch_dilate(const Dev& d, cudaStream_t s, bool backward);
 cudaError_t launch_dtile_flags(const Dev& d, cudaStream_t s);  // once per level, after the container
-// mark_step: the kernel's last block marks the iteration's Adam step (step mode)
-cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int pair_grid, bool mark_step);
+// the adjoint and the loss assembly; mark_step: the kernel's last block marks the iteration's Adam step
+// (step mode)
+cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step);
 cudaError_t launch_grad_reduce(const Dev& d, cudaStream_t s, bool mark_step);
 // applies a pending Adam step to all elements and clears the flag (before params are read)
 cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out = nullptr);
@@ -302,7 +302,6 @@ cudaError_t launch_ctrl_step(const Dev& d, cudaStream_t s, int mode);
 cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
                             unsigned* cand, int* n_cand, float* clear, int* placed, int* axis_out,
                             float* width_out);
-cudaError_t launch_loss(const Dev& d, cudaStream_t s);
 // the captured level schedule: records the step count at the start of a run; sets a level's loop
 // condition (1 while fewer than `target` iterations of the run are done and nothing latched)
 cudaError_t launch_sched_begin(const Dev& d, cudaStream_t s);

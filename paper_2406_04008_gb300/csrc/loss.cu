@@ -1,5 +1,5 @@
-// Even-distribution term (Eq. 7), loss assembly (Eq. 8), the deterministic gradient reduction and
-// the flush of a pending Adam step.
+// Even-distribution term (Eq. 7), the deterministic gradient reduction and the flush of a pending Adam
+// step.
 //
 // Eq. 7 as implemented: K box kernels of widths 5 + 6k pixels (k = 0..K-1) dilate the occupancy
 // O = 1 - Ihat; D_k = min(1, B_k) with B_k the zero-padded box sum; the term sums
@@ -373,84 +373,27 @@ __global__ void __launch_bounds__(256) k_dtile_flags(Dev d, int h) {
   }
 }
 
-// One block per problem: fixed-order float sums of the tile partials (strided per thread, then a
-// shuffle tree within and across warps), then Eq. 8.  Float throughout: FP64 arithmetic is slow on
-// this part and 1e-7 relative is ample for a sum of non-negative partials.
-constexpr int kLossThreads = 1024;
-__device__ __forceinline__ float warp_sum_f(float x) {
-  for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-__global__ void __launch_bounds__(kLossThreads) k_loss(Dev d) {
-  pdl_enter();
-  __shared__ float s_red[4][kLossThreads / 32];
-  const int p = blockIdx.x;
-  const int units = d.tile * d.tile / 64;
-  const int t0 = d.prob_tile_base[p] * units, t1 = d.prob_tile_base[p + 1] * units;
-  const bool use_u = d.L.gamma != 0.0f && d.L.n_dil > 0;
-  float a = 0.f, b = 0.f, c = 0.f, u = 0.f;
-#pragma unroll 4
-  for (int t = t0 + (int)threadIdx.x; t < t1; t += kLossThreads) {
-    const float4 v = d.lossA[t];
-    a += v.x;
-    b += v.y;
-    c += v.z;
-  }
-  if (use_u) {
-    const int u0 = d.prob_dtile_base[p], u1 = d.prob_dtile_base[p + 1];
-#pragma unroll 4
-    for (int t = u0 + (int)threadIdx.x; t < u1; t += kLossThreads) u += d.lossU[t];
-  }
-  a = warp_sum_f(a);
-  b = warp_sum_f(b);
-  c = warp_sum_f(c);
-  u = warp_sum_f(u);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    s_red[0][w] = a;
-    s_red[1][w] = b;
-    s_red[2][w] = c;
-    s_red[3][w] = u;
-  }
-  __syncthreads();
-  if (w == 0) {
-    a = warp_sum_f(s_red[0][lane]);
-    b = warp_sum_f(s_red[1][lane]);
-    c = warp_sum_f(s_red[2][lane]);
-    u = warp_sum_f(s_red[3][lane]);
-    if (lane == 0) {
-      const float np = (float)d.prob_res[p] * (float)d.prob_res[p];
-      const float Lc = a / np, Lo = b / np, Ld = c / np;
-      float* out = d.loss_terms + 5 * p;
-      out[0] = Lc;
-      out[1] = Lo;
-      out[2] = u;
-      out[3] = Ld;
-      out[4] = d.L.alpha * Lc + d.L.beta * Lo + d.L.gamma * u + d.L.delta * Ld;
-    }
-  }
-}
-
-// Deterministic mode: each element sums its (tile, element) partials, one warp per element.  Its pairs
-// take consecutive slots, its tile rectangle row-major, so lane l reads slots l, l + 32, ... of them (no
+// Deterministic mode: each element sums its units' partials, one warp per element.  Its pairs
+// take consecutive slots, its tile rectangle row-major, so lane l reads partials l, l + 32, ... of them (no
 // search) and the 32 lane sums are added by a fixed shuffle tree; the order of every addition is fixed,
 // so the result is bitwise reproducible.  Bound by the latency of two loads (5000 elements, 369 k pairs:
 // 24.8 us when each pair was found by bisection in its tile's sorted list, 11.8 us now).
 constexpr int kReduceWarps = 8;
 __global__ void __launch_bounds__(kReduceWarps * 32) k_grad_reduce(Dev d, int mark) {
   pdl_enter();
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, units = d.tile * d.tile / 64;
   const int g = blockIdx.x * kReduceWarps + (threadIdx.x >> 5);
   if (g < d.n_elems && !(*d.status & kStatusNoBins)) {
     const int4 rc = d.rect[g];
     const int base = d.elem_pbase[g];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (rc.z >= rc.x && rc.w >= rc.y) {
-      const int n = (rc.z - rc.x + 1) * (rc.w - rc.y + 1);
+      const int n = (rc.z - rc.x + 1) * (rc.w - rc.y + 1) * units;
+      const float4* part = d.partial + (size_t)base * units;
 #pragma unroll 4
       for (int i = lane; i < n; i += 32) {
-        if (!in_bounds(d, base + i >= 0 && base + i < d.cap)) continue;
-        const float4 v = d.partial[base + i];
+        if (!in_bounds(d, base >= 0 && base + i / units < d.cap)) continue;
+        const float4 v = part[i];
         acc.x += v.x;
         acc.y += v.y;
         acc.z += v.z;
@@ -558,10 +501,6 @@ cudaError_t launch_dtile_flags(const Dev& d, cudaStream_t s) {
   if (d.L.n_dil <= 0 || !d.dtile_flags || !d.dtile_list) return cudaSuccess;
   k_dtile_flags<<<d.total_dtiles, 256, 0, s>>>(d, dil_r(d.L.n_dil - 1));
   return cudaGetLastError();
-}
-
-cudaError_t launch_loss(const Dev& d, cudaStream_t s) {
-  return klaunch(d.pdl, k_loss, d.n_probs, kLossThreads, 0, s, d);
 }
 
 cudaError_t launch_grad_reduce(const Dev& d, cudaStream_t s, bool mark_step) {

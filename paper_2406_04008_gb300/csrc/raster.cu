@@ -72,7 +72,7 @@ __device__ __forceinline__ void seg_update(SegQuery& Q, float dx, float dy, floa
 
 constexpr int kSegCap = 1024;   // container segments staged per chunk
 constexpr int kRowCross = 16;   // crossings listed per pixel row of an emission chunk
-constexpr int kPairWarps = 4;   // pairs per block of the per-pair adjoint (one per warp)
+constexpr int kPairWarps = 4;   // units per block of the adjoint (one per warp)
 constexpr float kFar = 1e30f;   // |sd| of a pixel farther than the coverage margin
 
 // Winding number of a point (element frame) over every segment of an outline: the crossing test of
@@ -96,38 +96,40 @@ __device__ __noinline__ int winding_all(const Dev& d, int v0, int ns, float px, 
 //     row-major from the base the transform allocated) and records it in the tile's list (a
 //     list beyond its capacity latches a status bit: the host grows the lists and runs again);
 //  2. passes once over the element's segments, staging them in shared memory by index: a segment
-//     whose box meets a tile's pixel-centre box grown by the coverage margin m = rho + pad
-//     (+ stroke half-width) (+ 0.06 px of slack) is near that tile (a bit per segment and tile);
+//     whose box meets a unit's pixel-centre box grown by the coverage margin m = rho + pad
+//     (+ stroke half-width) (+ 0.06 px of slack) is near that unit (a bit per segment and unit);
+//     units are the 64 pixels a warp takes at once: a tile of 8 x 8, or four rows of a tile of 16 x 16;
 //     for every pixel row of the chunk that a segment crosses (half-open in y, on the dy the
 //     pixels form) the crossing x is listed for the row, or, when it lies right of every pixel of
 //     the chunk, added to the row's backdrop (+1 upward, -1 downward);
 //  3. classifies the tiles: a tile that no segment is near has saturated coverage on every pixel
 //     (0 or 1, as the winding number of its first pixel says) and needs no per-pixel work;
-//  4. its warps take the near tiles one at a time: per pixel, the minimum squared distance over
-//     the tile's near segments in index order (the lowest index wins ties, as the oracle's scan
+//  4. its warps take the near tiles' units one at a time: per pixel, the minimum squared distance over
+//     the unit's near segments in index order (the lowest index wins ties, as the oracle's scan
 //     does); winding = row backdrop + listed crossings right of the pixel (a row with more than
 //     kRowCross crossings tests every segment); sd = +-distance within the margin, else +-1e30
-//     (saturated); the (sd, closest segment) record is saved and pairs with a non-saturated pixel
+//     (saturated); the (sd, closest segment) record is saved and units with a non-saturated pixel
 //     are listed for the adjoint.
 // Outlines of more than kStageSegs segments are not staged: their tiles test every segment's box
 // on the fly, reading the outline from global memory.
-// A pixel beyond the margin from every segment near its tile is beyond it from all segments (the
+// A pixel beyond the margin from every segment near its unit is beyond it from all segments (the
 // near test is conservative), so the distance minimum over the near ones is exact wherever it
 // matters, and the winding counts every crossing right of the pixel exactly once.
 // ------------------------------------------------------------------------------------------------
 constexpr int kStageSegs = 512;   // outline segments staged in shared memory
 constexpr int kLiveBatch = 32;
 
-// Tiles of the chunk whose grown pixel-centre box a segment's box [x0, x1] x [y0, y1] (absolute
-// px) meets: columns [*c0, *c1], rows [*r0, *r1] relative to the chunk origin, clipped to it.
-__device__ __forceinline__ void seg_tiles(float x0, float x1, float y0, float y1, float m, int T,
-                                          int tx0, int ty0, int ctw, int cth, int* c0, int* c1,
-                                          int* r0, int* r1) {
-  const float fT = (float)T, iT = 1.0f / fT;  // T is a power of two: x * (1 / T) is x / T exactly
-  *c0 = max((int)floorf((x0 - m - (fT - 0.5f)) * iT) + 1 - tx0, 0);
-  *c1 = min((int)floorf((x1 + m - 0.5f) * iT) - tx0, ctw - 1);
-  *r0 = max((int)floorf((y0 - m - (fT - 0.5f)) * iT) + 1 - ty0, 0);
-  *r1 = min((int)floorf((y1 + m - 0.5f) * iT) - ty0, cth - 1);
+// Units (T x 64 / T pixels) of the chunk whose grown pixel-centre box a segment's box [x0, x1] x [y0, y1]
+// (absolute px) meets: columns [*c0, *c1], rows [*r0, *r1] relative to the chunk's first unit (ux0, uy0),
+// clipped to it.
+template <int T>
+__device__ __forceinline__ void seg_units(float x0, float x1, float y0, float y1, float m, int ux0, int uy0,
+                                          int cuw, int cuh, int* c0, int* c1, int* r0, int* r1) {
+  constexpr float W = (float)T, iW = 1.0f / W, H = 64.0f / W, iH = 1.0f / H;  // powers of two: exact
+  *c0 = max((int)floorf((x0 - m - (W - 0.5f)) * iW) + 1 - ux0, 0);
+  *c1 = min((int)floorf((x1 + m - 0.5f) * iW) - ux0, cuw - 1);
+  *r0 = max((int)floorf((y0 - m - (H - 0.5f)) * iH) + 1 - uy0, 0);
+  *r1 = min((int)floorf((y1 + m - 0.5f) * iH) - uy0, cuh - 1);
 }
 
 // Squared distance from (dx, dy) to the segment a + u e, u in [0, 1], with f = e / |e|^2 (the
@@ -139,19 +141,24 @@ __device__ __forceinline__ float seg_d2(float dx, float dy, float4 s, float2 f) 
   return fmaf(qx, qx, qy * qy);
 }
 
-// NT threads per block (128 or 256, the autotuner's choice); registers capped so that 1024
-// threads (T = 8) or 512 (T = 16, eight pixels per lane) are resident per SM.
+// NT threads per block (128 or 256, the autotuner's choice); registers capped so that 1024 threads are
+// resident per SM.  Bound by issue slots and by the latency of each chunk's phases.  (With 16-px tiles a
+// warp used to take a whole tile, eight pixels a lane, 114 registers, and tested every segment near the
+// tile at each of them: 100 outlines of 320 segments at 1000^2 37 us, EM1 now; 16 disks at 128^2 13.5,
+// EM2 now.)
 template <int T, int NT>
-__global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunks(Dev d) {
+__global__ void __launch_bounds__(NT, 1024 / NT) k_raster_chunks(Dev d) {
   pdl_enter();
-  constexpr int CW = kChunkPx / T, NCT = CW * CW, NP = T * T, PPL = NP / 32;
+  constexpr int CW = kChunkPx / T, NCT = CW * CW, NP = T * T, UNITS = NP / 64, UH = 64 / T;
+  constexpr int NCU = NCT * UNITS;  // units of a chunk
   constexpr int ROWS = kChunkPx, MW = kStageSegs / 32;
   __shared__ float4 s_seg[kStageSegs];  // start (px, relative to the translation), direction
   __shared__ float2 s_f[kStageSegs];    // direction / |direction|^2
-  __shared__ unsigned s_mask[NCT][MW];  // bit j of tile k: segment j is near tile k
+  __shared__ unsigned s_mask[NCU][MW];  // bit j of unit k: segment j is near unit k
   __shared__ int s_slot[NCT];           // pair slot of each tile (-1: void)
   __shared__ unsigned char s_tn[NCT];   // some segment is near the tile
-  __shared__ int2 s_ntile[NCT];         // the near tiles: (pair slot, tile | column << 8 | row << 16)
+  __shared__ int2 s_unit[NCU];          // the near tiles' units: (pair slot | unit in the tile << kSlotBits,
+                                        //   unit | column << 8 | row << 16)
   __shared__ int2 s_row[ROWS];          // per pixel row: (crossings right of every pixel, listed)
   __shared__ float2 s_rx[ROWS][kRowCross];  // listed crossings: (x, +1 upward / -1 downward)
   __shared__ int s_nt, s_take;
@@ -207,9 +214,9 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
       s_slot[tid] = slot;
       s_tn[tid] = 0;
     }
-    for (int q = tid; q < nct * mw; q += NT) s_mask[q / mw][q % mw] = 0u;
+    for (int q = tid; q < nct * UNITS * mw; q += NT) s_mask[q / mw][q % mw] = 0u;
     for (int q = tid; q < ROWS; q += NT) s_row[q] = make_int2(0, 0);
-    const float4 tp = d.tpx[g], bb = d.bbox[g];
+    const float4 tp = d.tpx[g];
     const float hwpx = closed ? 0.0f : d.elem_hw[g] * (float)res;
     const float mrg = d.L.rho_px + pad + hwpx, mrg2 = mrg * mrg;
     const float tpx = tp.x + tp.z, tpy = tp.y + tp.w;
@@ -217,9 +224,10 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
     // the chunk's pixel-centre box in the element frame, as the pixels form dx and dy
     const float min_dx = ((float)X0 + 0.5f - tp.x) - tp.z;
     const float max_dx = ((float)(X0 + ncol - 1) + 0.5f - tp.x) - tp.z;
-    const float sl = mrg + 0.06f;  // near test margin with slack
+    const float sl = mrg + 0.06f, rsl = 0.02f + 5e-7f * fabsf(tpy);  // slack of the near test, of the rows
+    const int ux0 = tx0, uy0 = ty0 * UNITS, cuh = cth * UNITS;  // (a unit is as wide as a tile)
     __syncthreads();
-    // 2. one pass over the segments: staging, the tiles they are near, row crossings
+    // 2. one pass over the segments: staging, the units they are near, row crossings
     if (ns > kStageSegs && tid == 0 && d.paths) atomicAdd(&d.paths[1], 1ull);
     for (int j = tid; j < ns; j += NT) {
       const float4 sa = d.segA[v0 + j];
@@ -231,17 +239,18 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
       const float bx = sa.x + sa.z, by = sb.x;
       const float x0 = fminf(sa.x, bx), x1 = fmaxf(sa.x, bx), y0 = fminf(sa.y, by), y1 = fmaxf(sa.y, by);
       int c0, c1, r0, r1;
-      seg_tiles(x0 + tpx, x1 + tpx, y0 + tpy, y1 + tpy, sl, T, tx0, ty0, ctw, cth, &c0, &c1, &r0, &r1);
+      seg_units<T>(x0 + tpx, x1 + tpx, y0 + tpy, y1 + tpy, sl, ux0, uy0, ctw, cuh, &c0, &c1, &r0, &r1);
       for (int rr = r0; rr <= r1; ++rr)
         for (int cc = c0; cc <= c1; ++cc) {
-          if (!in_bounds(d, rr * ctw + cc < NCT)) continue;
-          s_tn[rr * ctw + cc] = 1;
+          if (!in_bounds(d, rr * ctw + cc < NCU)) continue;
+          s_tn[rr / UNITS * ctw + cc] = 1;
           if (staged) atomicOr(&s_mask[rr * ctw + cc][j >> 5], 1u << (j & 31));
         }
       if (closed && y1 > y0 && x1 > min_dx) {  // crosses some row right of the first pixel column
-        // candidate rows (one row of slack each side), then the exact half-open test
-        const int q0 = max((int)floorf(y0 + tpy - 0.5f) - Y0 - 1, 0);
-        const int q1 = min((int)ceilf(y1 + tpy - 0.5f) - Y0 + 1, nrow - 1);
+        // candidate rows (with slack for the rounding of these sums; most segments of a curve cross one
+        // row or none), then the exact half-open test
+        const int q0 = max((int)ceilf(y0 + tpy - 0.5f - rsl) - Y0, 0);
+        const int q1 = min((int)floorf(y1 + tpy - 0.5f + rsl) - Y0, nrow - 1);
         const float slope = d.segS[v0 + j];
         for (int q = q0; q <= q1; ++q) {
           if (!in_bounds(d, q < ROWS)) break;
@@ -282,46 +291,45 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
           }
         }
         cls = w != 0 ? kPairIn : kPairOut;
-        if (d.deterministic) d.partial[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (d.deterministic)
+          for (int u = 0; u < UNITS; ++u) d.partial[(size_t)slot * UNITS + u] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
       const int t = tb + (ty0 + tid / ctw) * ntx + tx0 + tid % ctw;
       const uint2 entry = make_uint2((unsigned)slot | cls << kSlotBits, (unsigned)g);
       if (place < d.tile_cap) d.tile_list[(size_t)t * d.tile_cap + place] = entry;
       else atomicOr(d.status, kStatusTileCap);
     }
-    if (tid < 32) {  // warp 0: the near tiles, in tile order
+    if (tid < 32) {  // warp 0: the near tiles' units, in order
       int n = 0;
-      for (int k0 = 0; k0 < nct; k0 += 32) {
-        const int k = k0 + lane;
-        const bool nr = k < nct && s_slot[k] >= 0 && s_tn[k];
+      for (int k0 = 0; k0 < nct * UNITS; k0 += 32) {
+        const int k = k0 + lane, ur = k / ctw, uc = k - ur * ctw, tl = ur / UNITS * ctw + uc;
+        const bool nr = k < nct * UNITS && s_slot[tl] >= 0 && s_tn[tl];
         const unsigned bal = __ballot_sync(0xffffffffu, nr);
-        if (nr) s_ntile[n + __popc(bal & ((1u << lane) - 1u))] = make_int2(s_slot[k], k | (k % ctw) << 8 | (k / ctw) << 16);
+        if (nr)
+          s_unit[n + __popc(bal & ((1u << lane) - 1u))] =
+              make_int2(s_slot[tl] | (int)((unsigned)(ur % UNITS) << kSlotBits), k | uc << 8 | ur << 16);
         n += __popc(bal);
       }
       if (lane == 0) s_nt = n;
     }
     __syncthreads();
     const int nt = s_nt;
-    // 4. the near tiles, one per warp at a time (the next one taken while this one is worked on)
+    // 4. the near tiles' units, one per warp at a time (the next one taken while this one is worked on)
     int ni = 0;
     if (lane == 0) ni = atomicAdd(&s_take, 1);
     ni = __shfl_sync(0xffffffffu, ni, 0);
     while (ni < nt) {
       int nn = 0;
       if (lane == 0) nn = atomicAdd(&s_take, 1);
-      const int2 nti = s_ntile[ni];
-      const int slot = nti.x, k = nti.y & 0xff, kr = nti.y >> 16;
-      const int tcx = tx0 + ((nti.y >> 8) & 0xff), tcy = ty0 + kr;
-      float dx[PPL], dy[PPL], best[PPL];
-      int bidx[PPL];
+      const int2 nti = s_unit[ni];
+      const int k = nti.y & 0xff, kc = (nti.y >> 8) & 0xff, kr = nti.y >> 16;
+      // the lane's pixels: rows q and q + 32 / T of the chunk, one column
+      const int q = kr * UH + lane / T;
+      const float dx = ((float)((tx0 + kc) * T + lane % T) + 0.5f - tp.x) - tp.z;
+      float dy[2], best[2] = {FLT_MAX, FLT_MAX};
+      int bidx[2] = {0, 0};
 #pragma unroll
-      for (int e = 0; e < PPL; ++e) {
-        const int local = lane + 32 * e;
-        dx[e] = ((float)(tcx * T + local % T) + 0.5f - tp.x) - tp.z;
-        dy[e] = ((float)(tcy * T + local / T) + 0.5f - tp.y) - tp.w;
-        best[e] = FLT_MAX;
-        bidx[e] = 0;
-      }
+      for (int e = 0; e < 2; ++e) dy[e] = ((float)(Y0 + q + e * (32 / T)) + 0.5f - tp.y) - tp.w;
       if (staged) {
         for (int w = 0; w < mw; ++w) {
           unsigned bits = s_mask[k][w];
@@ -331,8 +339,8 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
             const float4 sg = s_seg[j];
             const float2 f = s_f[j];
 #pragma unroll
-            for (int e = 0; e < PPL; ++e) {
-              const float d2 = seg_d2(dx[e], dy[e], sg, f);
+            for (int e = 0; e < 2; ++e) {
+              const float d2 = seg_d2(dx, dy[e], sg, f);
               if (d2 < best[e]) {
                 best[e] = d2;
                 bidx[e] = j;
@@ -341,20 +349,19 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
           }
         }
       } else {
-        // the tile's near segments by the same box test as the marks, from global memory
-        const int kc = k % ctw, kr = k / ctw;
+        // the unit's near segments by the same box test as the marks, from global memory
         for (int j = 0; j < ns; ++j) {
           const float4 s = d.segA[v0 + j];
           const float2 sb = d.segB[v0 + j];
           const float bx = s.x + s.z;
           int c0, c1, r0, r1;
-          seg_tiles(fminf(s.x, bx) + tpx, fmaxf(s.x, bx) + tpx, fminf(s.y, sb.x) + tpy,
-                    fmaxf(s.y, sb.x) + tpy, sl, T, tx0, ty0, ctw, cth, &c0, &c1, &r0, &r1);
+          seg_units<T>(fminf(s.x, bx) + tpx, fmaxf(s.x, bx) + tpx, fminf(s.y, sb.x) + tpy,
+                       fmaxf(s.y, sb.x) + tpy, sl, ux0, uy0, ctw, cuh, &c0, &c1, &r0, &r1);
           if (kc < c0 || kc > c1 || kr < r0 || kr > r1) continue;
           const float2 f = make_float2(s.z * sb.y, s.w * sb.y);
 #pragma unroll
-          for (int e = 0; e < PPL; ++e) {
-            const float d2 = seg_d2(dx[e], dy[e], s, f);
+          for (int e = 0; e < 2; ++e) {
+            const float d2 = seg_d2(dx, dy[e], s, f);
             if (d2 < best[e]) {
               best[e] = d2;
               bidx[e] = j;
@@ -362,67 +369,60 @@ __global__ void __launch_bounds__(NT, (T == 8 ? 1024 : 512) / NT) k_raster_chunk
           }
         }
       }
-      float2* sv = d.saved + (size_t)slot * NP;
+      float2* sv = d.saved + (size_t)(nti.x & (int)kSlotMask) * NP + (unsigned)nti.x / (1u << kSlotBits) * 64 + lane;
       bool live = false;
 #pragma unroll
-      for (int e = 0; e < PPL; ++e) {
-        const int local = lane + 32 * e;
-        const int X = tcx * T + local % T, Y = tcy * T + local / T;
-        const bool act = X < res && Y < res && dx[e] >= bb.x && dx[e] <= bb.z && dy[e] >= bb.y &&
-                         dy[e] <= bb.w;
-        float sd = -kFar;
-        if (act) {
-          int w = 0;
-          if (closed) {
-            const int q = Y - Y0;
-            const int2 row = s_row[q];
-            if (row.y <= kRowCross) {
-              float wf = (float)row.x;
-              for (int c = 0; c < row.y; ++c) {
-                const float2 cr = s_rx[q][c];
-                if (dx[e] < cr.x) wf += cr.y;
-              }
-              w = (int)wf;
-            } else {
-              w = winding_all(d, v0, ns, dx[e], dy[e]);
+      for (int e = 0; e < 2; ++e) {
+        // (outside the element's box the crossings cancel and the distance is beyond the margin; a
+        // pixel beyond the image is never read)
+        int w = 0;
+        if (closed) {
+          const int2 row = s_row[q + e * (32 / T)];
+          if (row.y <= kRowCross) {
+            float wf = (float)row.x;
+            for (int c = 0; c < row.y; ++c) {
+              const float2 cr = s_rx[q + e * (32 / T)][c];
+              if (dx < cr.x) wf += cr.y;
             }
-          }
-          if (best[e] < mrg2) {
-            const float dist = sqrtf(best[e]);
-            sd = closed ? (w != 0 ? dist : -dist) : hwpx - dist;
+            w = (int)wf;
           } else {
-            sd = (closed && w != 0) ? kFar : -kFar;
+            w = winding_all(d, v0, ns, dx, dy[e]);
           }
-          live |= fabsf(sd * inv_rho) < 1.0f || fabsf((sd + pad) * inv_rho) < 1.0f;
         }
-        sv[local] = make_float2(sd, __int_as_float(bidx[e]));
+        float sd = closed && w != 0 ? kFar : -kFar;
+        if (best[e] < mrg2) {
+          const float dist = sqrtf(best[e]);
+          sd = closed ? (w != 0 ? dist : -dist) : hwpx - dist;
+        }
+        live |= fabsf(sd * inv_rho) < 1.0f || fabsf((sd + pad) * inv_rho) < 1.0f;
+        sv[32 * e] = make_float2(sd, __int_as_float(bidx[e]));
       }
-      if (d.paths && closed && lane < T && s_row[kr * T + lane].y > kRowCross)
-        atomicAdd(&d.paths[0], 1ull);
+      if (d.paths && closed && lane < UH && s_row[kr * UH + lane].y > kRowCross) atomicAdd(&d.paths[0], 1ull);
       if (__any_sync(0xffffffffu, live)) {
         if (lane == 0) {
-          const int4 lr = make_int4(slot, g, tcx | (tcy << 16), p);
-          const int q = atomicAdd(&s_nlive, 1);
-          if (q < kLiveBatch) {
-            s_live[q] = lr;
+          const int4 lr = make_int4(nti.x, g, (tx0 + kc) | (ty0 + kr / UNITS) << 16, p);
+          const int l = atomicAdd(&s_nlive, 1);
+          if (l < kLiveBatch) {
+            s_live[l] = lr;
           } else {
             const int at = atomicAdd(&d.work[1], 1);
-            if (in_bounds(d, at < d.cap)) d.live_list[at] = lr;
+            if (in_bounds(d, at < d.cap * UNITS)) d.live_list[at] = lr;
           }
         }
       } else if (lane == 0 && d.deterministic) {
-        d.partial[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+        d.partial[(size_t)(nti.x & (int)kSlotMask) * UNITS + (unsigned)nti.x / (1u << kSlotBits)] =
+            make_float4(0.f, 0.f, 0.f, 0.f);
       }
       ni = __shfl_sync(0xffffffffu, nn, 0);
     }
     __syncthreads();
-    // the chunk's live pairs go out with one atomic
+    // the chunk's live units go out with one atomic
     if (tid < 32) {
       const int n = min(s_nlive, kLiveBatch);
       int at = 0;
       if (lane == 0 && n > 0) at = atomicAdd(&d.work[1], n);
       at = __shfl_sync(0xffffffffu, at, 0);
-      if (lane < n && in_bounds(d, at + lane < d.cap)) d.live_list[at + lane] = s_live[lane];
+      if (lane < n && in_bounds(d, at + lane < d.cap * UNITS)) d.live_list[at + lane] = s_live[lane];
     }
     __syncthreads();  // s_live, s_nlive and the shared lists are reused by the next chunk
     i = s_next[it & 1];
@@ -745,39 +745,113 @@ __global__ void __launch_bounds__(kCompWarps * 32) k_empty_loss(Dev d) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Adjoint, one (tile, element) pair per warp: dL/dIhat and dL/dA_tau per pixel, then the chain
-// dL/dc -> dc/dsd -> dsd/d(closest segment) -> d/d(tx, ty, theta, s) of Eq. 2, reduced over the
-// tile's pixels by a fixed shuffle tree and added to the element's gradient (or stored per pair).
+// Adjoint, one unit (64 pixels) of a (tile, element) pair per warp: dL/dIhat and dL/dA_tau per pixel,
+// then the chain dL/dc -> dc/dsd -> dsd/d(closest segment) -> d/d(tx, ty, theta, s) of Eq. 2, reduced
+// over the unit's pixels by a fixed shuffle tree and added to the element's gradient (or stored per unit).
+// The grid's first blocks, one per problem, assemble the loss instead: its partials are complete, and
+// the work (a read of 16 B per unit) fits beside the adjoint's round trips without a launch, a second
+// stream and the two joins that the end of an iteration waited for.
+// What the kernels before the predecessor wrote is read before the predecessor has completed: the work
+// list, the saved distances and, when the distribution term's adjoint is the predecessor, the images.
 // ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float warp_sum_f(float x) {
+  for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// Loss of one problem (Eq. 8): fixed-order float sums of the partials (eight strided accumulators per
+// thread, then a shuffle tree within and across warps).  Float throughout: FP64 arithmetic is slow on this
+// part and 1e-7 relative is ample for a sum of non-negative partials.
+__device__ void assemble_loss(const Dev& d, int p) {
+  constexpr int NT = kPairWarps * 32, ACC = 8;
+  __shared__ float s_red[4][kPairWarps];
+  const int units = d.tile * d.tile / 64;
+  const int t0 = d.prob_tile_base[p] * units, t1 = d.prob_tile_base[p + 1] * units;
+  float a[ACC] = {}, b[ACC] = {}, c[ACC] = {}, u[ACC] = {};
+  for (int t = t0 + (int)threadIdx.x; t < t1; t += NT * ACC)
+#pragma unroll
+    for (int k = 0; k < ACC; ++k) {
+      const float4 v = t + k * NT < t1 ? d.lossA[t + k * NT] : make_float4(0.f, 0.f, 0.f, 0.f);
+      a[k] += v.x;
+      b[k] += v.y;
+      c[k] += v.z;
+    }
+  if (d.L.gamma != 0.0f && d.L.n_dil > 0) {
+    const int u1 = d.prob_dtile_base[p + 1];
+    for (int t = d.prob_dtile_base[p] + (int)threadIdx.x; t < u1; t += NT * ACC)
+#pragma unroll
+      for (int k = 0; k < ACC; ++k) u[k] += t + k * NT < u1 ? d.lossU[t + k * NT] : 0.0f;
+  }
+  auto sum = [](float (&x)[ACC]) {
+    return warp_sum_f(((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7])));
+  };
+  const float sa = sum(a), sb = sum(b), sc = sum(c), su = sum(u);
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    s_red[0][w] = sa;
+    s_red[1][w] = sb;
+    s_red[2][w] = sc;
+    s_red[3][w] = su;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float r[4];
+    for (int k = 0; k < 4; ++k) r[k] = (s_red[k][0] + s_red[k][1]) + (s_red[k][2] + s_red[k][3]);
+    const float np = (float)d.prob_res[p] * (float)d.prob_res[p];
+    const float Lc = r[0] / np, Lo = r[1] / np, Ld = r[2] / np;
+    float* out = d.loss_terms + 5 * p;
+    out[0] = Lc;
+    out[1] = Lo;
+    out[2] = r[3];
+    out[3] = Ld;
+    out[4] = d.L.alpha * Lc + d.L.beta * Lo + d.L.gamma * r[3] + d.L.delta * Ld;
+  }
+}
+
 template <int T, bool FIT>  // FIT: also dL/d(vertex) for outline fitting (d.fit)
-__global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark) {
-  pdl_enter();
-  constexpr int NP = T * T, PPL = NP / 32;
-  if (*d.status & kStatusNoBins) return;
+__global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark, int early) {
+  constexpr int NP = T * T, UNITS = NP / 64, DY = 32 / T;
+  if ((int)blockIdx.x < d.n_probs) {
+    pdl_enter();
+    if (*d.status & kStatusNoBins) return;
+    assemble_loss(d, blockIdx.x);
+    if (mark) mark_step_if_last(d);
+    return;
+  }
   const float inv_rho = 1.0f / d.L.rho_px, pad = d.L.pad_px, tau = d.L.tau;
   const bool use_u = d.L.gamma != 0.0f;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int n_live = d.work[1];  // pairs without a gradient-carrying pixel are not listed
-  const int stride = (int)gridDim.x * kPairWarps;
-  int i = blockIdx.x * kPairWarps + wid;
+  const int stride = ((int)gridDim.x - d.n_probs) * kPairWarps;
+  int i = ((int)blockIdx.x - d.n_probs) * kPairWarps + wid;
+  if (*d.status & kStatusNoBins) {
+    pdl_enter();
+    return;
+  }
+  const int n_live = min(d.work[1], d.cap * UNITS);  // units without a gradient-carrying pixel are not listed
+  bool waited = false;
+  auto wait = [&]() {
+    if (!waited) pdl_enter();
+    waited = true;
+  };
   int4 rec = i < n_live ? d.live_list[i] : make_int4(0, 0, 0, 0);
   for (; i < n_live; i += stride) {
-    // the next pair's record is read while this one is worked on
+    // the next unit's record is read while this one is worked on
     const int4 rec_next = i + stride < n_live ? d.live_list[i + stride] : rec;
-    const int slot = rec.x, g = rec.y, txy = rec.z, p = rec.w;
+    const int slot = rec.x & (int)kSlotMask, unit = (int)((unsigned)rec.x >> kSlotBits), g = rec.y, txy = rec.z, p = rec.w;
     if (!in_bounds(d, slot >= 0 && slot < d.cap && g >= 0 && g < d.n_elems && p >= 0 && p < d.n_probs)) {
       rec = rec_next;
       continue;
     }
-    const int tx = txy & 0xffff, ty = txy >> 16, res = d.prob_res[p];
-    const long long pixbase = d.prob_pix_base[p];
+    const int res = d.prob_res[p];
     const float inv_np = 1.0f / ((float)res * (float)res);
     const int v0 = d.elem_voff[g];
     const bool closed = d.elem_closed[g] != 0;
     const float4 tp = d.tpx[g];
     const float4 qg = d.q[g];
     const float s_inv = 1.0f / qg.w;
-    const float2* sv = d.saved + (size_t)slot * NP;
+    // the lane's pixels: one column, rows Y and Y + DY
+    const int X = (txy & 0xffff) * T + lane % T, Y = (txy >> 16) * T + unit * (64 / T) + lane / T;
+    const long long pix0 = d.prob_pix_base[p] + (long long)Y * res + X;
+    const float2* sv = d.saved + (size_t)slot * NP + unit * 64 + lane;
     // outline fitting: d(pixel)/d(local vertex) = s res R(theta), applied transposed below
     float fc = 0.0f, fs = 0.0f, sres = 0.0f;
     int nv = 0;
@@ -787,37 +861,38 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark)
       nv = d.elem_voff[g + 1] - v0;
     }
     // every per-pixel input of the warp's pixels in one round of loads
-    float2 srec[PPL];
-    float ihat[PPL], pt_s[PPL], cov[PPL], gou[PPL];
+    float2 srec[2];
+    float ihat[2], pt_s[2], cov[2], gou[2];
+    if (!early) wait();
 #pragma unroll
-    for (int k = 0; k < PPL; ++k) {
-      const int local = lane + 32 * k;
-      const int X = tx * T + local % T, Y = ty * T + local / T;
+    for (int k = 0; k < 2; ++k) {
       srec[k] = make_float2(kFar, 0.0f);
       ihat[k] = pt_s[k] = cov[k] = gou[k] = 0.0f;
-      if (X < res && Y < res) {
-        const long long pix = pixbase + (long long)Y * res + X;
-        srec[k] = sv[local];
+      if (X < res && Y + k * DY < res) {
+        const long long pix = pix0 + k * DY * res;
+        srec[k] = sv[32 * k];
         ihat[k] = d.img_I[pix];
         pt_s[k] = d.img_Pt[pix];
         cov[k] = d.covc[pix];
-        if (use_u) gou[k] = d.gOu[pix];
       }
     }
-    // dL/dsd per pixel, then the closest segments of the pixels that carry a gradient
-    float gsd[PPL];
-    float4 sa[PPL];
+    wait();
+    if (use_u)
 #pragma unroll
-    for (int k = 0; k < PPL; ++k) {
-      const int local = lane + 32 * k;
-      const int X = tx * T + local % T, Y = ty * T + local / T;
+      for (int k = 0; k < 2; ++k)
+        if (X < res && Y + k * DY < res) gou[k] = d.gOu[pix0 + k * DY * res];
+    // dL/dsd per pixel, then the closest segments of the pixels that carry a gradient
+    float gsd[2];
+    float4 sa[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
       const float sd = srec[k].x;
       const float x = sd * inv_rho, xp = (sd + pad) * inv_rho;
       gsd[k] = 0.0f;
       if (fabsf(x) < 1.0f || fabsf(xp) < 1.0f) {  // never for the out-of-range pixels (sd = 1e30)
         const float pt = fabsf(pt_s[k]);  // negative: the pixel is on the rising side of the Eq. 6 kink
         const float W = cov[k] >= 0.5f ? d.L.w_in : d.L.w_out;
-        const float py = (float)Y + 0.5f;
+        const float py = (float)(Y + k * DY) + 0.5f;
         // O = 1 - Ihat: the uniform and force terms enter dL/dIhat with a minus sign
         const float gI = d.L.alpha * inv_np * 2.0f * W * (ihat[k] - (1.0f - cov[k])) - d.L.gamma * gou[k] -
                          d.L.delta * inv_np *
@@ -837,12 +912,10 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark)
     }
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
-    for (int k = 0; k < PPL; ++k) {
+    for (int k = 0; k < 2; ++k) {
       if (gsd[k] == 0.0f) continue;
-      const int local = lane + 32 * k;
-      const int X = tx * T + local % T, Y = ty * T + local / T;
       const float sd = srec[k].x;
-      const float dx = ((float)X + 0.5f - tp.x) - tp.z, dy = ((float)Y + 0.5f - tp.y) - tp.w;
+      const float dx = ((float)X + 0.5f - tp.x) - tp.z, dy = ((float)(Y + k * DY) + 0.5f - tp.y) - tp.w;
       const float ex = sa[k].z, ey = sa[k].w, ee = ex * ex + ey * ey;
       const float wx = dx - sa[k].x, wy = dy - sa[k].y;
       const float u = ee > 0.0f ? __saturatef((wx * ex + wy * ey) / ee) : 0.0f;
@@ -892,7 +965,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark)
     }
     if (lane == 0) {
       if (d.deterministic) {
-        d.partial[slot] = make_float4(a0, a1, a2, a3);
+        d.partial[(size_t)slot * UNITS + unit] = make_float4(a0, a1, a2, a3);
       } else {
         atomicAdd(&d.dq[g].x, a0);
         atomicAdd(&d.dq[g].y, a1);
@@ -902,6 +975,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark)
     }
     rec = rec_next;
   }
+  wait();
   if (mark) mark_step_if_last(d);
 }
 
@@ -1025,15 +1099,17 @@ cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int t
   }
 }
 
-cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int pair_grid, bool mark_step) {
-  const int mk = mark_step ? 1 : 0;
+cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step) {
+  // the loss blocks take the place of as many resident ones (at most half of them), so that none waits
+  const int grid = max(unit_grid - d.n_probs, (unit_grid + 1) / 2) + d.n_probs, mk = mark_step ? 1 : 0;
+  const int early = d.L.gamma != 0.0f && d.L.n_dil > 0 ? 1 : 0;  // the predecessor is the distribution adjoint
   switch (d.tile) {
     case 8:
-      return klaunch(d.pdl, d.fit ? k_raster_bwd<8, true> : k_raster_bwd<8, false>, pair_grid,
-                     kPairWarps * 32, 0, s, d, mk);
+      return klaunch(d.pdl, d.fit ? k_raster_bwd<8, true> : k_raster_bwd<8, false>, grid, kPairWarps * 32, 0, s, d, mk,
+                     early);
     case 16:
-      return klaunch(d.pdl, d.fit ? k_raster_bwd<16, true> : k_raster_bwd<16, false>, pair_grid,
-                     kPairWarps * 32, 0, s, d, mk);
+      return klaunch(d.pdl, d.fit ? k_raster_bwd<16, true> : k_raster_bwd<16, false>, grid, kPairWarps * 32, 0, s, d,
+                     mk, early);
     default: return cudaErrorInvalidValue;
   }
 }
