@@ -248,11 +248,13 @@ collage_status collage_get_bins(collage_t h, void* stream, int* d_tile, int* d_e
 #define COLLAGE_STAGE_DILATE 4    /* distribution term forward and backward */
 #define COLLAGE_STAGE_RASTER_BWD 5
 #define COLLAGE_STAGE_REDUCE 6    /* deterministic gradient reduction */
-#define COLLAGE_STAGE_LOSS 7      /* loss assembly */
+#define COLLAGE_STAGE_LOSS 7      /* (empty: the adjoint's first blocks assemble the loss) */
 #define COLLAGE_STAGE_ADAM 8      /* (empty: the Adam step is applied by the next transform) */
 collage_status collage_stage_times(collage_t h, void* stream, int n_iters, float* h_ms);
 
-/* A launch configuration of the iteration's kernels, as the autotuner chooses it. */
+/* A launch configuration of the iteration's kernels, as the autotuner chooses it.  Until one is chosen
+ * or set, emit_threads and chunk_px follow the work of each level (128 threads and 64 px where the
+ * elements fill the device). */
 typedef struct {
   int tile;              /* raster tile side, 8 or 16 */
   int emit_threads;      /* threads per block of the emission / signed-distance kernel: 128, 256 */

@@ -66,6 +66,9 @@ struct collage_s {
   // launch configuration (the autotuner's choice): persistent grids are these multiples of the SM
   // count x resident blocks per SM
   float fwd_mult = 1.0f, bwd_mult = 1.0f, comp_mult = 1.0f;
+  bool tuned = false;  // the configuration was searched or set by the caller; else the emission's block
+                       // and chunk sizes follow each level's work (choose_emission)
+  std::vector<int> lv_chunks;  // 64-px chunks of each level when it was last probed
   collage_tuning tuning{};
   // device memory
   Dev d{};
@@ -430,6 +433,7 @@ static collage_status build_levels(collage_t h) {
   const int T = h->d.tile, L = o.n_levels, P = h->P;
   const long long last = o.level_res[L - 1];
   h->lv.resize(L);
+  h->lv_chunks.resize(L, 0);
   size_t np = 0, nt = 0, nd = 0;
   for (int l = 0; l < L; ++l) {
     collage_s::LevelTab& t = h->lv[l];
@@ -509,16 +513,33 @@ static cudaError_t enqueue_level_switch(const Dev& d, cudaStream_t s) {
   return e;
 }
 
-// Pairs that binning the current params at the selected level produces: the transform with an
-// unbounded capacity allocates the slots, and their count is read back (synchronises the stream).
+// The emission's block and chunk sizes for a level of `chunks` 64-px chunks, where the caller chose
+// none.  A chunk is one block's work, and its phases are a chain: with fewer chunks than the device holds
+// blocks (eight of 128 threads per SM), smaller chunks or wider blocks put the idle warps to work; with
+// enough of them the extra staging only costs issue slots.  Measured per iteration (us; 128/64, 128/32,
+// 256/64, 256/32 threads/px): 120 chunks 55.9, 56.2, 54.3, 52.0; 200 chunks 64.2, 54.4, 56.4, 58.4; 400
+// chunks (of 320 segments) 88.4, 70.8, 77.0, 73.8; 500 chunks 74.8, 72.8, 67.1, 72.3; 1000 chunks 92.7,
+// 95.7, 90.7, 100.4; 5000 chunks 398.8, 444.4, 432.3, 547.8.
+static void choose_emission(collage_t h, int chunks) {
+  if (h->tuned) return;
+  const bool small = chunks <= 3 * h->sms;
+  h->d.chunk_tiles = (small ? kChunkPx / 2 : kChunkPx) / h->d.tile;
+  h->d.emit_threads = chunks <= h->sms || (!small && chunks <= 4 * h->sms) ? 256 : 128;
+}
+
+// Pairs that binning the current params at the selected level produces, and its 64-px chunks: the
+// transform with an unbounded capacity allocates the slots, and the counts are read back (synchronises
+// the stream).
 // A pending Adam step is applied on the way, as the next iteration would.
-static collage_status probe_pairs(collage_t h, cudaStream_t s, size_t* need) {
+static collage_status probe_pairs(collage_t h, cudaStream_t s, size_t* need, int* chunks) {
   Dev& d = h->d;
   Dev probe = d;
   probe.cap = 0x7fffffff;
   probe.list_cap = 0;  // no chunk is listed
+  probe.chunk_tiles = kChunkPx / d.tile;
   CK(h, launch_transform(probe, s, false, false));
   CK(h, cudaMemcpyAsync(h->h_ctl + 2, d.pair_need, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CK(h, cudaMemcpyAsync(h->h_ctl + 13, d.chunk_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   // the probe allocated slots and counted chunks without an emission: reset both, and the pending
   // Adam step it applied
   CK(h, cudaMemsetAsync(d.pair_need, 0, sizeof(int), s));
@@ -530,6 +551,7 @@ static collage_status probe_pairs(collage_t h, cudaStream_t s, size_t* need) {
   h->ctl_current = false;  // h_ctl[1] was not read
   if (h->h_ctl[0] & kStatusBadParam) return fail(h, COLLAGE_ERR_INVALID_ARG, "params are not finite or s <= 0");
   *need = (size_t)h->h_ctl[2];
+  *chunks = h->h_ctl[13] + h->h_ctl[14];
   return COLLAGE_OK;
 }
 
@@ -546,10 +568,11 @@ static collage_status setup_level(collage_t h, int level) {
   CK(h, enqueue_level_switch(d, s));
   // size the pair buffers from the current params
   size_t need = 0;
-  st = probe_pairs(h, s, &need);
+  st = probe_pairs(h, s, &need, &h->lv_chunks[level]);
   if (st) return st;
   st = ensure_pairs(h, with_slack(need));
   if (st) return st;
+  choose_emission(h, h->lv_chunks[level]);
   set_grids(h);
   h->level = level;
   return COLLAGE_OK;
@@ -1052,6 +1075,7 @@ static cudaError_t capture_schedule(collage_t h, int start, cudaStream_t s) {
   int target = 0;
   for (int l = start; l < o.n_levels && e == cudaSuccess; ++l) {
     if (apply_level(h, l) != COLLAGE_OK) return cudaErrorInvalidValue;  // tables exist: host only
+    choose_emission(h, h->lv_chunks[l]);
     set_grids(h);
     const Dev& d = h->d;
     target += o.level_iters[l];
@@ -1110,7 +1134,7 @@ static collage_status build_schedule(collage_t h, int start) {
   for (int l = start; l < h->opt.n_levels && !st; ++l) {
     st = apply_level(h, l);
     size_t n = 0;
-    if (!st) st = probe_pairs(h, s, &n);
+    if (!st) st = probe_pairs(h, s, &n, &h->lv_chunks[l]);
     need = std::max(need, n);
   }
   collage_status st2 = apply_level(h, cur);
@@ -1129,6 +1153,7 @@ static collage_status build_schedule(collage_t h, int start) {
   const cudaError_t e = capture_schedule(h, start, s);
   const cudaError_t e2 = cudaStreamEndCapture(s, &g);
   st = apply_level(h, cur);  // the current level's view again
+  choose_emission(h, h->lv_chunks[cur]);
   set_grids(h);
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -1190,6 +1215,7 @@ extern "C" collage_status collage_run_schedule(collage_t h, void* stream) {
   if (done == total && !(h->h_ctl[0] & (kStatusVoid | kStatusInternal))) {
     st = apply_level(h, L - 1);
     if (st) return st;
+    choose_emission(h, h->lv_chunks[L - 1]);
     set_grids(h);
     h->level = L - 1;
     return check_and_grow(h, s, &over);  // grows the pair buffers if the last level used > 3/4
@@ -1447,6 +1473,7 @@ struct L2Evict {
 // Applies a choice (tile change: new level tables and pair buffers).
 static collage_status apply_choice(collage_t h, const TuneChoice& c) {
   const bool retile = c.tile != h->d.tile;
+  h->tuned = true;
   h->d.tile = c.tile;
   h->opt.tile = c.tile;
   h->d.emit_threads = c.emit_threads;
@@ -1518,6 +1545,7 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
   cudaStream_t s = (cudaStream_t)stream;
   const TuneChoice before{h->d.tile, h->d.emit_threads, h->d.chunk_tiles * h->d.tile, h->fwd_mult,
                           h->bwd_mult, h->comp_mult};
+  const bool was_tuned = h->tuned;
   // the key: pixels of the level, elements, and the pair density at 8-px tiles (half-octaves)
   long long pix = 0;
   for (int p = 0; p < h->P; ++p) pix += (long long)h->res[p] * h->res[p];
@@ -1599,6 +1627,7 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
   }
   if (st) {  // leave the handle as it was
     apply_choice(h, before);
+    h->tuned = was_tuned;
     return st;
   }
   st = apply_choice(h, best);
@@ -1644,10 +1673,12 @@ extern "C" collage_status collage_set_tuning(collage_t h, void* stream, const co
   CK(h, cudaDeviceSynchronize());
   const TuneChoice before{h->d.tile, h->d.emit_threads, h->d.chunk_tiles * h->d.tile, h->fwd_mult,
                           h->bwd_mult, h->comp_mult};
+  const bool was_tuned = h->tuned;
   const TuneChoice want{c->tile, c->emit_threads, c->chunk_px, c->fwd_grid, c->bwd_grid, c->comp_grid};
   collage_status st = apply_choice(h, want);
   if (st) {
     apply_choice(h, before);
+    h->tuned = was_tuned;
     return st;
   }
   h->tuning = collage_tuning{};
