@@ -171,27 +171,57 @@ struct IIGeom {
   static_assert(P % 2 == 1, "odd row stride");
 };
 
+// A dilation tile's place.
+struct DilTile {
+  int dt, x0, y0, res;
+  bool own;  // it has container coverage of its own
+  long long pb;
+};
+__device__ __forceinline__ DilTile dil_place(const Dev& d, int which, int li) {
+  DilTile t;
+  t.dt = min(max(dil_tile(d, which, li), 0), d.total_dtiles - 1);
+  t.own = (dil_flags(d, t.dt) & kFlagOwn) != 0;
+  const int p = find_prob_d(d.prob_dtile_base, d.n_probs, t.dt);
+  t.res = d.prob_res[p];
+  const int nd = (t.res + kDT - 1) / kDT, ld = t.dt - d.prob_dtile_base[p];
+  t.x0 = (ld % nd) * kDT;
+  t.y0 = (ld / nd) * kDT;
+  t.pb = d.prob_pix_base[p];
+  return t;
+}
+
 template <int K>
 __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
-  pdl_enter();
   constexpr int S = DilGeom<K>::S, P = IIGeom<K>::P, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
   constexpr float inv_q = 1.0f / (float)(1u << Q);
   extern __shared__ uint32_t sm[];
   __shared__ float s_red[kDThreads / 32];
-  if (*d.status & kStatusNoBins) return;
   uint32_t* II = sm;
   // the tiles with container coverage; on the others M_C (1 - O) = 0, dL_u/dO = 0 and the loss
-  // partial is 0, as written once per level
+  // partial is 0, as written once per level.  The lists and the coverage are the level's: the first
+  // tile's place and coverage are read before the composite has completed.
   const int n_own = dil_count(d, 0);
+  DilTile t{};
+  if ((int)blockIdx.x < n_own) t = dil_place(d, 0, blockIdx.x);
+  // the thread's output item: column c, rows r0..r0 + kVRows - 1
+  const int c = threadIdx.x % kDT, r0 = (threadIdx.x / kDT) * kVRows;
+  float Iv[kVRows], Mv[kVRows];
+  auto coverage = [&]() {  // from a clamped address, used only inside the image
+#pragma unroll
+    for (int i = 0; i < kVRows; ++i)
+      Mv[i] = d.covc[t.pb + min(t.y0 + r0 + i, t.res - 1) * t.res + min(t.x0 + c, t.res - 1)];
+  };
+  if ((int)blockIdx.x < n_own) coverage();
+  pdl_enter();
+  if (*d.status & kStatusNoBins) return;
   for (int li = blockIdx.x; li < n_own; li += gridDim.x) {
-    const int dt = dil_tile(d, 0, li);
-    if (!in_bounds(d, dt >= 0 && dt < d.total_dtiles)) continue;
-    const int p = find_prob_d(d.prob_dtile_base, d.n_probs, dt);
-    const int res = d.prob_res[p], nd = (res + kDT - 1) / kDT, ld = dt - d.prob_dtile_base[p];
-    const int x0 = (ld % nd) * kDT, y0 = (ld / nd) * kDT;
-    const long long pb = d.prob_pix_base[p];
+    if (li != (int)blockIdx.x) {
+      t = dil_place(d, 0, li);
+      coverage();
+    }
+    const int x0 = t.x0, y0 = t.y0, res = t.res, dt = t.dt;
+    const long long pb = t.pb;
     const float* Ib = d.img_I + pb;
-    const float* Mb = d.covc + pb;
     __syncthreads();
     {  // thread (column, first row): no division per element, 32-bit offsets from the problem's base
       constexpr int CW = DilGeom<K>::CW, RP = kDThreads / CW;
@@ -207,17 +237,10 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
       if (threadIdx.x < P) II[threadIdx.x] = 0u;              // row 0
       if (threadIdx.x < S) II[(threadIdx.x + 1) * P] = 0u;    // column 0
     }
-    // the thread's output item (column c, rows r0..r0 + kVRows - 1): its per-pixel inputs are
-    // read now (from a clamped address, used only inside the image), in flight during the scans
-    const int c = threadIdx.x % kDT, r0 = (threadIdx.x / kDT) * kVRows;
-    const int X = x0 + c, Xc = min(X, res - 1);
-    float Iv[kVRows], Mv[kVRows];
+    // the occupancy of the thread's pixels, in flight during the scans
+    const int X = x0 + c;
 #pragma unroll
-    for (int i = 0; i < kVRows; ++i) {
-      const int o = min(y0 + r0 + i, res - 1) * res + Xc;
-      Iv[i] = Ib[o];
-      Mv[i] = Mb[o];
-    }
+    for (int i = 0; i < kVRows; ++i) Iv[i] = Ib[min(y0 + r0 + i, res - 1) * res + min(X, res - 1)];
     __syncthreads();
     if (threadIdx.x < S) {  // rows: lanes take rows (odd stride, distinct banks)
       uint32_t* row = II + (threadIdx.x + 1) * P + 1;
@@ -283,24 +306,24 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
 
 template <int K>
 __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
-  pdl_enter();
   constexpr int S = DilGeom<K>::S, SP = DilGeom<K>::SP, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
   constexpr float inv_q = 1.0f / (float)(1u << Q);
   extern __shared__ uint32_t sm[];
-  if (*d.status & kStatusNoBins) return;
   uint32_t* sM = sm;
   uint32_t* H = sM + S * SP;
-  // the tiles with container coverage within the halo (G = 0 over the others and their halos)
+  // the tiles with container coverage within the halo (G = 0 over the others and their halos); the
+  // first one's place is read before the forward pass has completed
   const int n_halo = dil_count(d, 1);
+  DilTile t{};
+  if ((int)blockIdx.x < n_halo) t = dil_place(d, 1, blockIdx.x);
+  pdl_enter();
+  if (*d.status & kStatusNoBins) return;
   for (int li = blockIdx.x; li < n_halo; li += gridDim.x) {
-    const int dt = dil_tile(d, 1, li);
-    if (!in_bounds(d, dt >= 0 && dt < d.total_dtiles)) continue;
+    if (li != (int)blockIdx.x) t = dil_place(d, 1, li);
+    const int x0 = t.x0, y0 = t.y0, res = t.res;
+    const long long pb = t.pb;
     // a tile without coverage of its own was not written by the forward pass: store, not add
-    const bool own = (dil_flags(d, dt) & kFlagOwn) != 0;
-    const int p = find_prob_d(d.prob_dtile_base, d.n_probs, dt);
-    const int res = d.prob_res[p], nd = (res + kDT - 1) / kDT, ld = dt - d.prob_dtile_base[p];
-    const int x0 = (ld % nd) * kDT, y0 = (ld / nd) * kDT;
-    const long long pb = d.prob_pix_base[p];
+    const bool own = t.own;
     __syncthreads();
     {  // thread (column, first row): no division per element, 32-bit offsets from the problem's base
       constexpr int CW = DilGeom<K>::CW, RP = kDThreads / CW;

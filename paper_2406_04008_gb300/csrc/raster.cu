@@ -876,27 +876,38 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark,
         cov[k] = d.covc[pix];
       }
     }
+    // the closest segments of the pixels that may carry a gradient (never the out-of-range ones, whose
+    // sd is 1e30), in flight before the weights are formed
+    bool act[2];
+    float4 sa[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float sd = srec[k].x;
+      act[k] = fabsf(sd * inv_rho) < 1.0f || fabsf((sd + pad) * inv_rho) < 1.0f;
+      if (act[k] && !in_bounds(d, (unsigned)__float_as_int(srec[k].y) < (unsigned)(d.elem_voff[g + 1] - v0)))
+        act[k] = false;
+      if (act[k]) sa[k] = d.segA[v0 + __float_as_int(srec[k].y)];
+    }
     wait();
     if (use_u)
 #pragma unroll
       for (int k = 0; k < 2; ++k)
-        if (X < res && Y + k * DY < res) gou[k] = d.gOu[pix0 + k * DY * res];
-    // dL/dsd per pixel, then the closest segments of the pixels that carry a gradient
+        if (act[k]) gou[k] = d.gOu[pix0 + k * DY * res];
+    // dL/dsd per pixel
     float gsd[2];
-    float4 sa[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const float sd = srec[k].x;
       const float x = sd * inv_rho, xp = (sd + pad) * inv_rho;
       gsd[k] = 0.0f;
-      if (fabsf(x) < 1.0f || fabsf(xp) < 1.0f) {  // never for the out-of-range pixels (sd = 1e30)
+      if (act[k]) {
         const float pt = fabsf(pt_s[k]);  // negative: the pixel is on the rising side of the Eq. 6 kink
         const float W = cov[k] >= 0.5f ? d.L.w_in : d.L.w_out;
         const float py = (float)(Y + k * DY) + 0.5f;
         // O = 1 - Ihat: the uniform and force terms enter dL/dIhat with a minus sign
-        const float gI = d.L.alpha * inv_np * 2.0f * W * (ihat[k] - (1.0f - cov[k])) - d.L.gamma * gou[k] -
-                         d.L.delta * inv_np *
-                             force_potential(d.L, ((float)X + 0.5f) / (float)res, py / (float)res);
+        float gI = d.L.alpha * inv_np * 2.0f * W * (ihat[k] - (1.0f - cov[k])) - d.L.gamma * gou[k];
+        if (d.L.delta != 0.0f)
+          gI -= d.L.delta * inv_np * force_potential(d.L, ((float)X + 0.5f) / (float)res, py / (float)res);
         const float gA = pt_s[k] < 0.0f ? d.L.beta * inv_np : 0.0f;
         const float omc = Sfun(-x), cp = Sfun(xp);
         // dIhat/dc_i = -prod_{j != i}(1 - c_j) = -Ihat / (1 - c_i)   (0 when another c_j = 1)
@@ -905,10 +916,6 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark,
         const float gcp = gA * tau * pt / (1.0f - tau * cp);
         gsd[k] = (gc * dSfun(x) + gcp * dSfun(xp)) * inv_rho;
       }
-      if (gsd[k] != 0.0f && !in_bounds(d, (unsigned)__float_as_int(srec[k].y) <
-                                               (unsigned)(d.elem_voff[g + 1] - v0)))
-        gsd[k] = 0.0f;
-      if (gsd[k] != 0.0f) sa[k] = d.segA[v0 + __float_as_int(srec[k].y)];
     }
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
@@ -956,22 +963,15 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark,
         atomicAdd(&d.dv[jb].y, ly * u);
       }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-      a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-      a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-      a3 += __shfl_xor_sync(0xffffffffu, a3, o);
-    }
-    if (lane == 0) {
-      if (d.deterministic) {
-        d.partial[(size_t)slot * UNITS + unit] = make_float4(a0, a1, a2, a3);
-      } else {
-        atomicAdd(&d.dq[g].x, a0);
-        atomicAdd(&d.dq[g].y, a1);
-        atomicAdd(&d.dq[g].z, a2);
-        atomicAdd(&d.dq[g].w, a3);
-      }
+    // the four sums in one shuffle tree: after two steps lane l carries sum l / 8
+    const bool h = lane & 16, q8 = lane & 8;
+    const float b0 = (h ? a2 : a0) + __shfl_xor_sync(0xffffffffu, h ? a0 : a2, 16);
+    const float b1 = (h ? a3 : a1) + __shfl_xor_sync(0xffffffffu, h ? a1 : a3, 16);
+    float v = (q8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, q8 ? b0 : b1, 8);
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0) {
+      if (d.deterministic) reinterpret_cast<float*>(d.partial + (size_t)slot * UNITS + unit)[lane >> 3] = v;
+      else atomicAdd(reinterpret_cast<float*>(d.dq + g) + (lane >> 3), v);
     }
     rec = rec_next;
   }
