@@ -416,7 +416,6 @@ static collage_status ensure_level_bufs(collage_t h, size_t np, size_t nt, size_
   CK(h, dmalloc(h->level_bufs, d.lossA, nu));
   CK(h, dmalloc(h->level_bufs, d.loss0, nu));
   CK(h, dmalloc(h->level_bufs, d.lossU, nd));
-  CK(h, dmalloc(h->level_bufs, d.dtile_flags, nd));
   CK(h, dmalloc(h->level_bufs, d.dtile_list, 2 * nd));
   CK(h, dmalloc(h->level_bufs, d.dtile_n, 2));
   h->pix_cap = np;

@@ -133,9 +133,9 @@ struct Dev {
                                 //   tile: (sum W(I-Ic)^2, sum relu(A-tau), sum O(1-y), 0)
   float* loss0;                 // per unit: the first of these where nothing covers it (level constant)
   float* lossU;                 // [total_dtiles] weighted uniform-loss partial
-  uint8_t* dtile_flags;         // [total_dtiles] container coverage on the tile / its halo (or null)
-  int* dtile_list;              // [2 total_dtiles] the tiles with kFlagOwn from 0, with kFlagHalo
-                                //   from total_dtiles, in no particular order (or null: all tiles)
+  int4* dtile_list;             // [2 total_dtiles] the places of the dilation tiles with container coverage
+                                //   from 0, with coverage within the halo from total_dtiles, in no
+                                //   particular order (or null: all tiles)
   int* dtile_n;                 // [2] lengths of the two lists
   float4* dq;                   // [n] gradient
   float4* partial;              // [cap * units per tile] deterministic gradient partials, by slot
