@@ -13,14 +13,25 @@ import torch
 from . import _lib as L
 
 
+# (addresses go to the ABI as plain integers: its argument types convert them)
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dptr(t: torch.Tensor):
     if not t.is_cuda or not t.is_contiguous() or t.dtype != torch.float32:
         raise ValueError("expected a contiguous float32 CUDA tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _empty(*shape):
+    return torch.empty(shape, device="cuda", dtype=torch.float32)
+
+
+def _flat(t: torch.Tensor):
+    """The values as a contiguous float32 tensor, itself where it is one."""
+    t = t.detach()
+    return t if t.dtype == torch.float32 and t.is_contiguous() else t.contiguous().float()
 
 
 class Collage:
@@ -66,16 +77,14 @@ class Collage:
     # hot path -----------------------------------------------------------------------------------
     def render(self):
         n = self.info()["total_pixels"]
-        bw = torch.empty(n, device="cuda", dtype=torch.float32)
-        tau = torch.empty(n, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_render(self.h, _stream(), _dptr(bw), _dptr(tau)))
+        bw, tau = _empty(n), _empty(n)
+        self._check(self.lib.collage_render(self.h, _stream(), bw.data_ptr(), tau.data_ptr()))
         return bw, tau
 
     def loss_backward(self):
-        terms = torch.empty(self.n_probs * 5, device="cuda", dtype=torch.float32)
-        grad = torch.empty(self.n_elems * 4, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_loss_backward(self.h, _stream(), _dptr(terms), _dptr(grad)))
-        return terms.view(self.n_probs, 5), grad.view(self.n_elems, 4)
+        terms, grad = _empty(self.n_probs, 5), _empty(self.n_elems, 4)
+        self._check(self.lib.collage_loss_backward(self.h, _stream(), terms.data_ptr(), grad.data_ptr()))
+        return terms, grad
 
     def step(self, n_iters: int = 1):
         self._check(self.lib.collage_step(self.h, _stream(), n_iters))
@@ -96,18 +105,18 @@ class Collage:
         return pout, lout
 
     def loss(self):
-        t = torch.empty(self.n_probs * 5, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_get_loss(self.h, _stream(), _dptr(t)))
-        return t.view(self.n_probs, 5)
+        t = _empty(self.n_probs, 5)
+        self._check(self.lib.collage_get_loss(self.h, _stream(), t.data_ptr()))
+        return t
 
     # params / state -----------------------------------------------------------------------------
     def get_params(self) -> torch.Tensor:
-        t = torch.empty(self.n_elems * 4, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_get_params(self.h, _stream(), _dptr(t)))
-        return t.view(self.n_elems, 4)
+        t = _empty(self.n_elems, 4)
+        self._check(self.lib.collage_get_params(self.h, _stream(), t.data_ptr()))
+        return t
 
     def set_params(self, params: torch.Tensor):
-        p = params.detach().reshape(-1).contiguous().float()
+        p = _flat(params)
         self._check(self.lib.collage_set_params(self.h, _stream(), _dptr(p)))
 
     # skeleton-based initialisation ------------------------------------------------------------
@@ -126,20 +135,20 @@ class Collage:
 
     # outline points (fit_controls) ------------------------------------------------------------
     def get_controls(self) -> torch.Tensor:
-        t = torch.empty(self.n_pts * 2, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_get_controls(self.h, _stream(), _dptr(t)))
-        return t.view(self.n_pts, 2)
+        t = _empty(self.n_pts, 2)
+        self._check(self.lib.collage_get_controls(self.h, _stream(), t.data_ptr()))
+        return t
 
     def set_controls(self, pts: torch.Tensor):
-        p = pts.detach().reshape(-1).contiguous().float()
+        p = _flat(pts)
         if p.numel() != 2 * self.n_pts:
             raise ValueError(f"expected {2 * self.n_pts} floats")
         self._check(self.lib.collage_set_controls(self.h, _stream(), _dptr(p)))
 
     def control_grad(self) -> torch.Tensor:
-        t = torch.empty(self.n_pts * 2, device="cuda", dtype=torch.float32)
-        self._check(self.lib.collage_get_control_grad(self.h, _stream(), _dptr(t)))
-        return t.view(self.n_pts, 2)
+        t = _empty(self.n_pts, 2)
+        self._check(self.lib.collage_get_control_grad(self.h, _stream(), t.data_ptr()))
+        return t
 
     def get_state(self):
         t = torch.empty(self.n_elems * 12, device="cuda", dtype=torch.float32)
@@ -200,8 +209,8 @@ class CollageLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, params: torch.Tensor, col: Collage):
         col.set_params(params)
-        terms, grad = col.loss_backward()
-        ctx.save_for_backward(grad.clone())
+        terms, grad = col.loss_backward()  # fresh tensors: nothing else holds them
+        ctx.save_for_backward(grad)
         ctx.shape = params.shape
         return terms[:, 4].sum()
 

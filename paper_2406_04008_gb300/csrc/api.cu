@@ -91,6 +91,8 @@ struct collage_s {
   cudaGraphExec_t graph = nullptr;  // one iteration at the current level
   cudaGraphExec_t host_graph = nullptr;  // one iteration taking its params from h_in, then the
                                          // gathering kernel writing h_stage (collage_step_host)
+  cudaGraphExec_t grad_graph = nullptr;  // one loss + gradient pass and the read of the control words
+  int grad_calls = 0;                    // such passes since the level was set up or a buffer moved
   cudaGraphExec_t sched = nullptr;  // the schedule from level sched_start to the last
   int sched_start = -1;
   // quality-metric scratch (allocated by collage_metrics)
@@ -160,6 +162,9 @@ void drop_iter_graph(collage_t h) {
   h->graph = nullptr;
   if (h->host_graph) cudaGraphExecDestroy(h->host_graph);
   h->host_graph = nullptr;
+  if (h->grad_graph) cudaGraphExecDestroy(h->grad_graph);
+  h->grad_graph = nullptr;
+  h->grad_calls = 0;
 }
 
 void drop_graph(collage_t h) {
@@ -174,6 +179,7 @@ void drop_graph(collage_t h) {
 collage_s::~collage_s() {
   if (graph) cudaGraphExecDestroy(graph);
   if (host_graph) cudaGraphExecDestroy(host_graph);
+  if (grad_graph) cudaGraphExecDestroy(grad_graph);
   if (h_in) cudaFreeHost(h_in);
   if (sched) cudaGraphExecDestroy(sched);
   if (cap_stream) cudaStreamDestroy(cap_stream);
@@ -681,11 +687,32 @@ static collage_status ensure_host_graph(collage_t h) {
   return COLLAGE_OK;
 }
 
+// The loss + gradient pass as a graph that also reads the control words.
+static collage_status ensure_grad_graph(collage_t h) {
+  if (h->grad_graph) return COLLAGE_OK;
+  cudaGraph_t g = nullptr;
+  CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = enqueue_iter(h, h->cap_stream, kLossBwd, nullptr, nullptr);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->h_ctl, h->ctl, kCtlWords * sizeof(int), cudaMemcpyDeviceToHost, h->cap_stream);
+  cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return cuda_fail(h, e, "capture");
+  }
+  CK(h, e2);
+  e = cudaGraphInstantiate(&h->grad_graph, g, 0);
+  cudaGraphDestroy(g);
+  CK(h, e);
+  return COLLAGE_OK;
+}
+
 // After a batch of work: check the latched status; grow the pair buffers when the last binning
-// used more than 3/4 of them.  Returns OVERFLOW if the batch overflowed (caller re-runs).
-static collage_status check_and_grow(collage_t h, cudaStream_t s, bool* overflowed) {
+// used more than 3/4 of them.  Returns OVERFLOW if the batch overflowed (caller re-runs).  `read`: the
+// control words have been read already.
+static collage_status check_and_grow(collage_t h, cudaStream_t s, bool* overflowed, bool read = false) {
   *overflowed = false;
-  collage_status st = read_ctl(h, s);
+  collage_status st = read ? COLLAGE_OK : read_ctl(h, s);
   if (st) return st;
   const int status = h->h_ctl[0];
   const size_t need = (size_t)h->h_ctl[2];
@@ -732,9 +759,20 @@ static collage_status check_and_grow(collage_t h, cudaStream_t s, bool* overflow
 
 static collage_status run_checked(collage_t h, cudaStream_t s, int mode, float* out_bw, float* out_tau) {
   for (int attempt = 0; attempt < 4; ++attempt) {
-    CK(h, enqueue_iter(h, s, mode, out_bw, out_tau));
+    // a program that steps by itself calls this at every iteration: from its third pass on, one graph
+    // launch instead of a launch per kernel and a copy (capturing costs about four eager passes)
+    const bool graph = mode == kLossBwd && h->opt.use_graphs && ++h->grad_calls > 2;
+    if (graph) {
+      collage_status st = ensure_grad_graph(h);
+      if (st) return st;
+      CK(h, cudaGraphLaunch(h->grad_graph, s));
+      CK(h, cudaStreamSynchronize(s));
+      h->ctl_current = true;
+    } else {
+      CK(h, enqueue_iter(h, s, mode, out_bw, out_tau));
+    }
     bool over = false;
-    collage_status st = check_and_grow(h, s, &over);
+    collage_status st = check_and_grow(h, s, &over, graph);
     if (st) return st;
     if (!over) return COLLAGE_OK;
   }
@@ -1015,9 +1053,7 @@ extern "C" collage_status collage_loss_backward(collage_t h, void* stream, float
   cudaStream_t s = (cudaStream_t)stream;
   collage_status st = run_checked(h, s, kLossBwd, nullptr, nullptr);
   if (st) return st;
-  if (d_loss_terms)
-    CK(h, cudaMemcpyAsync(d_loss_terms, h->d.loss_terms, sizeof(float) * 5 * h->P, cudaMemcpyDeviceToDevice, s));
-  if (d_dparams) CK(h, launch_copy_grad(h->d, s, d_dparams));
+  if (d_loss_terms || d_dparams) CK(h, launch_copy_out(h->d, s, d_loss_terms, d_dparams));
   return COLLAGE_OK;
 }
 
@@ -1301,6 +1337,10 @@ extern "C" collage_status collage_get_loss(collage_t h, void* stream, float* d_l
 
 extern "C" collage_status collage_get_params(collage_t h, void* stream, float* d_params) {
   if (!h || !d_params) return fail(h, COLLAGE_ERR_INVALID_ARG, "NULL argument");
+  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0) {  // one kernel for the step and the copy
+    CK(h, launch_adam_flush(h->d, (cudaStream_t)stream, nullptr, nullptr, d_params));
+    return COLLAGE_OK;
+  }
   CK(h, launch_adam_flush(h->d, (cudaStream_t)stream));
   CK(h, cudaMemcpyAsync(d_params, h->d.q, sizeof(float4) * h->N, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
   return COLLAGE_OK;
@@ -1308,7 +1348,12 @@ extern "C" collage_status collage_get_params(collage_t h, void* stream, float* d
 
 extern "C" collage_status collage_set_params(collage_t h, void* stream, const float* d_params) {
   if (!h || !d_params) return fail(h, COLLAGE_ERR_INVALID_ARG, "NULL argument");
-  CK(h, launch_adam_flush(h->d, (cudaStream_t)stream));  // the step belongs to the old params
+  // (a pending step belongs to the old params)
+  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0) {
+    CK(h, launch_adam_flush(h->d, (cudaStream_t)stream, nullptr, d_params));
+    return COLLAGE_OK;
+  }
+  CK(h, launch_adam_flush(h->d, (cudaStream_t)stream));
   CK(h, cudaMemcpyAsync(h->d.q, d_params, sizeof(float4) * h->N, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
   return COLLAGE_OK;
 }

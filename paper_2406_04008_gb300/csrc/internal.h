@@ -292,8 +292,11 @@ cudaError_t launch_dtile_flags(const Dev& d, cudaStream_t s);  // once per level
 // (step mode)
 cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step);
 cudaError_t launch_grad_reduce(const Dev& d, cudaStream_t s, bool mark_step);
-// applies a pending Adam step to all elements and clears the flag (before params are read)
-cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out = nullptr);
+// applies a pending Adam step to all elements and clears the flag (before params are read); then, where
+// given, replaces the params by q_in, copies them to q_out (both 16-byte aligned, [4n]) and gathers them
+// with the loss terms and the control words into out
+cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out = nullptr, const float* q_in = nullptr,
+                              float* q_out = nullptr);
 // outline fitting, one block per element: mode 0 maps dv to dctrl (and clears dv); mode 1 also
 // takes an Adam step on ctrl at step *d.step and flattens again (vertices and bin radii); mode 2
 // only flattens
@@ -306,7 +309,7 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
 // condition (1 while fewer than `target` iterations of the run are done and nothing latched)
 cudaError_t launch_sched_begin(const Dev& d, cudaStream_t s);
 cudaError_t launch_sched_cond(const Dev& d, cudaStream_t s, cudaGraphConditionalHandle cond, int target);
-cudaError_t launch_copy_grad(const Dev& d, cudaStream_t s, float* out);
+cudaError_t launch_copy_out(const Dev& d, cudaStream_t s, float* terms, float* grad);
 // Resident blocks per SM of the raster kernels, the pairs one adjoint block and the tiles one
 // composite block take at once (the forward distance kernel takes one pair per block).
 struct RasterOcc {

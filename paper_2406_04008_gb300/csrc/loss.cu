@@ -434,12 +434,14 @@ __global__ void __launch_bounds__(kReduceWarps * 32) k_grad_reduce(Dev d, int ma
 // Applies a pending Adam step to every element (see adam_update); the last block to finish clears
 // the flag, once every block has read it.  With `out`, also gathers the params, the loss terms and
 // the control words (status, step, pair count, 0) into one buffer, [4n | 5 n_probs | 4], so that one
-// copy brings all of them to the host.
-__global__ void k_adam_flush(Dev d, float* out) {
+// copy brings all of them to the host.  With `q_in`, the params are then replaced; with `q_out`, copied out.
+__global__ void k_adam_flush(Dev d, float* out, const float4* q_in, float4* q_out) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const bool pend = *d.pending != 0;
   if (g < d.n_elems) {
     if (pend && !d.fit) adam_update(d, g, *d.step, d.dq[g]);
+    if (q_in) d.q[g] = q_in[g];
+    if (q_out) q_out[g] = d.q[g];
     if (out) reinterpret_cast<float4*>(out)[g] = d.q[g];
   }
   if (out && blockIdx.x == 0) {
@@ -528,13 +530,24 @@ cudaError_t launch_grad_reduce(const Dev& d, cudaStream_t s, bool mark_step) {
                  s, d, mark_step ? 1 : 0);
 }
 
-cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out) {
-  k_adam_flush<<<(d.n_elems + 255) / 256, 256, 0, s>>>(d, out);
+cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out, const float* q_in, float* q_out) {
+  k_adam_flush<<<(d.n_elems + 255) / 256, 256, 0, s>>>(d, out, reinterpret_cast<const float4*>(q_in),
+                                                       reinterpret_cast<float4*>(q_out));
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy_grad(const Dev& d, cudaStream_t s, float* out) {
-  return cudaMemcpyAsync(out, d.dq, sizeof(float4) * (size_t)d.n_elems, cudaMemcpyDeviceToDevice, s);
+// The loss terms and the gradient of the last pass into the caller's buffers (either may be null), one
+// launch for both.
+__global__ void k_copy_out(Dev d, float* terms, float* grad) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (grad && i < 4 * (size_t)d.n_elems) grad[i] = reinterpret_cast<const float*>(d.dq)[i];
+  if (terms && i < 5 * (size_t)d.n_probs) terms[i] = d.loss_terms[i];
+}
+
+cudaError_t launch_copy_out(const Dev& d, cudaStream_t s, float* terms, float* grad) {
+  const size_t n = 5 * (size_t)max(d.n_elems, d.n_probs);  // covers both
+  k_copy_out<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, terms, grad);
+  return cudaGetLastError();
 }
 
 }  // namespace collage
