@@ -87,6 +87,11 @@ __device__ __forceinline__ void hsum_one(const Src& src, uint32_t* H, int it) {
   }
 }
 
+// (The adjoint's summand is zero wherever a kernel's box holds a pixel's worth of occupancy, which for the
+// wide kernels is almost everywhere between crowded elements: `act` has a bit per kernel that some staged
+// pixel feeds, and the sums of the others are zero: 5000 elements at 2048^2 70 -> 59 us for the two passes
+// together with the staging of interior tiles without bounds tests, 64 collages 317 -> 301.)
+//
 // Vertical pass fused with the per-pixel output: a thread forms the box sums of all K kernels at
 // kVRows consecutive output rows of one column (a running window per kernel), then uses them
 // directly, so no per-kernel result image is kept in shared memory.
@@ -96,39 +101,44 @@ constexpr int kVItems = kDT * (kDT / kVRows);
 static_assert(kVItems == kDThreads, "one output item per thread");
 
 template <int K, int k = 0>
-__device__ __forceinline__ void vsums_col(const uint32_t* H, int c, int r0, uint32_t (&B)[K][kVRows]) {
+__device__ __forceinline__ void vsums_col(const uint32_t* H, int c, int r0, unsigned act, uint32_t (&B)[K][kVRows]) {
   if constexpr (k < K) {
     constexpr int r = dil_r(k);
-    const uint32_t* col = H + hbase(k) * kHP + c;
-    uint32_t acc = 0u;
 #pragma unroll
-    for (int j = 0; j <= 2 * r; ++j) acc += col[(r0 + j) * kHP];
-    B[k][0] = acc;
+    for (int i = 0; i < kVRows; ++i) B[k][i] = 0u;
+    if (act >> k & 1u) {
+      const uint32_t* col = H + hbase(k) * kHP + c;
+      uint32_t acc = 0u;
 #pragma unroll
-    for (int i = 1; i < kVRows; ++i) {
-      acc += col[(r0 + i + 2 * r) * kHP] - col[(r0 + i - 1) * kHP];
-      B[k][i] = acc;
+      for (int j = 0; j <= 2 * r; ++j) acc += col[(r0 + j) * kHP];
+      B[k][0] = acc;
+#pragma unroll
+      for (int i = 1; i < kVRows; ++i) {
+        acc += col[(r0 + i + 2 * r) * kHP] - col[(r0 + i - 1) * kHP];
+        B[k][i] = acc;
+      }
     }
-    vsums_col<K, k + 1>(H, c, r0, B);
+    vsums_col<K, k + 1>(H, c, r0, act, B);
   }
 }
 
-// Item `it` of the flattened list of all kernels' horizontal items: every thread of the block
-// gets work, whatever the kernel sizes.
+// Item `it` of the flattened list of the active kernels' horizontal items: every thread of the block
+// gets work, whatever the kernel sizes.  Returns false beyond the list.
 template <int K, int k = 0, class Src>
-__device__ __forceinline__ void hsum_item(const Src& src, uint32_t* H, int it) {
+__device__ __forceinline__ bool hsum_item(const Src& src, uint32_t* H, int it, unsigned act) {
   if constexpr (k < K) {
     constexpr int items_k = hrows(k) * kNSeg;
-    if (it < items_k) hsum_one<K, k>(src, H, it);
-    else hsum_item<K, k + 1>(src, H, it - items_k);
+    if (act >> k & 1u) {
+      if (it < items_k) {
+        hsum_one<K, k>(src, H, it);
+        return true;
+      }
+      it -= items_k;
+    }
+    return hsum_item<K, k + 1>(src, H, it, act);
   }
+  return false;
 }
-
-struct OccSrc {  // occupancy O of the staged region, the same for every kernel
-  const uint32_t* sO;
-  int SP;
-  __device__ uint32_t operator()(int, int rr, int cc) const { return sO[rr * SP + cc]; }
-};
 
 struct GSrc {  // G_k = M_C (1 - O) where B_k < 1, else 0; the staged word holds the fixed-point
                // M_C (1 - O) in bits 0..23 and the B_k < 1 bits from bit 24 on (one load per use)
@@ -142,8 +152,9 @@ struct GSrc {  // G_k = M_C (1 - O) where B_k < 1, else 0; the staged word holds
 };
 
 template <int K, class Src>
-__device__ __forceinline__ void hsums_all(const Src& src, uint32_t* H) {
-  for (int it = threadIdx.x; it < DilGeom<K>::HR * kNSeg; it += blockDim.x) hsum_item<K>(src, H, it);
+__device__ __forceinline__ void hsums_all(const Src& src, uint32_t* H, unsigned act) {
+  for (int it = threadIdx.x; hsum_item<K>(src, H, it, act); it += blockDim.x) {
+  }
 }
 
 // The tiles a pass visits: those with the given flag, from the per-level list (every tile when
@@ -226,10 +237,18 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
       const int c = threadIdx.x % CW, X = x0 + c - h;
       const bool col_in = X >= 0 && X < res;
       if (c < S) {
+        if (x0 >= h && y0 >= h && x0 + kDT + h <= res && y0 + kDT + h <= res) {  // all inside the image
+          const float* src = Ib + (y0 - h + (int)threadIdx.x / CW) * res + X;
+          uint32_t* dst = II + (threadIdx.x / CW + 1) * P + c + 1;
 #pragma unroll 8
-        for (int r = threadIdx.x / CW; r < S; r += RP) {  // unrolled: loads in flight together
-          const int Y = y0 + r - h;
-          II[(r + 1) * P + c + 1] = col_in && Y >= 0 && Y < res ? to_fixed<K>(1.0f - Ib[Y * res + X]) : 0u;
+          for (int r = threadIdx.x / CW; r < S; r += RP, src += RP * res, dst += RP * P)
+            *dst = to_fixed<K>(1.0f - *src);
+        } else {
+#pragma unroll 8
+          for (int r = threadIdx.x / CW; r < S; r += RP) {  // unrolled: loads in flight together
+            const int Y = y0 + r - h;
+            II[(r + 1) * P + c + 1] = col_in && Y >= 0 && Y < res ? to_fixed<K>(1.0f - Ib[Y * res + X]) : 0u;
+          }
         }
       }
       if (threadIdx.x < P) II[threadIdx.x] = 0u;              // row 0
@@ -286,7 +305,8 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
         const float M = Mv[i];
         const float mval = M * (1.0f - O);
         lu = fmaf(mval, s, lu);
-        d.dil_g[pb + o] = to_fixed<K>(mval) | (mask << 24);  // mval <= 1: at most 2^Q < 2^24
+        const uint32_t fx = to_fixed<K>(mval);  // mval <= 1: at most 2^Q < 2^24
+        d.dil_g[pb + o] = fx != 0u ? fx | (mask << 24) : 0u;
         d.gOu[pb + o] = -(M * s);  // d/dO(q) of M(q)(1 - O(q))(1 - D_k(q)), times M(q)
       }
     }
@@ -307,6 +327,7 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
   constexpr int S = DilGeom<K>::S, SP = DilGeom<K>::SP, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
   constexpr float inv_q = 1.0f / (float)(1u << Q);
   extern __shared__ uint32_t sm[];
+  __shared__ uint32_t s_or[kDThreads / 32];
   uint32_t* sM = sm;
   uint32_t* H = sM + S * SP;
   // the tiles with container coverage within the halo (G = 0 over the others and their halos); the
@@ -328,14 +349,29 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
       const int c = threadIdx.x % CW, X = x0 + c - h;
       const bool col_in = X >= 0 && X < res;
       const uint32_t* gsrc = d.dil_g + pb;
+      uint32_t any = 0u;
       if (c < S) {
+        if (x0 >= h && y0 >= h && x0 + kDT + h <= res && y0 + kDT + h <= res) {  // all inside the image
+          const uint32_t* src = gsrc + (y0 - h + (int)threadIdx.x / CW) * res + X;
+          uint32_t* dst = sM + (threadIdx.x / CW) * SP + c;
 #pragma unroll 8
-        for (int r = threadIdx.x / CW; r < S; r += RP) {  // unrolled: loads in flight together
-          const int Y = y0 + r - h;
-          const int o = Y * res + X;
-          sM[r * SP + c] = col_in && Y >= 0 && Y < res ? gsrc[o] : 0u;
+          for (int r = threadIdx.x / CW; r < S; r += RP, src += RP * res, dst += RP * SP) {
+            const uint32_t w = *src;
+            any |= w;
+            *dst = w;
+          }
+        } else {
+#pragma unroll 8
+          for (int r = threadIdx.x / CW; r < S; r += RP) {  // unrolled: loads in flight together
+            const int Y = y0 + r - h;
+            const uint32_t w = col_in && Y >= 0 && Y < res ? gsrc[Y * res + X] : 0u;
+            any |= w;
+            sM[r * SP + c] = w;
+          }
         }
       }
+      any = __reduce_or_sync(0xffffffffu, any);
+      if ((threadIdx.x & 31) == 0) s_or[threadIdx.x >> 5] = any;
     }
     // the thread's output item (column c, rows r0..r0 + kVRows - 1): the forward pass's direct
     // part of dL_u/dO is read now, in flight during the horizontal pass
@@ -346,14 +382,19 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
 #pragma unroll
     for (int i = 0; i < kVRows; ++i) gv[i] = own ? g[min(y0 + r0 + i, res - 1) * res + Xc] : 0.0f;
     __syncthreads();
-    hsums_all<K>(GSrc{sM, SP}, H);
+    uint32_t act = 0u;
+#pragma unroll
+    for (int w = 0; w < kDThreads / 32; ++w) act |= s_or[w];
+    act = act >> 24 & ((1u << K) - 1u);
+    if (act == 0u && own) continue;  // nothing to add
+    hsums_all<K>(GSrc{sM, SP}, H, act);
     __syncthreads();
     float wq[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) wq[k] = d.L.dil_w[k] * inv_q;
     {
       uint32_t B[K][kVRows];
-      vsums_col<K>(H, c, r0, B);
+      vsums_col<K>(H, c, r0, act, B);
 #pragma unroll
       for (int i = 0; i < kVRows; ++i) {
         const int Y = y0 + r0 + i;
