@@ -449,7 +449,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_raster_chunks(Dev d) {
 // 48 -> 34 us; 1000 elements at 1024^2: 18 us before and now, 8 of them the launch and the first reads.
 // ------------------------------------------------------------------------------------------------
 constexpr int kCompWarps = 4;
-constexpr int kCompGroup = 2;   // pairs whose records are read together
 constexpr int kCompWide = 256;  // lists of up to this many covering pairs are ranked in shared memory
 
 // A tile's place: origin in pixels (x | y << 16), side and first pixel of its problem.
@@ -487,9 +486,16 @@ __device__ __forceinline__ TilePos locate_tiles(const Dev& d, int base, int coun
   return {(unsigned)(tx * T) | (unsigned)(ty * T) << 16, d.prob_res[p], d.prob_pix_base[p]};
 }
 
-template <int T>
-__global__ void __launch_bounds__(kCompWarps * 32, 9) k_composite(Dev d, float* out_bw, float* out_tau, int flags,
-                                                                  int C) {
+// G pairs' records are read together: two where the tiles outnumber the warps and resident warps hide the
+// reads, eight (with twice the registers) where each warp has one tile at most, so that a crowded tile's
+// list is a shorter chain.  1000 elements, two -> eight: 20 -> 16 us at 128^2, 14 -> 12 at 256^2 (the whole
+// iteration 68 -> 64 and 70 -> 66); 200 blobs at 512^2: 50.6 -> 49.3 an iteration; with more tiles than
+// warps eight are slower, as fewer warps are resident (1000 elements at 1024^2: 87 -> 91, 64 collages: 863 ->
+// 943).
+constexpr int kCompWideGroup = 8;
+template <int T, int G>
+__global__ void __launch_bounds__(kCompWarps * 32, G == 2 ? 9 : 4) k_composite(Dev d, float* out_bw, float* out_tau,
+                                                                              int flags, int C) {
   constexpr int UNITS = T * T / 64, NP = T * T, DY = 32 / T;
   __shared__ unsigned s_ord[kCompWarps][kCompWide];   // the covering pairs' slots and classes, in order
   __shared__ unsigned s_elem[kCompWarps][kCompWide];  // a long list's element ids, in list order
@@ -627,21 +633,21 @@ __global__ void __launch_bounds__(kCompWarps * 32, 9) k_composite(Dev d, float* 
         if (in0) cov[0] = d.covc[at.pix + off];
         if (in1) cov[1] = d.covc[at.pix + off + DY * at.res];
       }
-      // products over the pairs in element order, in groups of kCompGroup pairs whose signed
+      // products over the pairs in element order, in groups of G pairs whose signed
       // distances are read before any is used
       float keep[2] = {1.0f, 1.0f}, keept[2] = {1.0f, 1.0f};
       int nfull[2] = {0, 0}, npos[2] = {0, 0};  // pairs with c^pad = 1, with c^pad > 0
       const float2* sv = d.saved + unit * 64 + lane;
-      for (int i0 = 0; i0 < na; i0 += kCompGroup) {
+      for (int i0 = 0; i0 < na; i0 += G) {
         if (wide && i0 % kCompWide == 0) {  // the next stretch of a very long list
           __syncwarp();
           for (int i = lane; i < min(kCompWide, na - i0); i += 32) w_ord[i] = d.tile_sorted[lb + i0 + i];
           __syncwarp();
         }
-        float sd[kCompGroup][2];
-        unsigned ent_u[kCompGroup];
+        float sd[G][2];
+        unsigned ent_u[G];
 #pragma unroll
-        for (int u = 0; u < kCompGroup; ++u) {
+        for (int u = 0; u < G; ++u) {
           ent_u[u] = i0 + u < na ? w_ord[(i0 + u) % kCompWide] : kPairOut << kSlotBits;
           if (ent_u[u] >> kSlotBits == kPairNear) {
             const float2* rec = sv + (size_t)(ent_u[u] & kSlotMask) * NP;
@@ -650,7 +656,7 @@ __global__ void __launch_bounds__(kCompWarps * 32, 9) k_composite(Dev d, float* 
           }
         }
 #pragma unroll
-        for (int u = 0; u < kCompGroup; ++u) {
+        for (int u = 0; u < G; ++u) {
           const unsigned cls = ent_u[u] >> kSlotBits;  // (the same in every lane)
           if (cls == kPairNear) {
 #pragma unroll
@@ -1096,7 +1102,9 @@ static cudaError_t fwd_t(const Dev& d, cudaStream_t s, int pair_grid, int tile_g
     int C = 1;
     while (C < 32 && 2ll * C * 4 * tile_grid * per_block <= d.total_tiles) C *= 2;
     const int grid = C > 1 ? (d.total_tiles + C * per_block - 1) / (C * per_block) : tile_grid;
-    e = klaunch(d.pdl, k_composite<T>, grid, kCompWarps * 32, 0, s, d, bw, tau, flags, C);
+    const bool few = d.total_tiles <= tile_grid * per_block;
+    e = klaunch(d.pdl, few ? k_composite<T, kCompWideGroup> : k_composite<T, 2>, grid, kCompWarps * 32, 0, s, d, bw,
+                tau, flags, C);
   }
   return e;
 }
@@ -1143,7 +1151,7 @@ static void per_sm_t(int emit_threads, RasterOcc* o) {
   if (emit_threads == 256) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_raster_chunks<T, 256>, 256, 0);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_raster_chunks<T, 128>, 128, 0);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_raster_bwd<T, false>, kPairWarps * 32, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k_composite<T>, kCompWarps * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k_composite<T, 2>, kCompWarps * 32, 0);
   o->fwd_per_sm = a > 0 ? a : 1;
   o->bwd_per_sm = b > 0 ? b : 1;
   o->tile_per_sm = c > 0 ? c : 1;
