@@ -526,6 +526,7 @@ static cudaError_t enqueue_level_switch(const Dev& d, cudaStream_t s) {
 // chunks (of 320 segments) 88.4, 70.8, 77.0, 73.8; 500 chunks 74.8, 72.8, 67.1, 72.3; 1000 chunks 92.7,
 // 95.7, 90.7, 100.4; 5000 chunks 398.8, 444.4, 432.3, 547.8.
 static void choose_emission(collage_t h, int chunks) {
+  h->d.few_chunks = chunks <= 8 * h->sms;
   if (h->tuned) return;
   const bool small = chunks <= 3 * h->sms;
   h->d.chunk_tiles = (small ? kChunkPx / 2 : kChunkPx) / h->d.tile;
@@ -990,6 +991,9 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(cudaMemset(d.paths, 0, sizeof(unsigned long long) * 4));
   CKC(dmalloc(h->owned, h->ctl, kCtlWords));
   CKC(cudaMemset(h->ctl, 0, sizeof(int) * kCtlWords));
+  CKC(dmalloc(h->owned, d.slots, 3 * kSlotInts));
+  CKC(cudaMemset(d.slots, 0, sizeof(int) * 3 * kSlotInts));
+  d.sms = h->sms;
   CKC(dmalloc(h->owned, d.elem_pbase, h->N));
   d.status = h->ctl;
   d.step = h->ctl + 1;

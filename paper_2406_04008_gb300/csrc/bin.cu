@@ -188,6 +188,8 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     d.work[1] = 0;
     d.work[3] = 0;
   }
+  if (blockIdx.x == 0)  // the distribution term's blocks count themselves again while the composite runs
+    for (int i = threadIdx.x; i < 2 * kSlotInts; i += kTfThreads) d.slots[kSlotInts + i] = 0;
   if (wid == 0) {
     const int e = E == 1 ? 0 : lane >> 3, k = lane & 3, ge = min((int)blockIdx.x * E + e, d.n_elems - 1);
     const bool writer = (E == 1 ? lane < 4 : (lane & 7) < 4) && (int)blockIdx.x * E + e < d.n_elems;

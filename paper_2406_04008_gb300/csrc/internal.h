@@ -149,6 +149,8 @@ struct Dev {
                                 //   [3] blocks of the last gradient kernel that have finished
                                 //   (zeroed by the transform), [5] blocks of the Adam flush that
                                 //   have finished (its last block zeroes it), [2, 4, 6, 7] spare
+  int* slots;                   // [3 * kSlotInts] block counts of balanced_slot: the emission's (zeroed by the
+                                //   composite), the distribution term's forward and adjoint ones (by the transform)
   unsigned long long* paths;    // [4] cumulative counts of the rarely taken kernel paths (since
                                 //   create): [0] pixel rows of a near pair whose crossings
                                 //   overflow the per-row list (winding over every segment),
@@ -158,6 +160,8 @@ struct Dev {
                                 //   memory), [3] container ring chunks after a ring's first
   LossParams L;
   int deterministic;
+  int sms;                      // SMs of the device
+  int few_chunks;               // 1: the level has at most eight chunks per SM, all taken in one wave of blocks
   int pdl;                      // launch the iteration's kernels with programmatic serialisation
   // ---- outline fitting (fit_controls): the points of each element are the parameters ----
   int fit;                      // 1: the adjoint accumulates dv and k_ctrl_step runs Adam on ctrl
@@ -241,6 +245,47 @@ __device__ __forceinline__ float force_potential(const LossParams& L, float px, 
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ---- which block takes which work item ----
+// Blocks that are launched while the predecessor drains go to whichever SM has room: one SM takes eight
+// consecutive blocks of the emission and another none (1000 elements at 1024^2: the 602 long outlines, first
+// in the list, lay on 86 of 152 SMs), and an SM that is free early takes up to 18 of the distribution term's
+// one-tile blocks, a mean of 6.7.  Where all blocks of a grid are resident at once, each takes its item by
+// its rank among the blocks on its own SM instead: the r-th block of an SM takes the next of items
+// [r n_sm, (r + 1) n_sm), so that each SM gets an even share of the front of the list, and the grid's idle
+// rest lies on the SMs with the most blocks.  A block whose range is spent takes the last free item; as there
+// are as many items as blocks, each item is taken exactly once whatever the placement.  Runs before the wait
+// on the predecessor (`c` has been zero since the predecessor's predecessor or earlier), so that its two
+// atomics are hidden; one thread of each block calls it once.  Per iteration: 1000 elements at 1024^2 86.9 ->
+// 81.1 us, at 128^2 to 512^2 64.7, 65.6, 70.8 -> 62.6, 61.6, 64.7; 100 outlines at 1000^2 66.0 -> 62.1; 120
+// elements at 200^2 48.6 -> 46.4.  (Dealing the items over the block indices by a multiplier left up to
+// eight long outlines on some SMs and none on others: half the gain.)
+constexpr int kSlotSms = 256, kSlotRanks = 32, kSlotInts = kSlotSms + kSlotRanks;
+__device__ __forceinline__ int balanced_slot(int* c, int n_sm) {
+  const int G = (int)gridDim.x, n = (G + n_sm - 1) / n_sm;
+  unsigned sm;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+  auto take = [&](int r) {
+    const int i = r * n_sm + atomicAdd(&c[kSlotSms + r], 1);
+    return i < min((r + 1) * n_sm, G) ? i : -1;
+  };
+  const int rank = atomicAdd(&c[sm % kSlotSms], 1);
+  int i = rank < n ? take(rank) : -1;
+  for (int r = n - 1; i < 0 && r >= 0; --r) i = take(r);
+  return i < 0 ? G : i;
+}
+// The block's item: by balanced_slot, or by its index where n_sm is 0 (the same in every thread).
+__device__ __forceinline__ int first_item(int* c, int n_sm) {
+  __shared__ int s_first;
+  if (n_sm == 0) return (int)blockIdx.x;
+  if (threadIdx.x == 0) s_first = balanced_slot(c, n_sm);
+  __syncthreads();
+  return s_first;
+}
+// The n_sm of a grid of `grid` blocks: 0 beyond per_sm per SM (at most kSlotRanks).
+inline int slot_sms(const Dev& d, long long grid, int per_sm) {
+  return grid <= (long long)d.sms * per_sm ? d.sms : 0;
 }
 
 template <typename... KArgs, typename... Args>

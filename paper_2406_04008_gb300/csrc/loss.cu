@@ -200,7 +200,7 @@ struct IIGeom {
 };
 
 template <int K>
-__global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
+__global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d, int n_sm) {
   constexpr int S = DilGeom<K>::S, P = IIGeom<K>::P, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
   constexpr float inv_q = 1.0f / (float)(1u << Q);
   extern __shared__ uint32_t sm[];
@@ -209,9 +209,10 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
   // the tiles with container coverage; on the others M_C (1 - O) = 0, dL_u/dO = 0 and the loss
   // partial is 0, as written once per level.  The lists and the coverage are the level's: the first
   // tile's place and coverage are read before the composite has completed.
+  const int first = first_item(d.slots + kSlotInts, n_sm);
   const int n_own = dil_count(d, 0);
   DilTile t{};
-  if ((int)blockIdx.x < n_own) t = dil_place(d, 0, blockIdx.x);
+  if (first < n_own) t = dil_place(d, 0, first);
   // the thread's output item: column c, rows r0..r0 + kVRows - 1
   const int c = threadIdx.x % kDT, r0 = (threadIdx.x / kDT) * kVRows;
   float Iv[kVRows], Mv[kVRows];
@@ -220,11 +221,11 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
     for (int i = 0; i < kVRows; ++i)
       Mv[i] = d.covc[t.pb + min(t.y0 + r0 + i, t.res - 1) * t.res + min(t.x0 + c, t.res - 1)];
   };
-  if ((int)blockIdx.x < n_own) coverage();
+  if (first < n_own) coverage();
   pdl_enter();
   if (*d.status & kStatusNoBins) return;
-  for (int li = blockIdx.x; li < n_own; li += gridDim.x) {
-    if (li != (int)blockIdx.x) {
+  for (int li = first; li < n_own; li += gridDim.x) {
+    if (li != first) {
       t = dil_place(d, 0, li);
       coverage();
     }
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d) {
 }
 
 template <int K>
-__global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
+__global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d, int n_sm) {
   constexpr int S = DilGeom<K>::S, SP = DilGeom<K>::SP, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
   constexpr float inv_q = 1.0f / (float)(1u << Q);
   extern __shared__ uint32_t sm[];
@@ -332,13 +333,14 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d) {
   uint32_t* H = sM + S * SP;
   // the tiles with container coverage within the halo (G = 0 over the others and their halos); the
   // first one's place is read before the forward pass has completed
+  const int first = first_item(d.slots + 2 * kSlotInts, n_sm);
   const int n_halo = dil_count(d, 1);
   DilTile t{};
-  if ((int)blockIdx.x < n_halo) t = dil_place(d, 1, blockIdx.x);
+  if (first < n_halo) t = dil_place(d, 1, first);
   pdl_enter();
   if (*d.status & kStatusNoBins) return;
-  for (int li = blockIdx.x; li < n_halo; li += gridDim.x) {
-    if (li != (int)blockIdx.x) t = dil_place(d, 1, li);
+  for (int li = first; li < n_halo; li += gridDim.x) {
+    if (li != first) t = dil_place(d, 1, li);
     const int x0 = t.x0, y0 = t.y0, res = t.res;
     const long long pb = t.pb;
     // a tile without coverage of its own was not written by the forward pass: store, not add
@@ -542,8 +544,10 @@ cudaError_t prepare_dilate(int n_dil) {
 template <int K>
 static cudaError_t launch_k(const Dev& d, cudaStream_t s, bool backward) {
   const size_t sm = dilate_smem(K, backward);
-  if (backward) return klaunch(d.pdl, k_dilate_bwd<K>, d.total_dtiles, kDThreads, sm, s, d);
-  return klaunch(d.pdl, k_dilate_fwd<K>, d.total_dtiles, kDThreads, sm, s, d);
+  // one tile a block: balanced while the blocks fit the SMs at once; beyond, later blocks even the load out
+  const int n_sm = slot_sms(d, d.total_dtiles, 8);
+  if (backward) return klaunch(d.pdl, k_dilate_bwd<K>, d.total_dtiles, kDThreads, sm, s, d, n_sm);
+  return klaunch(d.pdl, k_dilate_fwd<K>, d.total_dtiles, kDThreads, sm, s, d, n_sm);
 }
 
 cudaError_t launch_dilate(const Dev& d, cudaStream_t s, bool backward) {

@@ -147,7 +147,8 @@ __device__ __forceinline__ float seg_d2(float dx, float dy, float4 s, float2 f) 
 // tile at each of them: 120 elements at 200^2 28 us, 22.6 now; 64 collages at 8-px tiles, by
 // the same code, 251 -> 235.)
 template <int T, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_raster_chunks(Dev d) {
+__global__ void __launch_bounds__(NT, 1024 / NT) k_raster_chunks(Dev d, int n_sm) {
+  const int first = first_item(d.slots, n_sm);
   pdl_enter();
   constexpr int CW = kChunkPx / T, NCT = CW * CW, NP = T * T, UNITS = NP / 64, UH = 64 / T;
   constexpr int NCU = NCT * UNITS;  // units of a chunk
@@ -177,7 +178,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_raster_chunks(Dev d) {
     *d.pending = 0;
   }
   // the slots are void when the pairs exceed the capacity (the transform latched it)
-  for (int i = (*d.status & kStatusOverflow) ? n_chunks : blockIdx.x, it = 0; i < n_chunks; ++it) {
+  for (int i = (*d.status & kStatusOverflow) ? n_chunks : first, it = 0; i < n_chunks; ++it) {
     if (tid == 0) {
       // chunks beyond the grid are taken by an atomic count (none when the grid covers them all)
       s_next[it & 1] = n_chunks > (int)gridDim.x ? (int)gridDim.x + atomicAdd(&d.work[0], 1) : n_chunks;
@@ -513,6 +514,8 @@ __global__ void __launch_bounds__(kCompWarps * 32, G == 2 ? 9 : 4) k_composite(D
   };
   if (base < d.total_tiles) place();
   pdl_enter();
+  if (blockIdx.x == 0)  // the emission has completed
+    for (int i = threadIdx.x; i < kSlotInts; i += kCompWarps * 32) d.slots[i] = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // the emission has completed: its work list is spent
     d.chunk_count[0] = d.chunk_count[1] = 0;
     d.work[0] = 0;
@@ -1091,10 +1094,13 @@ struct TileCfg<16> {
 template <int T>
 static cudaError_t fwd_t(const Dev& d, cudaStream_t s, int pair_grid, int tile_grid, float* bw,
                          float* tau, int part, int flags) {
+
   cudaError_t e = cudaSuccess;
+  // (with more chunks than blocks the first wave is all long outlines, and the rest are taken as blocks end)
+  const int n_sm = d.few_chunks ? slot_sms(d, pair_grid, kSlotRanks) : 0;
   if (part & 1)
-    e = d.emit_threads == 256 ? klaunch(d.pdl, k_raster_chunks<T, 256>, pair_grid, 256, 0, s, d)
-                              : klaunch(d.pdl, k_raster_chunks<T, 128>, pair_grid, 128, 0, s, d);
+    e = d.emit_threads == 256 ? klaunch(d.pdl, k_raster_chunks<T, 256>, pair_grid, 256, 0, s, d, n_sm)
+                              : klaunch(d.pdl, k_raster_chunks<T, 128>, pair_grid, 128, 0, s, d, n_sm);
   if (e == cudaSuccess && (part & 2)) {
     // tiles a warp takes at once: a power of two that leaves four resident waves of blocks, so that dense
     // and empty stretches even out; then one run per warp
