@@ -49,7 +49,7 @@ struct collage_s {
   struct LevelTab {
     std::vector<int> res, ntx, tile_base, dtile_base;
     std::vector<long long> pix_base;
-    int total_tiles = 0, total_dtiles = 0;
+    int total_tiles = 0, total_dtiles = 0, max_tiles = 0;
     long long total_pix = 0;
     int* d_res = nullptr;
     int* d_ntx = nullptr;
@@ -457,6 +457,8 @@ static collage_status build_levels(collage_t h) {
       t.pix_base[p + 1] = t.pix_base[p] + (long long)r * r;
     }
     t.total_tiles = t.tile_base[P];
+    t.max_tiles = 0;
+    for (int p = 0; p < P; ++p) t.max_tiles = std::max(t.max_tiles, t.tile_base[p + 1] - t.tile_base[p]);
     t.total_dtiles = t.dtile_base[P];
     t.total_pix = t.pix_base[P];
     np = std::max(np, (size_t)t.total_pix);
@@ -496,6 +498,7 @@ static collage_status apply_level(collage_t h, int level) {
   d.prob_dtile_base = t.d_dtile_base;
   d.prob_pix_base = t.d_pix_base;
   d.total_tiles = t.total_tiles;
+  d.max_tiles = t.max_tiles;
   d.total_dtiles = t.total_dtiles;
   d.total_pix = t.total_pix;
   h->res = t.res;
@@ -987,6 +990,9 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(cudaMemset(d.dq, 0, sizeof(float4) * h->N));
   CKC(dmalloc(h->owned, d.loss_terms, 5 * h->P));
   CKC(cudaMemset(d.loss_terms, 0, sizeof(float) * 5 * h->P));
+  CKC(dmalloc(h->owned, d.loss_part, (size_t)h->P * kLossParts));
+  CKC(dmalloc(h->owned, d.loss_done, h->P));
+  CKC(cudaMemset(d.loss_done, 0, sizeof(int) * h->P));
   CKC(dmalloc(h->owned, d.paths, 4));
   CKC(cudaMemset(d.paths, 0, sizeof(unsigned long long) * 4));
   CKC(dmalloc(h->owned, h->ctl, kCtlWords));

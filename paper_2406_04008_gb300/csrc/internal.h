@@ -20,6 +20,8 @@ namespace collage {
 
 constexpr int kMaxDil = 8;
 constexpr int kTrigSteps = 1024;        // angles of the transform's table
+constexpr int kLossUnits = 2048;        // 64-px units of an image per part of its loss,
+constexpr int kLossParts = 16;          //   in at most this many parts
 constexpr int kCtlWords = 24;           // device control words (status first, see Dev)
 constexpr int kChunkPx = 64;            // side, in pixels, of the emission's chunks of an element
 constexpr int kHeavyChunk = 1024;       // segments x tiles above which a chunk is taken first
@@ -77,6 +79,7 @@ struct Dev {
   const long long* prob_pix_base;  // [P+1]
   const int* prob_dtile_base;   // [P+1] dilation tiles
   int total_tiles, total_dtiles;
+  int max_tiles;                // tiles of the largest problem
   long long total_pix;
   int tile;                     // raster tile side
   int emit_threads;             // threads per block of the emission / distance kernel (128, 256)
@@ -140,6 +143,8 @@ struct Dev {
   float4* dq;                   // [n] gradient
   float4* partial;              // [cap * units per tile] deterministic gradient partials, by slot
   float* loss_terms;            // [P*5]
+  float4* loss_part;            // [P * kLossParts] the sums over each part of a problem's loss partials
+  int* loss_done;               // [P] parts summed so far (the last one zeroes it)
   int* status;                  // [1]
   int* step;                    // [1] Adam step count (the last gradient kernel advances it)
   int* pending;                 // [1] 1: the Adam step `step` is computed (dq) but not yet applied

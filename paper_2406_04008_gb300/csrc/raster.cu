@@ -757,8 +757,8 @@ __global__ void __launch_bounds__(kCompWarps * 32) k_empty_loss(Dev d) {
 // Adjoint, one unit (64 pixels) of a (tile, element) pair per warp: dL/dIhat and dL/dA_tau per pixel,
 // then the chain dL/dc -> dc/dsd -> dsd/d(closest segment) -> d/d(tx, ty, theta, s) of Eq. 2, reduced
 // over the unit's pixels by a fixed shuffle tree and added to the element's gradient (or stored per unit).
-// The grid's first blocks, one per problem, assemble the loss instead: its partials are complete, and
-// the work (a read of 16 B per unit) fits beside the adjoint's round trips without a launch, a second
+// The grid's first blocks, one per problem or more, assemble the loss instead: its partials are complete,
+// and the work (a read of 16 B per unit) fits beside the adjoint's round trips without a launch, a second
 // stream and the two joins that the end of an iteration waited for.
 // What the kernels before the predecessor wrote is read before the predecessor has completed: the work
 // list, the saved distances and, when the distribution term's adjoint is the predecessor, the images.
@@ -767,14 +767,28 @@ __device__ __forceinline__ float warp_sum_f(float x) {
   for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
 }
-// Loss of one problem (Eq. 8): fixed-order float sums of the partials (eight strided accumulators per
-// thread, then a shuffle tree within and across warps).  Float throughout: FP64 arithmetic is slow on this
-// part and 1e-7 relative is ample for a sum of non-negative partials.
-__device__ void assemble_loss(const Dev& d, int p) {
+// Loss of one problem (Eq. 8) in parts of kLossUnits units or more, by its own size alone, so that it has the
+// same bits in any batch: fixed-order float sums of a part's partials (eight strided accumulators per thread,
+// then a shuffle tree within and across warps), and the block that ends last adds the parts in order.  Float
+// throughout: FP64 arithmetic is slow on this part and 1e-7 relative is ample for a sum of non-negative
+// partials.  A block reads 1024 units in a round trip, and one block for the 16384 of a 1024^2 image ended 4 to 7
+// us after the adjoint's others; in parts, summed before the predecessor has completed where that is the
+// distribution term's adjoint, an iteration of 100 outlines at 1000^2 takes 56.4 us instead of 61.9, of 64
+// outline fits at 256^2 96.5 instead of 99.3, of 5000 elements at 2048^2 370 instead of 373.
+// Returns whether the problem has more than one part and this was one of them.
+__device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
   constexpr int NT = kPairWarps * 32, ACC = 8;
   __shared__ float s_red[4][kPairWarps];
   const int units = d.tile * d.tile / 64;
-  const int t0 = d.prob_tile_base[p] * units, t1 = d.prob_tile_base[p + 1] * units;
+  int t0 = d.prob_tile_base[p] * units, t1 = d.prob_tile_base[p + 1] * units;
+  const int parts = min(max((t1 - t0) / kLossUnits, 1), kLossParts);
+  if (wait) pdl_enter();  // the place is the level's: read before the predecessor has completed
+  if (part >= parts) return false;
+  if (parts > 1) {
+    const int n = (t1 - t0 + parts - 1) / parts;
+    t0 += part * n;
+    t1 = min(t0 + n, t1);
+  }
   float a[ACC] = {}, b[ACC] = {}, c[ACC] = {}, u[ACC] = {};
   for (int t = t0 + (int)threadIdx.x; t < t1; t += NT * ACC)
 #pragma unroll
@@ -785,8 +799,13 @@ __device__ void assemble_loss(const Dev& d, int p) {
       c[k] += v.z;
     }
   if (d.L.gamma != 0.0f && d.L.n_dil > 0) {
-    const int u1 = d.prob_dtile_base[p + 1];
-    for (int t = d.prob_dtile_base[p] + (int)threadIdx.x; t < u1; t += NT * ACC)
+    int u0 = d.prob_dtile_base[p], u1 = d.prob_dtile_base[p + 1];
+    if (parts > 1) {
+      const int n = (u1 - u0 + parts - 1) / parts;
+      u0 += part * n;
+      u1 = min(u0 + n, u1);
+    }
+    for (int t = u0 + (int)threadIdx.x; t < u1; t += NT * ACC)
 #pragma unroll
       for (int k = 0; k < ACC; ++k) u[k] += t + k * NT < u1 ? d.lossU[t + k * NT] : 0.0f;
   }
@@ -805,6 +824,22 @@ __device__ void assemble_loss(const Dev& d, int p) {
   if (threadIdx.x == 0) {
     float r[4];
     for (int k = 0; k < 4; ++k) r[k] = (s_red[k][0] + s_red[k][1]) + (s_red[k][2] + s_red[k][3]);
+    if (parts > 1) {
+      float4* sums = d.loss_part + (size_t)p * kLossParts;
+      __stcg(&sums[part], make_float4(r[0], r[1], r[2], r[3]));
+      __threadfence();
+      if (atomicAdd(&d.loss_done[p], 1) != parts - 1) return true;
+      __threadfence();
+      d.loss_done[p] = 0;
+      r[0] = r[1] = r[2] = r[3] = 0.0f;
+      for (int k = 0; k < parts; ++k) {
+        const float4 v = __ldcg(&sums[k]);
+        r[0] += v.x;
+        r[1] += v.y;
+        r[2] += v.z;
+        r[3] += v.w;
+      }
+    }
     const float np = (float)d.prob_res[p] * (float)d.prob_res[p];
     const float Lc = r[0] / np, Lo = r[1] / np, Ld = r[2] / np;
     float* out = d.loss_terms + 5 * p;
@@ -814,6 +849,7 @@ __device__ void assemble_loss(const Dev& d, int p) {
     out[3] = Ld;
     out[4] = d.L.alpha * Lc + d.L.beta * Lo + d.L.gamma * r[3] + d.L.delta * Ld;
   }
+  return parts > 1;
 }
 
 // a / b for normal b: the reciprocal's quotient with one residual correction (Markstein 1990), within an
@@ -834,20 +870,30 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
 }
 
 template <int T, bool FIT>  // FIT: also dL/d(vertex) for outline fitting (d.fit)
-__global__ void __launch_bounds__(kPairWarps * 32) k_raster_bwd(Dev d, int mark, int early) {
+__global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev d, int mark, int early, int n_loss) {
   constexpr int NP = T * T, UNITS = NP / 64, DY = 32 / T;
-  if ((int)blockIdx.x < d.n_probs) {
-    pdl_enter();
-    if (*d.status & kStatusNoBins) return;
-    assemble_loss(d, blockIdx.x);
-    if (mark) mark_step_if_last(d);
+  if ((int)blockIdx.x < n_loss) {
+    const bool ok = !(*d.status & kStatusNoBins);
+    int p = blockIdx.x, part = 0, per = 1;  // blocks per problem
+    if (n_loss > d.n_probs) {
+      per = n_loss / d.n_probs;
+      part = p / d.n_probs;
+      p -= part * d.n_probs;
+    }
+    bool wait = !early;
+    for (; ok && part < kLossParts && assemble_loss(d, p, part, wait); part += per) {
+      wait = false;
+      __syncthreads();
+    }
+    if (early || !ok) pdl_enter();
+    if (ok && mark) mark_step_if_last(d);
     return;
   }
   const float inv_rho = 1.0f / d.L.rho_px, pad = d.L.pad_px, tau = d.L.tau;
   const bool use_u = d.L.gamma != 0.0f;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int stride = ((int)gridDim.x - d.n_probs) * kPairWarps;
-  int i = ((int)blockIdx.x - d.n_probs) * kPairWarps + wid;
+  const int stride = ((int)gridDim.x - n_loss) * kPairWarps;
+  int i = ((int)blockIdx.x - n_loss) * kPairWarps + wid;
   if (*d.status & kStatusNoBins) {
     pdl_enter();
     return;
@@ -1126,15 +1172,20 @@ cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int t
 
 cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step) {
   // the loss blocks take the place of as many resident ones (at most half of them), so that none waits
-  const int grid = max(unit_grid - d.n_probs, (unit_grid + 1) / 2) + d.n_probs, mk = mark_step ? 1 : 0;
+  const int units = (int)min((long long)d.max_tiles * (d.tile * d.tile / 64), (long long)kLossUnits * kLossParts);
+  // a block for each part of the largest problem, in a sixteenth of the resident blocks: more of them leave
+  // the units' strided share to fewer warps (64 collages, an eighth and a half: 118.8 -> 122.9 and 190 us)
+  const int lb = max(min(units / kLossUnits, unit_grid / (16 * d.n_probs)), 1);
+  const int n_loss = d.n_probs * lb;
+  const int grid = max(unit_grid - n_loss, (unit_grid + 1) / 2) + n_loss, mk = mark_step ? 1 : 0;
   const int early = d.L.gamma != 0.0f && d.L.n_dil > 0 ? 1 : 0;  // the predecessor is the distribution adjoint
   switch (d.tile) {
     case 8:
       return klaunch(d.pdl, d.fit ? k_raster_bwd<8, true> : k_raster_bwd<8, false>, grid, kPairWarps * 32, 0, s, d, mk,
-                     early);
+                     early, n_loss);
     case 16:
       return klaunch(d.pdl, d.fit ? k_raster_bwd<16, true> : k_raster_bwd<16, false>, grid, kPairWarps * 32, 0, s, d,
-                     mk, early);
+                     mk, early, n_loss);
     default: return cudaErrorInvalidValue;
   }
 }
