@@ -122,8 +122,8 @@ typedef struct {
                                   every segment of the outline */
   long long path_long_near;    /* emission chunks of outlines of more than 512 segments (not
                                   staged in shared memory: read from global memory per tile) */
-  long long path_wide_tile;    /* tiles listing more than 32 elements (the composite ranks the
-                                  list in global memory instead of by warp shuffles) */
+  long long path_wide_tile;    /* tiles listing more than 32 elements (the composite ranks the list
+                                  in shared memory, beyond 256 covering ones in global memory) */
   long long path_ring_chunk;   /* container chunks after the first 1024 segments of a ring */
 } collage_info;
 

@@ -161,8 +161,8 @@ struct Dev {
                                 //   overflow the per-row list (winding over every segment),
                                 //   [1] emission chunks of outlines with more segments than
                                 //   are staged in shared memory,
-                                //   [2] tiles listing more than 32 pairs (ranked in global
-                                //   memory), [3] container ring chunks after a ring's first
+                                //   [2] tiles listing more than 32 pairs (ranked in shared
+                                //   or global memory), [3] container ring chunks after a ring's first
   LossParams L;
   int deterministic;
   int sms;                      // SMs of the device
@@ -312,7 +312,7 @@ inline cudaError_t klaunch(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 b
 // The last block of the kernel that completes an iteration's gradient marks the iteration's Adam
 // step pending (applied by the next transform) and advances the step count, unless the iteration
 // overflowed or met non-finite params.  Every block calls this once, after its last write to the
-// gradient; the counter work[3] is zeroed by the tile scan of each iteration.
+// gradient; the counter work[3] is zeroed by the transform of each iteration.
 __device__ __forceinline__ void mark_step_if_last(const Dev& d) {
   __syncthreads();
   if (threadIdx.x == 0) {
