@@ -191,6 +191,8 @@ collage_status collage_step_host(collage_t h, void* stream, int n_iters, const f
 
 /* Loss terms of the most recent iteration, [n_probs*5] (device). */
 collage_status collage_get_loss(collage_t h, void* stream, float* d_loss_terms);
+/* Params out and in, [4*n_elems] (device): one kernel where the buffer lies on the handle's device at a
+ * 16-byte boundary, else a copy by the runtime (another device's memory included). */
 collage_status collage_get_params(collage_t h, void* stream, float* d_params);
 collage_status collage_set_params(collage_t h, void* stream, const float* d_params);
 

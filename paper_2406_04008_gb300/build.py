@@ -17,6 +17,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libcollage.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libcollage_checked.so")
 SOURCES = ["api.cu", "bin.cu", "raster.cu", "loss.cu", "fit.cu", "mat.cu", "metrics.cu", "noalloc.cu", "peak.cu", "sched.cu"]
+HEADERS = ["edt.h", "internal.h", "route.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off",
          "-I" + INCLUDE, "-I" + CSRC]
@@ -29,7 +30,7 @@ def _nvcc():
 
 def _deps():
     return [os.path.join(CSRC, s) for s in SOURCES] + [
-        os.path.join(CSRC, "edt.h"), os.path.join(CSRC, "internal.h"), os.path.join(INCLUDE, "collage.h")]
+        os.path.join(CSRC, h) for h in HEADERS] + [os.path.join(INCLUDE, "collage.h")]
 
 
 def _fresh(lib):

@@ -117,6 +117,8 @@ class Collage:
 
     def set_params(self, params: torch.Tensor):
         p = _flat(params)
+        if p.numel() < 4 * self.n_elems:  # (the library reads four floats of every element)
+            raise ValueError(f"expected {4 * self.n_elems} floats")
         self._check(self.lib.collage_set_params(self.h, _stream(), _dptr(p)))
 
     # skeleton-based initialisation ------------------------------------------------------------

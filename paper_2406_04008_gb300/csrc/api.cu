@@ -13,6 +13,7 @@
 
 #include "collage.h"
 #include "internal.h"
+#include "route.h"
 
 #ifdef COLLAGE_CHECKED
 #include <nvtx3/nvToolsExt.h>
@@ -31,6 +32,7 @@ enum Mode { kRender = 0, kLossBwd = 1, kStep = 2 };
 struct collage_s {
   collage_options opt{};
   int P = 0, N = 0, V = 0;
+  int device = 0;  // the device that was current at create: its memory and kernels are the handle's
   // host copies of the problem
   std::vector<int> elem_prob, elem_voff, prob_elem_base, prob_grid, ring_off, prob_ring_base;
   std::vector<uint8_t> elem_closed;
@@ -866,6 +868,7 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
     cuda_fail(h, ce, "cudaGetDevice");
     return bail(COLLAGE_ERR_CUDA);
   }
+  h->device = dev;
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
   if (h->sms < 1) h->sms = 1;
   Dev& d = h->d;
@@ -1057,13 +1060,32 @@ extern "C" collage_status collage_render(collage_t h, void* stream, float* d_img
   return run_checked(h, (cudaStream_t)stream, kRender, d_img_bw, d_img_tau);
 }
 
+// Whether one of the handle's kernels may take the caller's buffer directly.  Another device's memory
+// and memory that no device owns go through the runtime's copy, which reaches the one and refuses the
+// other; a kernel would fault on either.
+static bool own_memory(collage_t h, const void* p) {
+  if (!p) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();  // (not a fault of the call)
+    return false;
+  }
+  return kernel_route(a.type, a.device, h->device);
+}
+
 extern "C" collage_status collage_loss_backward(collage_t h, void* stream, float* d_loss_terms,
                                                 float* d_dparams) {
   if (!h) return fail(nullptr, COLLAGE_ERR_INVALID_ARG, "handle is NULL");
   cudaStream_t s = (cudaStream_t)stream;
   collage_status st = run_checked(h, s, kLossBwd, nullptr, nullptr);
   if (st) return st;
-  if (d_loss_terms || d_dparams) CK(h, launch_copy_out(h->d, s, d_loss_terms, d_dparams));
+  float* k_terms = own_memory(h, d_loss_terms) ? d_loss_terms : nullptr;
+  float* k_grad = own_memory(h, d_dparams) ? d_dparams : nullptr;
+  if (k_terms || k_grad) CK(h, launch_copy_out(h->d, s, k_terms, k_grad));
+  if (d_loss_terms && !k_terms)
+    CK(h, cudaMemcpyAsync(d_loss_terms, h->d.loss_terms, sizeof(float) * 5 * h->P, cudaMemcpyDeviceToDevice, s));
+  if (d_dparams && !k_grad)
+    CK(h, cudaMemcpyAsync(d_dparams, h->d.dq, sizeof(float4) * h->N, cudaMemcpyDeviceToDevice, s));
   return COLLAGE_OK;
 }
 
@@ -1347,7 +1369,8 @@ extern "C" collage_status collage_get_loss(collage_t h, void* stream, float* d_l
 
 extern "C" collage_status collage_get_params(collage_t h, void* stream, float* d_params) {
   if (!h || !d_params) return fail(h, COLLAGE_ERR_INVALID_ARG, "NULL argument");
-  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0) {  // one kernel for the step and the copy
+  // one kernel for the step and the copy
+  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0 && own_memory(h, d_params)) {
     CK(h, launch_adam_flush(h->d, (cudaStream_t)stream, nullptr, nullptr, d_params));
     return COLLAGE_OK;
   }
@@ -1359,7 +1382,7 @@ extern "C" collage_status collage_get_params(collage_t h, void* stream, float* d
 extern "C" collage_status collage_set_params(collage_t h, void* stream, const float* d_params) {
   if (!h || !d_params) return fail(h, COLLAGE_ERR_INVALID_ARG, "NULL argument");
   // (a pending step belongs to the old params)
-  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0) {
+  if (reinterpret_cast<uintptr_t>(d_params) % sizeof(float4) == 0 && own_memory(h, d_params)) {
     CK(h, launch_adam_flush(h->d, (cudaStream_t)stream, nullptr, d_params));
     return COLLAGE_OK;
   }
