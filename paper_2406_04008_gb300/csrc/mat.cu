@@ -104,7 +104,8 @@ __device__ __forceinline__ void warp_max2(unsigned& hi, unsigned& lo) {
   hi = m;
 }
 
-// Greedy placement, one block per problem.  The elements' order is fixed before the first step
+// Greedy placement, one block per problem, or a cluster of eight where the axis pixels exceed one block's
+// shared memory (kPlaceBlocks).  The elements' order is fixed before the first step
 // (sorted by radius), and each step chooses one axis pixel (a candidate), so the steps are a serial
 // chain: what bounds this kernel is the latency of one step, not the candidates' arithmetic.
 //
@@ -128,7 +129,14 @@ constexpr int kPlaceWarps = kPlaceThreads / 32;
 constexpr int kPlaceRankMax = 4096;        // elements sorted in shared memory (more: a reduction per step)
 constexpr int kPlaceCells = 32;            // cells a side of the candidates' spatial order
 constexpr int kPlaceFast = kPlaceThreads;  // groups kept one per lane, their pixels in shared memory
-constexpr int kPlaceSmem = 221 * 1024;     // keys and candidates (else in global memory)
+// Shared memory for the keys and the candidates.  (The cluster form's exchange takes 2 KB more.)
+__host__ __device__ constexpr int place_smem(int blocks) { return (blocks == 1 ? 221 : 219) * 1024; }
+// A problem whose candidates one block can not hold (14 to 16 k of them: the star from 1024^2 on, the disk
+// and the annulus from 1100^2 on) is placed by a cluster of eight blocks, each with an eighth of the list:
+// a step's choices meet in every block's shared memory behind one cluster barrier, a step of 1.0 us.  (By
+// one block with the candidates in global memory a step took 3.3 us, more than the 2.2 us of a scan of every
+// candidate: 1000 elements in the star at 1200^2 4.2 ms for the whole initialisation, 1.08 now.)
+constexpr int kPlaceBlocks = 8;
 
 __device__ __forceinline__ unsigned long long elem_key(const Dev& d, int e, float fres) {
   const float r = __fmul_rn(__fmul_rn(d.elem_rbin[e], d.q[e].w), fres);
@@ -160,13 +168,30 @@ struct PlaceGroup {
 };
 constexpr unsigned kRoomKey = 0xd0000000u;
 
+// ---- the cluster form ----
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {  // every thread of every block, converged warps
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Into the same variable of block `rank`.
+__device__ __forceinline__ void store_remote(uint2* at, unsigned rank, uint2 v) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(at), r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(r), "r"(v.x), "r"(v.y) : "memory");
+}
+
 // FAST: the candidates in shared memory and at most one group per lane; else both in global memory.
-template <bool FAST>
+// NB blocks place a problem together, each with its share of nc candidates, and take the same steps.
+template <bool FAST, int NB>
 __device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, unsigned long long* s_key,
                             unsigned* cxy, float* ccl, const unsigned* cd2, PlaceGroup* groups, const unsigned* d2,
-                            int* placed) {
-  __shared__ unsigned long long s_red[kPlaceWarps];
-  __shared__ uint2 s_part[2][kPlaceWarps];  // per step parity: each warp's best (key, pixel)
+                            int* placed, unsigned long long* s_red, uint2 (*s_part)[NB * kPlaceWarps]) {
+  const unsigned rank = NB > 1 ? cluster_rank() : 0u;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, ng = (nc + 31) / 32;
   const int res = d.prob_res[p], e0 = d.prob_elem_base[p];
   const long long pb = d.prob_pix_base[p];
@@ -262,10 +287,25 @@ __device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, un
       }
       warp_max2(best.x, best.y);
     }
-    if (lane == 0) s_part[step & 1][wid] = best;
+    if (NB > 1) {
+      if (lane < NB) store_remote(&s_part[step & 1][rank * kPlaceWarps + wid], (unsigned)lane, best);
+    } else if (lane == 0) {
+      s_part[step & 1][wid] = best;
+    }
     if (ranked) r_bits = s_key32[2 * min(step + 1, ne - 1) + 1];  // the next step's radius
-    __syncthreads();  // (the buffer is written again two steps on, after the next step's barrier)
-    uint2 win = s_part[step & 1][lane % kPlaceWarps];
+    // (the buffer is written again two steps on, after the next step's barrier)
+    if (NB > 1) {
+      __syncwarp();
+      cluster_sync();
+    } else {
+      __syncthreads();
+    }
+    uint2 win = s_part[step & 1][lane % (NB * kPlaceWarps)];
+#pragma unroll
+    for (int i = 32; i < NB * kPlaceWarps; i += 32) {
+      const uint2 o = s_part[step & 1][i + lane];
+      if (o.x > win.x || (o.x == win.x && o.y > win.y)) win = o;
+    }
     warp_max2(win.x, win.y);
     px = (int)(~win.y & 0xffffu);
     py = (int)(~win.y >> 16);
@@ -275,34 +315,50 @@ __device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, un
         s_key32[2 * step + 1] = ~win.y;  // the pixel, beside the element
       } else {
         const int e = (int)(0xffffffffu - e_inv);
-        placed[e] = 1;
-        d.q[e].x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
-        d.q[e].y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
+        placed[e] = 1;  // (by every block: its own next reduction reads it)
+        if (rank == 0) {
+          d.q[e].x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
+          d.q[e].y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
+        }
       }
     }
     if (!ranked) __syncthreads();  // the mark is visible to the next step's reduction
   }
 }
 
-__global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* cand, const int* n_cand,
-                                                             const unsigned* d2, unsigned* gxy, float* clear,
-                                                             int* placed) {
+// Whether the keys and nc candidates of a problem of ne elements fit one block's shared memory and lanes.
+__device__ __forceinline__ bool place_fits(int nc, int ne, int smem, int* n_keys) {
+  int nk = 0;  // keys, padded to a power of two
+  if (ne <= kPlaceRankMax)
+    for (nk = 1; nk < ne;) nk <<= 1;
+  *n_keys = nk;
+  const int ng = (nc + 31) / 32;
+  return ng <= kPlaceFast && 8 * nk + ng * (32 * 12 + (int)sizeof(PlaceGroup)) <= smem;
+}
+
+// One problem, by the NB blocks of a cluster.
+template <int NB>
+__device__ void place(const Dev& d, int p, unsigned* cand, int n_cand, const unsigned* d2, unsigned* gxy, float* clear,
+                      int* placed) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ int s_cell[kPlaceCells * kPlaceCells];
   __shared__ int s_wsum[kPlaceWarps];
+  __shared__ unsigned long long s_red[kPlaceWarps];
+  __shared__ uint2 s_part[2][NB * kPlaceWarps];  // per step parity: each warp's best (key, pixel)
   static_assert(kPlaceCells * kPlaceCells == 2 * kPlaceThreads, "two cells per thread in the scan");
-  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int res = d.prob_res[p], nc = n_cand[p];
-  const long long pb = d.prob_pix_base[p];
-  const int e0 = d.prob_elem_base[p], ne = d.prob_elem_base[p + 1] - e0;
-  if (nc == 0) return;  // no inside pixel: the params stay
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int res = d.prob_res[p], e0 = d.prob_elem_base[p], ne = d.prob_elem_base[p + 1] - e0;
   const float fres = (float)res;
+  // the block's share of the candidates, and its place in the arrays of them
+  const int rank = NB > 1 ? (int)cluster_rank() : 0;
+  const int c_lo = (int)((long long)n_cand * rank / NB), nc = (int)((long long)n_cand * (rank + 1) / NB) - c_lo;
+  const long long pix0 = d.prob_pix_base[p], pb = pix0 + c_lo;
+  int nk;
+  const bool fast = place_fits((n_cand + NB - 1) / NB, ne, place_smem(NB), &nk);  // (the same in every block)
   // ---- the elements in placement order: decreasing key (radius bits, then the lower index) ----
   const bool ranked = ne <= kPlaceRankMax;
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_dyn);
-  int nk = 0;  // keys, padded to a power of two
   if (ranked) {
-    for (nk = 1; nk < ne;) nk <<= 1;
     for (int i = tid; i < nk; i += kPlaceThreads) s_key[i] = i < ne ? elem_key(d, e0 + i, fres) : 0ull;
     for (int k = 2; k <= nk; k <<= 1)
       for (int j = k >> 1; j > 0; j >>= 1) {
@@ -322,7 +378,6 @@ __global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* ca
   // ---- the candidates by cell, and the groups ----
   const int ng = (nc + 31) / 32;
   unsigned char* s_cand = s_dyn + sizeof(unsigned long long) * nk;
-  const bool fast = ng <= kPlaceFast && 8 * nk + ng * (32 * 12 + (int)sizeof(PlaceGroup)) <= kPlaceSmem;
   unsigned* cxy = fast ? reinterpret_cast<unsigned*>(s_cand) : gxy + pb;
   float* ccl = fast ? reinterpret_cast<float*>(s_cand) + 32 * ng : clear + pb;
   unsigned* cd2 = reinterpret_cast<unsigned*>(s_cand) + 64 * ng;  // in shared memory only
@@ -362,7 +417,7 @@ __global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* ca
   for (int gi = wid; gi < ng; gi += kPlaceWarps) {
     const int c = gi * 32 + lane;
     unsigned xy = c < nc ? cxy[c] : 0xffffffffu;
-    unsigned w = c < nc ? d2[pb + (long long)(xy >> 16) * res + (xy & 0xffffu)] : 0u;
+    unsigned w = c < nc ? d2[pix0 + (long long)(xy >> 16) * res + (xy & 0xffffu)] : 0u;
     const unsigned x = xy & 0xffffu, y = xy >> 16;
     const unsigned x0 = __reduce_min_sync(0xffffffffu, x), x1 = __reduce_max_sync(0xffffffffu, c < nc ? x : 0u);
     const unsigned y0 = __reduce_min_sync(0xffffffffu, y), y1 = __reduce_max_sync(0xffffffffu, c < nc ? y : 0u);
@@ -387,10 +442,13 @@ __global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* ca
     if (lane == 0) groups[gi] = PlaceGroup{(float)x0, (float)x1, (float)y0, (float)y1, FLT_MAX, FLT_MAX, 0u, 0u};
   }
   __syncthreads();
-  if (fast) place_steps<true>(d, p, nc, ne, ranked, s_key, reinterpret_cast<unsigned*>(s_cand),
-                              reinterpret_cast<float*>(s_cand) + 32 * ng, cd2, groups, d2, placed);
-  else place_steps<false>(d, p, nc, ne, ranked, s_key, gxy + pb, clear + pb, nullptr, groups, d2, placed);
-  if (!ranked) return;
+  if (NB > 1) cluster_sync();  // every block has started (before the first store into another's shared memory)
+  if (fast) place_steps<true, NB>(d, p, nc, ne, ranked, s_key, reinterpret_cast<unsigned*>(s_cand),
+                                  reinterpret_cast<float*>(s_cand) + 32 * ng, cd2, groups, d2, placed, s_red, s_part);
+  else if (NB > 1)
+    place_steps<false, NB>(d, p, nc, ne, ranked, s_key, gxy + pb, clear + pb, nullptr, groups, d2, placed, s_red,
+                           s_part);
+  if (!ranked || rank != 0) return;
   __syncthreads();
   for (int i = tid; i < ne; i += kPlaceThreads) {
     const unsigned xy = (unsigned)(s_key[i] >> 32);
@@ -398,6 +456,26 @@ __global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* ca
     d.q[e].x = __fdiv_rn(__fadd_rn((float)(xy & 0xffffu), 0.5f), fres);
     d.q[e].y = __fdiv_rn(__fadd_rn((float)(xy >> 16), 0.5f), fres);
   }
+}
+
+__global__ void __launch_bounds__(kPlaceThreads) k_mat_place(Dev d, unsigned* cand, const int* n_cand,
+                                                             const unsigned* d2, int* placed) {
+  pdl_enter();
+  const int p = blockIdx.x, nc = n_cand[p];
+  int nk;
+  if (nc == 0 || !place_fits(nc, d.prob_elem_base[p + 1] - d.prob_elem_base[p], place_smem(1), &nk)) return;
+  place<1>(d, p, cand, nc, d2, nullptr, nullptr, placed);
+}
+// The problems that the other kernel leaves, scheduled while that one runs.  (No inside pixel: the params
+// stay.)
+__global__ void __cluster_dims__(kPlaceBlocks) __launch_bounds__(kPlaceThreads)
+    k_mat_place_wide(Dev d, unsigned* cand, const int* n_cand, const unsigned* d2, unsigned* gxy, float* clear,
+                     int* placed) {
+  pdl_enter();
+  const int p = blockIdx.x / kPlaceBlocks, nc = n_cand[p];
+  int nk;
+  if (place_fits(nc, d.prob_elem_base[p + 1] - d.prob_elem_base[p], place_smem(1), &nk)) return;  // (the cluster's blocks agree)
+  place<kPlaceBlocks>(d, p, cand, nc, d2, gxy, clear, placed);
 }
 
 cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
@@ -409,7 +487,9 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
     e = cudaFuncSetAttribute(k_edt_cols<OutsideSite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
   if (e == cudaSuccess && rs > 48 * 1024)
     e = cudaFuncSetAttribute(k_mat_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlaceSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(1));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mat_place_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(kPlaceBlocks));
   if (e != cudaSuccess) return e;
   unsigned short* gcol = reinterpret_cast<unsigned short*>(g);
   k_edt_cols<<<dim3((max_res + kEdtCols - 1) / kEdtCols, d.n_probs), kEdtThreads, cs, s>>>(
@@ -419,8 +499,10 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
       d, d2, cand, n_cand, axis_out, width_out);
   // g is free after the row pass: it holds the candidates' coordinates when they do not fit in
   // shared memory
-  k_mat_place<<<d.n_probs, kPlaceThreads, kPlaceSmem, s>>>(d, cand, n_cand, d2, g, clear, placed);
-  return cudaGetLastError();
+  k_mat_place<<<d.n_probs, kPlaceThreads, place_smem(1), s>>>(d, cand, n_cand, d2, placed);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return klaunch(d.pdl, k_mat_place_wide, d.n_probs * kPlaceBlocks, kPlaceThreads, place_smem(kPlaceBlocks), s, d, cand,
+                 n_cand, d2, g, clear, placed);
 }
 
 }  // namespace collage
