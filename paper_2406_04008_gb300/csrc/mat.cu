@@ -17,6 +17,7 @@
 //    so every decision is reproducible.  The element's translation becomes its pixel centre;
 //    rotation and scale are kept.
 #include <cfloat>
+#include <type_traits>
 
 #include "collage.h"
 #include "edt.h"
@@ -120,8 +121,8 @@ __device__ __forceinline__ void warp_max2(unsigned& hi, unsigned& lo) {
 // In a group the pixels are in order of their key (D2, then the lower pixel), so the widest with room
 // is the first set bit of a ballot.  The warps' choices meet in one double-buffered exchange and one
 // barrier a step, and every warp reduces them by itself.  1000 elements on 16 k candidates: 0.05 ms to
-// sort and 0.7 us a step, 0.55 us once the first disks are placed (eight clustered blocks that scanned
-// every candidate at each step, with 64-bit shuffle reductions and a cluster barrier: 2.2 us a step).
+// sort and 0.45 us a step once the first disks are placed (eight clustered blocks that scanned every
+// candidate at each step, with 64-bit shuffle reductions and a cluster barrier: 2.2 us a step).
 // Sixteen warps: with 32 the barrier and the shared issue slots cost more than the fewer groups a
 // warp looks at save.
 constexpr int kPlaceThreads = 512;
@@ -187,8 +188,10 @@ __device__ __forceinline__ void store_remote(uint2* at, unsigned rank, uint2 v) 
 
 // FAST: the candidates in shared memory and at most one group per lane; else both in global memory.
 // NB blocks place a problem together, each with its share of nc candidates, and take the same steps.
-template <bool FAST, int NB>
-__device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, unsigned long long* s_key,
+// ranked: the elements' order is in s_key; else each thread keeps the largest of every 512th element, and looks
+// again when it is placed (5000 elements: 1.9 us a step; with a look at every element in each step 2.8).
+template <bool FAST, int NB, bool ranked>
+__device__ void place_steps(const Dev& d, int p, int nc, int ne, unsigned long long* s_key,
                             unsigned* cxy, float* ccl, const unsigned* cd2, PlaceGroup* groups, const unsigned* d2,
                             int* placed, unsigned long long* s_red, uint2 (*s_part)[NB * kPlaceWarps]) {
   const unsigned rank = NB > 1 ? cluster_rank() : 0u;
@@ -204,18 +207,24 @@ __device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, un
   unsigned r_bits = ranked ? s_key32[1] : 0u;
   int px = 0, py = 0;  // the previous element's pixel and radius (none before the first step)
   float pr = -1.0f, r_last = 0.0f;
+  unsigned long long ek = 0;  // not ranked: the thread's largest element not yet placed
+  bool own_placed = true;
   for (int step = 0; step < ne; ++step) {
     unsigned e_inv = 0u;
-    if (!ranked) {  // the largest element not yet placed, by a reduction
-      unsigned long long ek = 0;
-      for (int i = tid; i < ne; i += kPlaceThreads) {
-        if (placed[e0 + i]) continue;
-        const unsigned long long k = elem_key(d, e0 + i, fres);
-        ek = k > ek ? k : ek;
+    if (!ranked) {
+      if (own_placed) {
+        ek = 0;
+        for (int i = tid; i < ne; i += kPlaceThreads) {
+          if (placed[e0 + i]) continue;
+          const unsigned long long k = elem_key(d, e0 + i, fres);
+          ek = k > ek ? k : ek;
+        }
       }
-      ek = block_max(ek, s_red);
-      r_bits = (unsigned)(ek >> 32);
-      e_inv = (unsigned)ek;
+      const unsigned long long top = block_max(ek, s_red);
+      r_bits = (unsigned)(top >> 32);
+      e_inv = (unsigned)top;
+      own_placed = top == ek;  // (the keys differ by the element)
+      if (own_placed) placed[0xffffffffu - e_inv] = 1;
     }
     const float r = __uint_as_float(r_bits);
     // the groups' choices hold for radii that do not grow (the keys order the radii by their bits,
@@ -313,16 +322,12 @@ __device__ void place_steps(const Dev& d, int p, int nc, int ne, bool ranked, un
     if (tid == 0) {
       if (ranked) {
         s_key32[2 * step + 1] = ~win.y;  // the pixel, beside the element
-      } else {
+      } else if (rank == 0) {
         const int e = (int)(0xffffffffu - e_inv);
-        placed[e] = 1;  // (by every block: its own next reduction reads it)
-        if (rank == 0) {
-          d.q[e].x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
-          d.q[e].y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
-        }
+        d.q[e].x = __fdiv_rn(__fadd_rn((float)px, 0.5f), fres);
+        d.q[e].y = __fdiv_rn(__fadd_rn((float)py, 0.5f), fres);
       }
     }
-    if (!ranked) __syncthreads();  // the mark is visible to the next step's reduction
   }
 }
 
@@ -443,11 +448,20 @@ __device__ void place(const Dev& d, int p, unsigned* cand, int n_cand, const uns
   }
   __syncthreads();
   if (NB > 1) cluster_sync();  // every block has started (before the first store into another's shared memory)
-  if (fast) place_steps<true, NB>(d, p, nc, ne, ranked, s_key, reinterpret_cast<unsigned*>(s_cand),
-                                  reinterpret_cast<float*>(s_cand) + 32 * ng, cd2, groups, d2, placed, s_red, s_part);
-  else if (NB > 1)
-    place_steps<false, NB>(d, p, nc, ne, ranked, s_key, gxy + pb, clear + pb, nullptr, groups, d2, placed, s_red,
-                           s_part);
+  auto steps = [&](auto in_smem, auto in_order) {  // (shared memory by its own addresses, not by generic ones)
+    constexpr bool FAST = decltype(in_smem)::value, ORDER = decltype(in_order)::value;
+    if constexpr (FAST)
+      place_steps<true, NB, ORDER>(d, p, nc, ne, s_key, reinterpret_cast<unsigned*>(s_cand),
+                                   reinterpret_cast<float*>(s_cand) + 32 * ng, cd2, groups, d2, placed, s_red, s_part);
+    else
+      place_steps<false, NB, ORDER>(d, p, nc, ne, s_key, gxy + pb, clear + pb, nullptr, groups, d2, placed, s_red, s_part);
+  };
+  using std::true_type;
+  using std::false_type;
+  if (fast && ranked) steps(true_type{}, true_type{});
+  else if (fast) steps(true_type{}, false_type{});
+  else if (NB > 1 && ranked) steps(false_type{}, true_type{});
+  else if (NB > 1) steps(false_type{}, false_type{});
   if (!ranked || rank != 0) return;
   __syncthreads();
   for (int i = tid; i < ne; i += kPlaceThreads) {
