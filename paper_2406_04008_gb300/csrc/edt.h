@@ -18,6 +18,15 @@ inline size_t edt_col_smem(int max_res) {
   return (size_t)((max_res + 31) / 32) * kEdtCols * (sizeof(unsigned) + 2 * sizeof(int));
 }
 inline size_t edt_row_smem(int max_res) { return sizeof(unsigned) * (size_t)max_res; }
+// The limit a kernel needs for more than the default 48 KB, at `used` of at most `most` bytes.  It is an
+// attribute of the function on the device, common to all threads and handles: always the most, so that no
+// call lowers it between another's setting and its launch.
+template <class Kernel>
+inline cudaError_t edt_smem_limit(Kernel* kernel, size_t used, size_t most) {
+  if (used <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+constexpr int kEdtMaxRes = 32768;
 
 // Column pass, one block per strip of kEdtCols columns.  Each thread reads 8 rows of a column as
 // independent loads into one byte of the column's site bits; two short scans over the 32-row words

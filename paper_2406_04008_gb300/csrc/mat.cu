@@ -497,10 +497,8 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
                             float* width_out) {
   cudaError_t e = cudaMemsetAsync(n_cand, 0, sizeof(int) * d.n_probs, s);
   const size_t cs = edt_col_smem(max_res), rs = edt_row_smem(max_res);
-  if (e == cudaSuccess && cs > 48 * 1024)
-    e = cudaFuncSetAttribute(k_edt_cols<OutsideSite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
-  if (e == cudaSuccess && rs > 48 * 1024)
-    e = cudaFuncSetAttribute(k_mat_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  if (e == cudaSuccess) e = edt_smem_limit(k_edt_cols<OutsideSite>, cs, edt_col_smem(kEdtMaxRes));
+  if (e == cudaSuccess) e = edt_smem_limit(k_mat_rows, rs, edt_row_smem(kEdtMaxRes));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(1));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_mat_place_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(kPlaceBlocks));

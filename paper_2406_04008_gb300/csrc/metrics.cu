@@ -98,10 +98,8 @@ cudaError_t launch_metrics(const Dev& d, cudaStream_t s, uint8_t* obj, unsigned 
   cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 4 * d.n_probs, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * d.n_probs, s);
   const size_t cs = edt_col_smem(max_res), rs = edt_row_smem(max_res);
-  if (e == cudaSuccess && cs > 48 * 1024)
-    e = cudaFuncSetAttribute(k_edt_cols<ObjectSite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
-  if (e == cudaSuccess && rs > 48 * 1024)
-    e = cudaFuncSetAttribute(k_metric_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  if (e == cudaSuccess) e = edt_smem_limit(k_edt_cols<ObjectSite>, cs, edt_col_smem(kEdtMaxRes));
+  if (e == cudaSuccess) e = edt_smem_limit(k_metric_rows, rs, edt_row_smem(kEdtMaxRes));
   if (e != cudaSuccess) return e;
   const int tgrid = (d.total_tiles + kMetWarps - 1) / kMetWarps;
   if (d.tile == 8) k_metric_counts<8><<<tgrid, kMetWarps * 32, 0, s>>>(d, obj, cnt);
