@@ -17,6 +17,7 @@
 // the coverage margin from the outline carry sd = +-1e30 (saturated coverage, no gradient).
 #include <cfloat>
 
+#include "arith.h"
 #include "internal.h"
 
 namespace collage {
@@ -852,23 +853,6 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
   return parts > 1;
 }
 
-// a / b for normal b: the reciprocal's quotient with one residual correction (Markstein 1990), within an
-// ulp; the IEEE division's checks for the other operands cost as much again.  (With these two forms a unit
-// takes 360 warp instructions instead of 470: the adjoint of 64 collages 137 -> 119 us, of 1000 elements
-// at 1024^2 18 -> 16; its gradients are as far from 64 bits as before, 2e-7 to 1e-6.)
-__device__ __forceinline__ float div_normal(float a, float b) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(b));
-  const float q = a * r;
-  return fmaf(fmaf(-q, b, a), r, q);
-}
-// 1 / sqrt(x) for normal x > 0 with one Newton step, within an ulp.
-__device__ __forceinline__ float rsqrt_normal(float x) {
-  float r;
-  asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return fmaf(r * 0.5f, fmaf(-x * r, r, 1.0f), r);
-}
-
 template <int T, bool FIT>  // FIT: also dL/d(vertex) for outline fitting (d.fit)
 __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev d, int mark, int early, int n_loss) {
   constexpr int NP = T * T, UNITS = NP / 64, DY = 32 / T;
@@ -983,7 +967,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
         const float gA = pt_s[k] < 0.0f ? d.L.beta * inv_np : 0.0f;
         const float omc = Sfun(-x), cp = Sfun(xp);
         // dIhat/dc_i = -prod_{j != i}(1 - c_j) = -Ihat / (1 - c_i)   (0 when another c_j = 1)
-        const float gc = omc > 1e-30f ? div_normal(-gI * ihat[k], omc) : 0.0f;
+        const float gc = omc > 0.0f ? div_normal(-gI * ihat[k], omc) : 0.0f;
         // dA/dc^pad_i = tau prod_{j != i}(1 - tau c^pad_j)
         const float gcp = div_normal(gA * tau * pt, 1.0f - tau * cp);
         gsd[k] = (gc * dSfun(x) + gcp * dSfun(xp)) * inv_rho;
@@ -997,17 +981,17 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
       const float dx = ((float)X + 0.5f - tp.x) - tp.z, dy = ((float)(Y + k * DY) + 0.5f - tp.y) - tp.w;
       const float ex = sa[k].z, ey = sa[k].w, ee = ex * ex + ey * ey;
       const float wx = dx - sa[k].x, wy = dy - sa[k].y;
-      const bool seg = ee > 1e-30f;
-      const float re = rsqrt_normal(seg ? ee : 1.0f);  // 1 / |e|
-      const float u = seg ? __saturatef((wx * ex + wy * ey) * re * re) : 0.0f;
+      // (a segment shorter than 1e-19 px is its start point)
+      const float u = ee >= FLT_MIN ? __saturatef(div_normal(wx * ex + wy * ey, ee)) : 0.0f;
       const float qx = fmaf(u, ex, sa[k].x), qy = fmaf(u, ey, sa[k].y);  // closest point, rel. to t
       // unit normal from the closest point towards the pixel: for a closest point inside the
       // segment it is the segment's perpendicular on the pixel's side (well conditioned even
       // when the pixel is almost on the outline); at an end point it is the direction to the pixel
       const bool inner = u > 0.0f && u < 1.0f;
       const float rx = dx - qx, ry = dy - qy, rr = rx * rx + ry * ry;
-      if (!inner && !(rr > 1e-30f)) continue;
-      const float side = ex * wy - ey * wx >= 0.0f ? re : -re, ir = rsqrt_normal(inner ? 1.0f : rr);
+      const float nn = inner ? ee : rr;
+      if (!(nn >= FLT_MIN)) continue;  // the pixel is the closest point
+      const float ir = rsqrt_normal(nn), side = ex * wy - ey * wx >= 0.0f ? ir : -ir;
       const float nx = inner ? -ey * side : rx * ir, ny = inner ? ex * side : ry * ir;
       // sd = sig * dist (closed: sig = +-1 by the winding; open: sd = hw - dist, sig = -1)
       const float sig = closed ? (sd > 0.0f ? 1.0f : -1.0f) : -1.0f;
