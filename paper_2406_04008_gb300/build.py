@@ -17,7 +17,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libcollage.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libcollage_checked.so")
 SOURCES = ["api.cu", "bin.cu", "raster.cu", "loss.cu", "fit.cu", "mat.cu", "metrics.cu", "noalloc.cu", "peak.cu", "sched.cu"]
-HEADERS = ["arith.h", "edt.h", "internal.h", "route.h"]
+HEADERS = ["arith.h", "edt.h", "internal.h", "route.h", "trig.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off",
          "-I" + INCLUDE, "-I" + CSRC]

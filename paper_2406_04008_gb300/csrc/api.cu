@@ -14,6 +14,7 @@
 #include "collage.h"
 #include "internal.h"
 #include "route.h"
+#include "trig.h"
 
 #ifdef COLLAGE_CHECKED
 #include <nvtx3/nvToolsExt.h>
@@ -968,7 +969,7 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
     }
   }
   {
-    std::vector<float4> trig(kTrigSteps);
+    std::vector<float4> trig(kTrigSteps / 4 + 1);
     trig_table(trig.data());
     float4* p_trig;
     CKC(upload(h->owned, p_trig, trig));

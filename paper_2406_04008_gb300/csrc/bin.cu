@@ -8,6 +8,7 @@
 // so every tile lists its elements in increasing order whatever the order of the atomics.  The tile rectangle follows a fixed float formula
 // (bin_rect), so the bins are bit-exact against the oracle's rule.
 #include "internal.h"
+#include "trig.h"
 
 namespace collage {
 
@@ -39,7 +40,7 @@ __device__ int4 bin_rect(float4 q, float rbin, float hw, int res, int T, float r
 }
 
 // Vertex of an element relative to its translation, in pixels: (s res R(theta)) v.  The matrix is
-// formed in double once per element and split into float hi + lo parts; the per-vertex product uses
+// formed once per element as float hi + lo parts (csrc/trig.h); the per-vertex product uses
 // error-free transformations in float (FMA two-product and Knuth's two-sum, as in Ogita, Rump &
 // Oishi 2005), so the result is within about one float ulp of the exact value without FP64 work
 // per vertex (FP64 throughput is low on this part).  Explicit round-to-nearest intrinsics keep the
@@ -61,81 +62,6 @@ __device__ __forceinline__ float dot2_ff(const float (&a)[2], const float (&b)[2
 
 __device__ __forceinline__ float2 vertex_px(const float2 v, const RotFF& M) {
   return make_float2(dot2_ff(M.m[0], M.m[1], v.x, v.y), dot2_ff(M.m[2], M.m[3], v.x, v.y));
-}
-
-// Float pairs (hi + lo).  FP64 runs at 1/64 of the FP32 rate on this part, and one element's sine and
-// cosine in double were a dependent chain of about a hundred such instructions: 2 us of the
-// transform's 12 at 1000 elements, and most of its 100 at 26 k.  The pairs below carry 46
-// bits (|error| <= 2^-46 over |angle| <= 8192, measured), past the 2^-24 to which a vertex is rounded.
-// Sum a + b as hi + lo, exactly (Knuth); the second form needs |a| >= |b| or a = 0 (Dekker).
-__device__ __forceinline__ float two_sum(float a, float b, float& lo) {
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  lo = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return s;
-}
-__device__ __forceinline__ float fast_two_sum(float a, float b, float& lo) {
-  const float s = __fadd_rn(a, b);
-  lo = __fsub_rn(b, __fsub_rn(s, a));
-  return s;
-}
-// Product a b as hi + lo, exactly (FMA).
-__device__ __forceinline__ float two_prod(float a, float b, float& lo) {
-  const float p = __fmul_rn(a, b);
-  lo = __fmaf_rn(a, b, -p);
-  return p;
-}
-
-// Sine and cosine of an angle |z| <= kTrigMax as unevaluated float pairs.  z = k (2 pi / 1024) + x with
-// the step in three floats (Cody & Waite 1980) and the products and differences carried exactly, then
-// the angle sum of the tabled sin, cos of k (2 pi / 1024) with sin x = x - x^3/6 + x^5/120 and
-// cos x - 1 = -x^2/2 + x^4/24, |x| <= 0.0031, of which only the leading terms need the low part.
-constexpr float kTrigMax = 8192.0f;
-constexpr double kTrigStep = 6.283185307179586 / kTrigSteps;                // 2 pi / 1024
-constexpr double kTrigStepLow = 2.4492935982947064e-16 / kTrigSteps;  // ... beyond a double
-constexpr float kTrigC1 = (float)kTrigStep;
-constexpr float kTrigC2 = (float)(kTrigStep - (double)kTrigC1);
-constexpr float kTrigC3 = (float)(kTrigStep - (double)kTrigC1 - (double)kTrigC2 + kTrigStepLow);
-
-// One of the pair: T + A x' + B y', with T, A the tabled values (hi, lo), x' = sin x (xh + xl) and
-// y = cos x - 1 (yh + yl) multiplying T: sin(k + x) = S + C sin x + S (cos x - 1), and so on.
-__device__ __forceinline__ float trig_sum(float th, float tl, float ah, float al, float xh, float xl, float yh,
-                                          float yl, float& lo) {
-  float e1, e2, f1, f2;
-  const float p1 = two_prod(ah, xh, e1), p2 = two_prod(th, yh, e2);
-  const float s1 = two_sum(th, p1, f1);
-  const float s2 = two_sum(s1, p2, f2);
-  const float rest = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), __fadd_rn(f1, f2)),
-                               __fmaf_rn(ah, xl, __fmaf_rn(al, xh, __fmaf_rn(th, yl, __fmaf_rn(tl, yh, tl)))));
-  return fast_two_sum(s2, rest, lo);
-}
-
-__device__ __forceinline__ void sincos_ff(float z, const float4* table, float (&s)[2], float (&c)[2]) {
-  const float k = rintf(__fmul_rn(z, 1.0f / kTrigC1));
-  const float4 t = table[(int)k & (kTrigSteps - 1)];  // sin hi, lo, cos hi, lo
-  float e, q, b, dd;
-  const float p = two_prod(k, kTrigC1, e);
-  const float u = two_prod(k, kTrigC2, q);
-  const float a1 = two_sum(__fsub_rn(z, p), -e, b);  // z - p is exact: p is within a factor 2 of z
-  const float a2 = two_sum(a1, -u, dd);
-  float xl;
-  const float xh = fast_two_sum(a2, __fsub_rn(__fadd_rn(b, dd), __fmaf_rn(k, kTrigC3, q)), xl);
-  float y2l;
-  const float y2 = two_prod(xh, xh, y2l);
-  y2l = __fmaf_rn(2.0f * xh, xl, y2l);
-  // sin x beyond its leading term x, cos x - 1 beyond -x^2/2
-  const float sl = __fmaf_rn(__fmul_rn(xh, y2), __fmaf_rn(y2, 1.0f / 120.0f, -1.0f / 6.0f), xl);
-  const float yl = __fmaf_rn(__fmul_rn(y2, y2), 1.0f / 24.0f, -0.5f * y2l);
-  s[0] = trig_sum(t.x, t.y, t.z, t.w, xh, sl, -0.5f * y2, yl, s[1]);
-  c[0] = trig_sum(t.z, t.w, -t.x, -t.y, xh, sl, -0.5f * y2, yl, c[1]);
-}
-
-__device__ __noinline__ void sincos_wide(float z, float (&s)[2], float (&c)[2]) {  // any other angle
-  double sn, cs;
-  sincos((double)z, &sn, &cs);
-  s[0] = (float)sn;
-  s[1] = (float)(sn - (double)s[0]);
-  c[0] = (float)cs;
-  c[1] = (float)(cs - (double)c[0]);
 }
 
 // E = 1 or 4 elements per block: the pending Adam step of the previous iteration, then segment records
@@ -216,19 +142,10 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     const float z = __shfl_sync(0xffffffffu, x, 2, 4), sc = __shfl_sync(0xffffffffu, x, 3, 4);
     if (writer) {
       reinterpret_cast<float*>(&s_q[e])[k] = x;
-      float s[2], c[2];
-      if (fabsf(z) <= kTrigMax) sincos_ff(z, d.trig, s, c);
-      else sincos_wide(z, s, c);
       // entry k of s res [cos, -sin; sin, cos]
-      float th = k == 0 || k == 3 ? c[0] : s[0], tl = k == 0 || k == 3 ? c[1] : s[1];
-      if (k == 1) {
-        th = -th;
-        tl = -tl;
-      }
-      float hl, pl, lo;
-      const float hh = two_prod(sc, (float)re, hl), pp = two_prod(hh, th, pl);
-      s_rot[e].m[k][0] = fast_two_sum(pp, __fadd_rn(pl, __fmaf_rn(hh, tl, __fmul_rn(hl, th))), lo);
-      s_rot[e].m[k][1] = lo;
+      const float f = k == 1 ? -sc : sc;
+      if (fabsf(z) <= kTrigMax) trig_entry(z, k == 0 || k == 3, f, (float)re, d.trig, s_rot[e].m[k]);
+      else trig_wide(z, k == 0 || k == 3, f, (float)re, s_rot[e].m[k]);
     }
   }
   __syncthreads();
@@ -313,13 +230,6 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     float lx, ly;
     const float hx = two_prod(q.x, (float)res, lx), hy = two_prod(q.y, (float)res, ly);
     d.tpx[g] = make_float4(hx, hy, lx, ly);
-  }
-}
-
-void trig_table(float4* t) {
-  for (int k = 0; k < kTrigSteps; ++k) {
-    const double a = k * (6.283185307179586 / kTrigSteps), s = sin(a), c = cos(a);
-    t[k] = make_float4((float)s, (float)(s - (double)(float)s), (float)c, (float)(c - (double)(float)c));
   }
 }
 

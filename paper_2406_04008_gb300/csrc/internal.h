@@ -19,7 +19,7 @@
 namespace collage {
 
 constexpr int kMaxDil = 8;
-constexpr int kTrigSteps = 1024;        // angles of the transform's table
+constexpr int kTrigSteps = 4096;        // steps to a turn of the transform's table of sines
 constexpr int kLossUnits = 2048;        // 64-px units of an image per part of its loss,
 constexpr int kLossParts = 16;          //   in at most this many parts
 constexpr int kCtlWords = 24;           // device control words (status first, see Dev)
@@ -92,7 +92,7 @@ struct Dev {
   const float4* q_in;           // [n] params the transform takes in place of q (the host-buffer
                                 //   step's mapped input), or null
   const uchar4* trainable;      // may be null
-  const float4* trig;           // [kTrigSteps] sin (hi, lo), cos (hi, lo) of k (2 pi / kTrigSteps)
+  const float4* trig;           // [kTrigSteps / 4 + 1] sines of k (2 pi / kTrigSteps), in three floats each
   float lr, b1, b2, eps, s_min, s_max;
   // ---- per iteration ----
   float4* segA;                 // [V] segment k: start (px, relative to the translation), direction
@@ -326,7 +326,6 @@ __device__ __forceinline__ void mark_step_if_last(const Dev& d) {
 }
 
 // ---- launchers (each enqueues on `s`, returns the launch error) ----
-void trig_table(float4* t);  // host: fills the table of Dev::trig
 // follows: the previous launch on `s` is another iteration's, so the outlines were written long before
 // and are read while it ends (never the first launch after a call that may replace them)
 cudaError_t launch_transform(const Dev& d, cudaStream_t s, bool zero_grad, bool follows);

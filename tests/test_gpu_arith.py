@@ -1,5 +1,6 @@
-"""csrc/arith.h against IEEE arithmetic, to the bounds it states: every significand of the divisor and of the
-root's argument, over the exponents for which the bounds hold."""
+"""csrc/arith.h and csrc/trig.h to the bounds they state: quotients and reciprocal roots against IEEE
+arithmetic, over every significand of the divisor and of the root's argument and the exponents for which
+the bounds hold; rotation entries against longer arithmetic."""
 import ctypes as C
 import subprocess
 
@@ -78,3 +79,62 @@ def test_reciprocal_roots(arith, e):
         y, ref = arith(2, None, x).astype(np.float64), 1.0 / np.sqrt(x.astype(np.float64))
         ulp = np.ldexp(1.0, np.floor(np.log2(ref)).astype(int) - 23)
         assert (np.abs(y - ref) <= 0.51 * ulp).all()
+
+
+TRIG = """
+#include <vector>
+#include "trig.h"
+__global__ void k(const float* z, const float* a, float b, const float4* t, float2* s, float2* c, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float m[2];
+  collage::trig_entry(z[i], false, a[i], b, t, m);
+  s[i] = make_float2(m[0], m[1]);
+  collage::trig_entry(z[i], true, a[i], b, t, m);
+  c[i] = make_float2(m[0], m[1]);
+}
+extern "C" int trig(const float* z, const float* a, float b, float2* s, float2* c, int n) {
+  std::vector<float4> h(collage::kTrigSteps / 4 + 1);
+  collage::trig_table(h.data());
+  float4* t;
+  if (cudaMalloc(&t, sizeof(float4) * h.size())) return 1;
+  cudaMemcpy(t, h.data(), sizeof(float4) * h.size(), cudaMemcpyHostToDevice);
+  k<<<(n + 255) / 256, 256>>>(z, a, b, t, s, c, n);
+  const int e = cudaDeviceSynchronize();
+  cudaFree(t);
+  return e;
+}
+"""
+
+
+@pytest.mark.parametrize("b", [1.0, 200.0, 1024.0, 32767.0])  # (a resolution: a float is exact)
+def test_rotation_entries_as_exact_as_a_split_double(build_so, b):
+    # each entry a b sin z, a b cos z is within half a unit of its low part (2^-48 of a b; the reference and its
+    # split add 2^-52), and no further from the exact value on average than the FP64 value split into a pair
+    f = build_so(TRIG).trig
+    f.argtypes = [C.c_void_p, C.c_void_p, C.c_float, C.c_void_p, C.c_void_p, C.c_int]
+    rng = np.random.default_rng(int(b))
+    k = rng.integers(-5300000, 5300000, 1 << 16).astype(np.float64)
+    mid = (k * (2 * np.pi / 4096)).astype(np.float32)  # beside the table's angles, and half a step from them
+    half = ((k + 0.5) * (2 * np.pi / 4096)).astype(np.float32)
+    z = np.concatenate([
+        mid, half, rng.uniform(-8192, 8192, 1 << 17).astype(np.float32), rng.uniform(-7, 7, 1 << 17).astype(np.float32),
+        (10.0 ** rng.uniform(-30, 0, 1 << 15)).astype(np.float32), np.float32(np.pi / 2 * np.arange(-5200, 5200)),
+        np.float32([0.0, -0.0, 8192.0, -8192.0, 8191.9995])])
+    z = z[np.abs(z) <= 8192]
+    a = np.exp(rng.uniform(-3, 3, len(z))).astype(np.float32)
+    zt, at = torch.from_numpy(z).cuda(), torch.from_numpy(a).cuda()
+    s, c = (torch.empty(len(z), 2, device="cuda") for _ in range(2))
+    torch.cuda.synchronize()
+    assert f(zt.data_ptr(), at.data_ptr(), b, s.data_ptr(), c.data_ptr(), len(z)) == 0
+    assert np.finfo(np.longdouble).nmant >= 63
+    ab = a.astype(np.longdouble) * np.longdouble(b)
+    for got, fn in ((s, np.sin), (c, np.cos)):
+        exact = ab * fn(z.astype(np.longdouble))
+        double = a.astype(np.float64) * b * fn(z.astype(np.float64))
+        hi = double.astype(np.float32)
+        split = hi.astype(np.longdouble) + (double - hi).astype(np.float32)
+        m = got.cpu().numpy().astype(np.longdouble)
+        err, ref = ((v - exact) / ab for v in (m[:, 0] + m[:, 1], split))
+        assert np.abs(err).max() <= 2.0 ** -48
+        assert np.sqrt((err ** 2).mean()) <= np.sqrt((ref ** 2).mean())
