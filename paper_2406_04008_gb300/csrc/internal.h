@@ -243,10 +243,23 @@ __device__ __forceinline__ float force_potential(const LossParams& L, float px, 
 // ---- programmatic dependent launch ----
 // With Dev::pdl set, the kernels of an iteration are launched with programmatic stream
 // serialisation: a kernel may be scheduled while its predecessor on the stream still runs.  Every
-// such kernel starts with pdl_enter(): griddepcontrol.wait returns once the predecessor grid has
-// completed and its memory operations are visible (before any global access or early return, so
-// completion stays transitive along the chain), then launch_dependents lets the successor be
-// scheduled.  Launched without the attribute, both instructions are no-ops.
+// thread of such a kernel calls pdl_enter() before it ends: griddepcontrol.wait returns once the
+// predecessor grid has completed and its memory operations are visible, then launch_dependents lets
+// the successor be scheduled (the wait comes first in every thread, so completion is transitive along
+// the chain: when a kernel starts, all but its predecessor have completed).  Launched without the
+// attribute, both instructions are no-ops.
+//
+// What a kernel K_n may touch before its own wait:
+//  1. memory that no kernel of an iteration writes: the problem, the level's tables, the container
+//     raster and the dilation tiles' lists.  They change only in work that the host separates from
+//     iterations (create, a level switch, replaced outlines), and a launch that may follow such work
+//     directly does not read them early (`follows` of the transform);
+//  2. what K_{n-2} or an earlier kernel wrote and K_{n-1} does not write, by accesses that L2 serves:
+//     atomics (the counts of balanced_slot) or __ldcg loads (the adjoint).  Those kernels have completed
+//     and their writes lie in L2, but only the wait is documented to make a grid's writes visible to
+//     ordinary loads, which may hit a line that this SM's L1 kept from an earlier iteration;
+//  3. nothing else: no store before the wait except to what only K_n itself writes and reads in this
+//     iteration (the loss terms and their parts).
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

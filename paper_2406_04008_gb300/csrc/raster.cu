@@ -761,8 +761,10 @@ __global__ void __launch_bounds__(kCompWarps * 32) k_empty_loss(Dev d) {
 // The grid's first blocks, one per problem or more, assemble the loss instead: its partials are complete,
 // and the work (a read of 16 B per unit) fits beside the adjoint's round trips without a launch, a second
 // stream and the two joins that the end of an iteration waited for.
-// What the kernels before the predecessor wrote is read before the predecessor has completed: the work
-// list, the saved distances and, when the distribution term's adjoint is the predecessor, the images.
+// Where the distribution term's adjoint is the predecessor, what the kernels before that one wrote (the
+// work list, the transforms, the saved distances and segments, the images, the loss partials) is read
+// while it drains, from L2 (pdl_enter's second rule): 100 outlines at 1000^2 52.0 us an iteration instead of
+// 55.2, 200 blobs at 512^2 43.1 instead of 45.7.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ float warp_sum_f(float x) {
   for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -794,7 +796,7 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
   for (int t = t0 + (int)threadIdx.x; t < t1; t += NT * ACC)
 #pragma unroll
     for (int k = 0; k < ACC; ++k) {
-      const float4 v = t + k * NT < t1 ? d.lossA[t + k * NT] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 v = t + k * NT < t1 ? __ldcg(&d.lossA[t + k * NT]) : make_float4(0.f, 0.f, 0.f, 0.f);
       a[k] += v.x;
       b[k] += v.y;
       c[k] += v.z;
@@ -808,7 +810,7 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
     }
     for (int t = u0 + (int)threadIdx.x; t < u1; t += NT * ACC)
 #pragma unroll
-      for (int k = 0; k < ACC; ++k) u[k] += t + k * NT < u1 ? d.lossU[t + k * NT] : 0.0f;
+      for (int k = 0; k < ACC; ++k) u[k] += t + k * NT < u1 ? __ldcg(&d.lossU[t + k * NT]) : 0.0f;
   }
   auto sum = [](float (&x)[ACC]) {
     return warp_sum_f(((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7])));
@@ -857,7 +859,7 @@ template <int T, bool FIT>  // FIT: also dL/d(vertex) for outline fitting (d.fit
 __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev d, int mark, int early, int n_loss) {
   constexpr int NP = T * T, UNITS = NP / 64, DY = 32 / T;
   if ((int)blockIdx.x < n_loss) {
-    const bool ok = !(*d.status & kStatusNoBins);
+    const bool ok = !(__ldcg(d.status) & kStatusNoBins);
     int p = blockIdx.x, part = 0, per = 1;  // blocks per problem
     if (n_loss > d.n_probs) {
       per = n_loss / d.n_probs;
@@ -878,20 +880,20 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int stride = ((int)gridDim.x - n_loss) * kPairWarps;
   int i = ((int)blockIdx.x - n_loss) * kPairWarps + wid;
-  if (*d.status & kStatusNoBins) {
+  if (__ldcg(d.status) & kStatusNoBins) {
     pdl_enter();
     return;
   }
-  const int n_live = min(d.work[1], d.cap * UNITS);  // units without a gradient-carrying pixel are not listed
+  const int n_live = min(__ldcg(&d.work[1]), d.cap * UNITS);  // units without a gradient-carrying pixel are not listed
   bool waited = false;
   auto wait = [&]() {
     if (!waited) pdl_enter();
     waited = true;
   };
-  int4 rec = i < n_live ? d.live_list[i] : make_int4(0, 0, 0, 0);
+  int4 rec = i < n_live ? __ldcg(&d.live_list[i]) : make_int4(0, 0, 0, 0);
   for (; i < n_live; i += stride) {
     // the next unit's record is read while this one is worked on
-    const int4 rec_next = i + stride < n_live ? d.live_list[i + stride] : rec;
+    const int4 rec_next = i + stride < n_live ? __ldcg(&d.live_list[i + stride]) : rec;
     const int slot = rec.x & (int)kSlotMask, unit = (int)((unsigned)rec.x >> kSlotBits), g = rec.y, txy = rec.z, p = rec.w;
     if (!in_bounds(d, slot >= 0 && slot < d.cap && g >= 0 && g < d.n_elems && p >= 0 && p < d.n_probs)) {
       rec = rec_next;
@@ -901,8 +903,8 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
     const float inv_np = 1.0f / ((float)res * (float)res);
     const int v0 = d.elem_voff[g];
     const bool closed = d.elem_closed[g] != 0;
-    const float4 tp = d.tpx[g];
-    const float4 qg = d.q[g];
+    const float4 tp = __ldcg(&d.tpx[g]);
+    const float4 qg = __ldcg(&d.q[g]);
     const float s_inv = 1.0f / qg.w;
     // the lane's pixels: one column, rows Y and Y + DY
     const int X = (txy & 0xffff) * T + lane % T, Y = (txy >> 16) * T + unit * (64 / T) + lane / T;
@@ -926,9 +928,9 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
       ihat[k] = pt_s[k] = cov[k] = gou[k] = 0.0f;
       if (X < res && Y + k * DY < res) {
         const long long pix = pix0 + k * DY * res;
-        srec[k] = sv[32 * k];
-        ihat[k] = d.img_I[pix];
-        pt_s[k] = d.img_Pt[pix];
+        srec[k] = __ldcg(&sv[32 * k]);
+        ihat[k] = __ldcg(&d.img_I[pix]);
+        pt_s[k] = __ldcg(&d.img_Pt[pix]);
         cov[k] = d.covc[pix];
       }
     }
@@ -942,7 +944,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
       act[k] = fabsf(sd * inv_rho) < 1.0f || fabsf((sd + pad) * inv_rho) < 1.0f;
       if (act[k] && !in_bounds(d, (unsigned)__float_as_int(srec[k].y) < (unsigned)(d.elem_voff[g + 1] - v0)))
         act[k] = false;
-      if (act[k]) sa[k] = d.segA[v0 + __float_as_int(srec[k].y)];
+      if (act[k]) sa[k] = __ldcg(&d.segA[v0 + __float_as_int(srec[k].y)]);
     }
     wait();
     if (use_u)
