@@ -98,6 +98,7 @@ struct collage_s {
   int grad_calls = 0;                    // such passes since the level was set up or a buffer moved
   cudaGraphExec_t sched = nullptr;  // the schedule from level sched_start to the last
   int sched_start = -1;
+  float* grad_out = nullptr;  // [4N] gradient on its way to a buffer that no kernel takes
   // quality-metric scratch (allocated by collage_metrics)
   uint8_t* met_obj = nullptr;
   unsigned short* met_gcol = nullptr;
@@ -990,8 +991,9 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(dmalloc(h->owned, d.segS, h->V));
   CKC(dmalloc(h->owned, d.tpx, h->N));
   CKC(dmalloc(h->owned, d.rect, h->N));
-  CKC(dmalloc(h->owned, d.dq, h->N));
-  CKC(cudaMemset(d.dq, 0, sizeof(float4) * h->N));
+  CKC(dmalloc(h->owned, d.dq, 4 * (size_t)h->N));
+  CKC(cudaMemset(d.dq, 0, sizeof(double) * 4 * h->N));
+  CKC(dmalloc(h->owned, h->grad_out, 4 * (size_t)h->N));
   CKC(dmalloc(h->owned, d.loss_terms, 5 * h->P));
   CKC(cudaMemset(d.loss_terms, 0, sizeof(float) * 5 * h->P));
   CKC(dmalloc(h->owned, d.loss_part, (size_t)h->P * kLossParts));
@@ -1080,13 +1082,13 @@ extern "C" collage_status collage_loss_backward(collage_t h, void* stream, float
   cudaStream_t s = (cudaStream_t)stream;
   collage_status st = run_checked(h, s, kLossBwd, nullptr, nullptr);
   if (st) return st;
-  float* k_terms = own_memory(h, d_loss_terms) ? d_loss_terms : nullptr;
-  float* k_grad = own_memory(h, d_dparams) ? d_dparams : nullptr;
-  if (k_terms || k_grad) CK(h, launch_copy_out(h->d, s, k_terms, k_grad));
-  if (d_loss_terms && !k_terms)
+  const bool own_terms = own_memory(h, d_loss_terms), own_grad = own_memory(h, d_dparams);
+  float* k_grad = !d_dparams || own_grad ? d_dparams : h->grad_out;
+  if (own_terms || k_grad) CK(h, launch_copy_out(h->d, s, own_terms ? d_loss_terms : nullptr, k_grad));
+  if (d_loss_terms && !own_terms)
     CK(h, cudaMemcpyAsync(d_loss_terms, h->d.loss_terms, sizeof(float) * 5 * h->P, cudaMemcpyDeviceToDevice, s));
-  if (d_dparams && !k_grad)
-    CK(h, cudaMemcpyAsync(d_dparams, h->d.dq, sizeof(float4) * h->N, cudaMemcpyDeviceToDevice, s));
+  if (d_dparams && !own_grad)
+    CK(h, cudaMemcpyAsync(d_dparams, h->grad_out, sizeof(float4) * h->N, cudaMemcpyDeviceToDevice, s));
   return COLLAGE_OK;
 }
 

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     const bool step = *d.pending && !d.fit;
     if (step) {
       float m = reinterpret_cast<const float*>(d.m + ge)[k], v = reinterpret_cast<const float*>(d.v + ge)[k];
-      const float gr = reinterpret_cast<const float*>(d.dq + ge)[k];
+      const float gr = (float)d.dq[4 * (size_t)ge + k];
       const bool tr = !d.trainable || reinterpret_cast<const unsigned char*>(d.trainable + ge)[k];
       const float pw = powf((lane & 4) ? d.b2 : d.b1, (float)*d.step);
       const AdamScale a = adam_scale(d, __shfl_sync(0xffffffffu, pw, 0), __shfl_sync(0xffffffffu, pw, 4));
@@ -162,7 +162,10 @@ __global__ void __launch_bounds__(kTfThreads) k_transform(Dev d, int zero_grad, 
     else if (lane == 0) atomicOr(d.status, kStatusBadParam);
     if (lane == 0) {
       d.rect[g] = r;
-      if (zero_grad) d.dq[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (zero_grad) {
+        double2* dq = reinterpret_cast<double2*>(d.dq + 4 * (size_t)g);
+        dq[0] = dq[1] = make_double2(0.0, 0.0);
+      }
     }
     if (r.z >= r.x && r.w >= r.y) {
       // the pair slots of the rectangle; beyond the capacity the bins of the iteration are void

@@ -140,7 +140,8 @@ struct Dev {
                                 //   from 0, with coverage within the halo from total_dtiles, in no
                                 //   particular order (or null: all tiles)
   int* dtile_n;                 // [2] lengths of the two lists
-  float4* dq;                   // [n] gradient
+  double* dq;                   // [4n] gradient, summed in FP64: the adjoint's units add to it in whatever order
+                                //   they end, which FP32 sums showed in their last bits
   float4* partial;              // [cap * units per tile] deterministic gradient partials, by slot
   float* loss_terms;            // [P*5]
   float4* loss_part;            // [P * kLossParts] the sums over each part of a problem's loss partials

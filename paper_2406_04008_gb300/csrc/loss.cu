@@ -469,7 +469,11 @@ __global__ void __launch_bounds__(kReduceWarps * 32) k_grad_reduce(Dev d, int ma
       acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
       acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
     }
-    if (lane == 0) d.dq[g] = acc;
+    if (lane == 0) {
+      double2* dq = reinterpret_cast<double2*>(d.dq + 4 * (size_t)g);
+      dq[0] = make_double2((double)acc.x, (double)acc.y);
+      dq[1] = make_double2((double)acc.z, (double)acc.w);
+    }
   }
   if (mark) mark_step_if_last(d);
 }
@@ -482,7 +486,10 @@ __global__ void k_adam_flush(Dev d, float* out, const float4* q_in, float4* q_ou
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const bool pend = *d.pending != 0;
   if (g < d.n_elems) {
-    if (pend && !d.fit) adam_update(d, g, *d.step, d.dq[g]);
+    if (pend && !d.fit) {
+      const double* dq = d.dq + 4 * (size_t)g;
+      adam_update(d, g, *d.step, make_float4((float)dq[0], (float)dq[1], (float)dq[2], (float)dq[3]));
+    }
     if (q_in) d.q[g] = q_in[g];
     if (q_out) q_out[g] = d.q[g];
     if (out) reinterpret_cast<float4*>(out)[g] = d.q[g];
@@ -585,7 +592,7 @@ cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out, const fl
 // launch for both.
 __global__ void k_copy_out(Dev d, float* terms, float* grad) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (grad && i < 4 * (size_t)d.n_elems) grad[i] = reinterpret_cast<const float*>(d.dq)[i];
+  if (grad && i < 4 * (size_t)d.n_elems) grad[i] = (float)d.dq[i];
   if (terms && i < 5 * (size_t)d.n_probs) terms[i] = d.loss_terms[i];
 }
 

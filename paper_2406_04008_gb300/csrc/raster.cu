@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
     for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((lane & 7) == 0) {
       if (d.deterministic) reinterpret_cast<float*>(d.partial + (size_t)slot * UNITS + unit)[lane >> 3] = v;
-      else atomicAdd(reinterpret_cast<float*>(d.dq + g) + (lane >> 3), v);
+      else atomicAdd(d.dq + 4 * (size_t)g + (lane >> 3), (double)v);
     }
     rec = rec_next;
   }
