@@ -270,10 +270,10 @@ __device__ __forceinline__ void pdl_enter() {
 // Blocks that are launched while the predecessor drains go to whichever SM has room: one SM takes eight
 // consecutive blocks of the emission and another none (1000 elements at 1024^2: the 602 long outlines, first
 // in the list, lay on 86 of 152 SMs), and an SM that is free early takes up to 18 of the distribution term's
-// one-tile blocks, a mean of 6.7.  Where all blocks of a grid are resident at once, each takes its item by
-// its rank among the blocks on its own SM instead: the r-th block of an SM takes the next of items
+// one-tile blocks, a mean of 6.7.  Where the items are few for the SMs (the callers' limits), each block takes
+// its item by its rank among the blocks on its own SM instead: the r-th block of an SM takes the next of items
 // [r n_sm, (r + 1) n_sm), so that each SM gets an even share of the front of the list, and the grid's idle
-// rest lies on the SMs with the most blocks.  A block whose range is spent takes the last free item; as there
+// rest lies on the SMs with the most blocks (resident at once or not: a later block ranks behind).  A block whose range is spent takes the last free item; as there
 // are as many items as blocks, each item is taken exactly once whatever the placement.  Runs before the wait
 // on the predecessor (`c` has been zero since the predecessor's predecessor or earlier), so that its two
 // atomics are hidden; one thread of each block calls it once.  Per iteration: 1000 elements at 1024^2 86.9 ->

@@ -199,6 +199,15 @@ struct IIGeom {
   static_assert(P % 2 == 1, "odd row stride");
 };
 
+// Listed tiles per SM up to which the blocks take theirs by rank on their SM, whatever the number of kernels
+// (and so of resident blocks).  Up to there the blocks of the front of the list crowd onto some SMs; beyond, most
+// SMs have as many as they hold anyway and the two atomics cost more.  Iterations with the limit at 0 (by
+// index), 3, 4, 5 and 8 (us; K = 4 where not said): the star at 700^2 45.1, 43.0, 43.1, 43.1, 43.1, at 1000^2 52.7,
+// 50.8, 50.6, 50.4, 50.5 (K = 8: 74.0, 72.6, 73.0, 72.9, 72.8); the annulus at 850^2 52.5, 52.5, 51.5, 51.4, 51.2, at
+// 1000^2 62.9, 62.8, 63.0, 63.2, 63.3 (K = 1: 55.7, 55.8, 55.8, 57.6, 57.7; K = 8: 87.9, 88.0, 88.1, 87.9, 90.4);
+// the open rectangle at 1000^2 76.0, 76.0, 75.9, 76.0, 77.1 (K = 8: 105.0, 105.1, 105.0, 105.1, 107.5).
+constexpr int kBalanced = 4;
+
 template <int K>
 __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d, int n_sm) {
   constexpr int S = DilGeom<K>::S, P = IIGeom<K>::P, h = DilGeom<K>::h, Q = DilGeom<K>::Q;
@@ -209,8 +218,8 @@ __global__ void __launch_bounds__(kDThreads, 5) k_dilate_fwd(Dev d, int n_sm) {
   // the tiles with container coverage; on the others M_C (1 - O) = 0, dL_u/dO = 0 and the loss
   // partial is 0, as written once per level.  The lists and the coverage are the level's: the first
   // tile's place and coverage are read before the composite has completed.
-  const int first = first_item(d.slots + kSlotInts, n_sm);
   const int n_own = dil_count(d, 0);
+  const int first = first_item(d.slots + kSlotInts, n_own <= kBalanced * n_sm ? n_sm : 0);
   DilTile t{};
   if (first < n_own) t = dil_place(d, 0, first);
   // the thread's output item: column c, rows r0..r0 + kVRows - 1
@@ -333,8 +342,8 @@ __global__ void __launch_bounds__(kDThreads, 6) k_dilate_bwd(Dev d, int n_sm) {
   uint32_t* H = sM + S * SP;
   // the tiles with container coverage within the halo (G = 0 over the others and their halos); the
   // first one's place is read before the forward pass has completed
-  const int first = first_item(d.slots + 2 * kSlotInts, n_sm);
   const int n_halo = dil_count(d, 1);
+  const int first = first_item(d.slots + 2 * kSlotInts, n_halo <= kBalanced * n_sm ? n_sm : 0);
   DilTile t{};
   if (first < n_halo) t = dil_place(d, 1, first);
   pdl_enter();
@@ -551,7 +560,7 @@ cudaError_t prepare_dilate(int n_dil) {
 template <int K>
 static cudaError_t launch_k(const Dev& d, cudaStream_t s, bool backward) {
   const size_t sm = dilate_smem(K, backward);
-  // one tile a block: balanced while the blocks fit the SMs at once; beyond, later blocks even the load out
+  // one tile a block
   const int n_sm = slot_sms(d, d.total_dtiles, 8);
   if (backward) return klaunch(d.pdl, k_dilate_bwd<K>, d.total_dtiles, kDThreads, sm, s, d, n_sm);
   return klaunch(d.pdl, k_dilate_fwd<K>, d.total_dtiles, kDThreads, sm, s, d, n_sm);
