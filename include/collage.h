@@ -254,9 +254,10 @@ collage_status collage_get_bins(collage_t h, void* stream, int* d_tile, int* d_e
 #define COLLAGE_STAGE_ADAM 8      /* (empty: the Adam step is applied by the next transform) */
 collage_status collage_stage_times(collage_t h, void* stream, int n_iters, float* h_ms);
 
-/* A launch configuration of the iteration's kernels, as the autotuner chooses it.  Until one is chosen
- * or set, emit_threads and chunk_px follow the work of each level (128 threads and 64 px where the
- * elements fill the device). */
+/* A launch configuration of the iteration's kernels, as the autotuner chooses it.  emit_threads and
+ * chunk_px follow the work of each level (128 threads and 64 px where the elements fill the device),
+ * except at a level where a search found another shape faster; collage_set_tuning sets them for every
+ * level. */
 typedef struct {
   int tile;              /* raster tile side, 8 or 16 */
   int emit_threads;      /* threads per block of the emission / signed-distance kernel: 128, 256 */
@@ -265,15 +266,16 @@ typedef struct {
   float fwd_grid;        /* persistent grids of the emission, adjoint and composite kernels, as */
   float bwd_grid;        /*   multiples of (SM count x blocks resident per SM): 0.5, 1 or 2 */
   float comp_grid;
-  float default_ms;      /* loss + gradient iteration time of the defaults (tile 16, 128 threads,
-                            64-px chunks, grids x1), ms; 0 when the choice came from the cache */
+  float default_ms;      /* loss + gradient iteration time of the defaults (tile 16, the emission's
+                            shape by the level's work, grids x1), ms; 0 when the choice came from the
+                            cache */
   float best_ms;         /* iteration time of the chosen configuration, ms */
   int trials;            /* configurations timed */
   int from_cache;        /* 1: the choice of an earlier search with the same key was reused */
 } collage_tuning;
 
 /* The autotuner (no counterpart in the paper): at the current level, times the raster tile sizes
- * with the other parameters at their defaults, then in turn the emission block size, the
+ * with the other parameters as an untuned handle has them, then in turn the emission block size, the
  * emission's chunk side and the persistent-grid multiples of the emission, adjoint and composite
  * kernels (each candidate a
  * captured one-iteration graph of loss and gradient, no Adam step, the fastest of three batches of
@@ -281,7 +283,8 @@ typedef struct {
  * scratch buffer the call allocates and frees), and keeps the fastest; a launch parameter other than the tile changes only
  * when its candidate is more than 3% faster.  The choice is cached for the process, keyed on (pixels of the level, element
  * count, pair density in half-octaves, deterministic mode); a handle with the same key reuses it
- * without a search.  One configuration serves the whole handle (every problem of a batch).
+ * without a search.  Tile and grids serve the whole handle (every level and every problem of a batch),
+ * the emission's shape the current level.
  * h_best_ms (may be NULL) receives the chosen configuration's iteration time.  Params and Adam
  * state are not changed (a pending Adam step is applied as the next iteration would).
  * Synchronises the device; drops captured graphs.  On failure the previous configuration is

@@ -28,6 +28,15 @@ thread_local std::string g_create_error;
 
 enum Mode { kRender = 0, kLossBwd = 1, kStep = 2 };
 
+// The emission's shape as the caller set it (at every level) or a search chose it (at its level); elsewhere
+// it follows the level's work (choose_emission).
+struct EmissionPin {
+  static constexpr int kNone = -1, kEvery = -2;
+  int level = kNone;
+  int threads = 128, chunk_px = kChunkPx;
+  bool at(int l) const { return level == kEvery || level == l; }
+};
+
 }  // namespace
 
 struct collage_s {
@@ -69,8 +78,7 @@ struct collage_s {
   // launch configuration (the autotuner's choice): persistent grids are these multiples of the SM
   // count x resident blocks per SM
   float fwd_mult = 1.0f, bwd_mult = 1.0f, comp_mult = 1.0f;
-  bool tuned = false;  // the configuration was searched or set by the caller; else the emission's block
-                       // and chunk sizes follow each level's work (choose_emission)
+  EmissionPin pin;  // the emission's block and chunk sizes where they do not follow the level's work
   std::vector<int> lv_chunks;  // 64-px chunks of each level when it was last probed
   collage_tuning tuning{};
   // device memory
@@ -525,19 +533,26 @@ static cudaError_t enqueue_level_switch(const Dev& d, cudaStream_t s) {
   return e;
 }
 
-// The emission's block and chunk sizes for a level of `chunks` 64-px chunks, where the caller chose
-// none.  A chunk is one block's work, and its phases are a chain: with fewer chunks than the device holds
-// blocks (eight of 128 threads per SM), smaller chunks or wider blocks put the idle warps to work; with
-// enough of them the extra staging only costs issue slots.  Measured per iteration (us; 128/64, 128/32,
-// 256/64, 256/32 threads/px): 120 chunks 55.9, 56.2, 54.3, 52.0; 200 chunks 64.2, 54.4, 56.4, 58.4; 400
-// chunks (of 320 segments) 88.4, 70.8, 77.0, 73.8; 500 chunks 74.8, 72.8, 67.1, 72.3; 1000 chunks 92.7,
-// 95.7, 90.7, 100.4; 5000 chunks 398.8, 444.4, 432.3, 547.8.
-static void choose_emission(collage_t h, int chunks) {
-  h->d.few_chunks = chunks <= 8 * h->sms;
-  if (h->tuned) return;
+// The emission's block and chunk sizes by the level's 64-px chunks, where none are pinned.  A chunk is one
+// block's work, and its phases are a chain: with fewer chunks than the device holds blocks (eight of 128
+// threads per SM), smaller chunks or wider blocks put the idle warps to work; with enough of them the extra
+// staging only costs issue slots.  Measured per iteration from set_params on (us; 128/64, 128/32, 256/64,
+// 256/32 threads/px): 120 chunks 50.7, 49.1, 47.3, 45.7; 200 chunks 53.2, 49.4, 50.2, 54.5; 300 chunks 53.2,
+// 52.1, 51.2, 57.4; 400 chunks (of 320 segments) 71.6, 55.5, 61.4, 60.8; 500 chunks 59.5, 64.7, 59.5, 67.1;
+// 700 chunks 73.3, 78.5, 78.5, 82.6; 1000 chunks 78.8, 90.6, 83.9, 94.6; 5000 chunks 367, 413, 401, 516.
+static EmissionPin emission_rule(const collage_s* h, int level) {
+  const int chunks = h->lv_chunks[level];
   const bool small = chunks <= 3 * h->sms;
-  h->d.chunk_tiles = (small ? kChunkPx / 2 : kChunkPx) / h->d.tile;
-  h->d.emit_threads = chunks <= h->sms || (!small && chunks <= 4 * h->sms) ? 256 : 128;
+  EmissionPin e;
+  e.threads = chunks <= h->sms || (!small && chunks <= 4 * h->sms) ? 256 : 128;
+  e.chunk_px = small ? kChunkPx / 2 : kChunkPx;
+  return e;
+}
+static void choose_emission(collage_t h, int level) {
+  h->d.few_chunks = h->lv_chunks[level] <= 8 * h->sms;
+  const EmissionPin e = h->pin.at(level) ? h->pin : emission_rule(h, level);
+  h->d.emit_threads = e.threads;
+  h->d.chunk_tiles = e.chunk_px / h->d.tile;
 }
 
 // Pairs that binning the current params at the selected level produces, and its 64-px chunks: the
@@ -585,7 +600,7 @@ static collage_status setup_level(collage_t h, int level) {
   if (st) return st;
   st = ensure_pairs(h, with_slack(need));
   if (st) return st;
-  choose_emission(h, h->lv_chunks[level]);
+  choose_emission(h, level);
   set_grids(h);
   h->level = level;
   return COLLAGE_OK;
@@ -1145,7 +1160,7 @@ static cudaError_t capture_schedule(collage_t h, int start, cudaStream_t s) {
   int target = 0;
   for (int l = start; l < o.n_levels && e == cudaSuccess; ++l) {
     if (apply_level(h, l) != COLLAGE_OK) return cudaErrorInvalidValue;  // tables exist: host only
-    choose_emission(h, h->lv_chunks[l]);
+    choose_emission(h, l);
     set_grids(h);
     const Dev& d = h->d;
     target += o.level_iters[l];
@@ -1223,7 +1238,7 @@ static collage_status build_schedule(collage_t h, int start) {
   const cudaError_t e = capture_schedule(h, start, s);
   const cudaError_t e2 = cudaStreamEndCapture(s, &g);
   st = apply_level(h, cur);  // the current level's view again
-  choose_emission(h, h->lv_chunks[cur]);
+  choose_emission(h, cur);
   set_grids(h);
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -1285,7 +1300,7 @@ extern "C" collage_status collage_run_schedule(collage_t h, void* stream) {
   if (done == total && !(h->h_ctl[0] & (kStatusVoid | kStatusInternal))) {
     st = apply_level(h, L - 1);
     if (st) return st;
-    choose_emission(h, h->lv_chunks[L - 1]);
+    choose_emission(h, L - 1);
     set_grids(h);
     h->level = L - 1;
     return check_and_grow(h, s, &over);  // grows the pair buffers if the last level used > 3/4
@@ -1550,20 +1565,43 @@ struct L2Evict {
 };
 }  // namespace
 
-// Applies a choice (tile change: new level tables and pair buffers).
-static collage_status apply_choice(collage_t h, const TuneChoice& c) {
+// Applies a choice (tile change: new level tables and pair buffers), its emission shape at `level` (or
+// EmissionPin::kEvery level, or none: the rule's shape).
+static collage_status apply_choice(collage_t h, const TuneChoice& c, int level) {
   const bool retile = c.tile != h->d.tile;
-  h->tuned = true;
+  h->pin = EmissionPin{level, c.emit_threads, c.chunk_px};
   h->d.tile = c.tile;
   h->opt.tile = c.tile;
-  h->d.emit_threads = c.emit_threads;
-  h->d.chunk_tiles = std::max(1, c.chunk_px / c.tile);
   h->fwd_mult = c.fwd;
   h->bwd_mult = c.bwd;
   h->comp_mult = c.comp;
   drop_graph(h);
   if (retile) return setup_level(h, h->level);
+  choose_emission(h, h->level);
   set_grids(h);
+  return COLLAGE_OK;
+}
+
+// The configuration to return to when a call fails.
+struct TuneBefore {
+  TuneChoice choice;
+  EmissionPin pin;
+  explicit TuneBefore(const collage_s* h)
+      : choice{h->d.tile, h->d.emit_threads, h->d.chunk_tiles * h->d.tile, h->fwd_mult, h->bwd_mult, h->comp_mult},
+        pin(h->pin) {}
+  void restore(collage_t h) const {
+    apply_choice(h, choice, EmissionPin::kEvery);
+    h->pin = pin;
+  }
+};
+
+// A search's choice: its emission shape holds at the level it was timed at, and only if it is not the one
+// that the level's work asks for anyway (then every level keeps following its own).
+static collage_status apply_search(collage_t h, const TuneChoice& c) {
+  collage_status st = apply_choice(h, c, h->level);
+  if (st) return st;
+  const EmissionPin rule = emission_rule(h, h->level);
+  if (rule.threads == c.emit_threads && rule.chunk_px == c.chunk_px) h->pin.level = EmissionPin::kNone;
   return COLLAGE_OK;
 }
 
@@ -1623,9 +1661,7 @@ static collage_status time_config(collage_t h, cudaStream_t s, int reps, const L
 extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_best_ms) {
   if (!h) return fail(nullptr, COLLAGE_ERR_INVALID_ARG, "handle is NULL");
   cudaStream_t s = (cudaStream_t)stream;
-  const TuneChoice before{h->d.tile, h->d.emit_threads, h->d.chunk_tiles * h->d.tile, h->fwd_mult,
-                          h->bwd_mult, h->comp_mult};
-  const bool was_tuned = h->tuned;
+  const TuneBefore before(h);
   // the key: pixels of the level, elements, and the pair density at 8-px tiles (half-octaves)
   long long pix = 0;
   for (int p = 0; p < h->P; ++p) pix += (long long)h->res[p] * h->res[p];
@@ -1645,11 +1681,13 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
-      collage_status st = apply_choice(h, it->second);
-      if (st) return st;
       float ms = 0.0f;
-      st = time_config(h, s, 10, ev2, &ms);
-      if (st) return st;
+      collage_status st = apply_search(h, it->second);
+      if (!st) st = time_config(h, s, 10, ev2, &ms);
+      if (st) {
+        before.restore(h);
+        return st;
+      }
       h->tuning.tile = it->second.tile;
       h->tuning.emit_threads = it->second.emit_threads;
       h->tuning.chunk_px = it->second.chunk_px;
@@ -1667,18 +1705,21 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
   int trials = 0;
   TuneChoice best{16, 128, kChunkPx, 1.0f, 1.0f, 1.0f};
   float best_ms = 1e30f, default_ms = 0.0f;
-  auto trial = [&](const TuneChoice& c, float* out) -> collage_status {
-    collage_status st = apply_choice(h, c);
+  auto trial = [&](const TuneChoice& c, float* out, int pin) -> collage_status {
+    collage_status st = apply_choice(h, c, pin);
     if (!st) st = time_config(h, s, reps, ev2, out);
     ++trials;
     return st;
   };
   collage_status st = COLLAGE_OK;
-  // the tile first (the defaults of everything else), then each launch parameter in turn
+  // the tile first (everything else as an untuned handle has it, the emission's shape by the level's work
+  // included), then each launch parameter in turn
   for (int T : {16, 8}) {
     float ms = 0.0f;
-    const TuneChoice c{T, 128, kChunkPx, 1.0f, 1.0f, 1.0f};
-    if ((st = trial(c, &ms))) break;
+    TuneChoice c{T, 128, kChunkPx, 1.0f, 1.0f, 1.0f};
+    if ((st = trial(c, &ms, EmissionPin::kNone))) break;
+    c.emit_threads = h->d.emit_threads;
+    c.chunk_px = h->d.chunk_tiles * T;
     if (T == 16) default_ms = ms;
     if (ms < best_ms) {
       best_ms = ms;
@@ -1688,7 +1729,7 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
   const float mults[3] = {0.5f, 1.0f, 2.0f};
   for (int dim = 0; dim < 5 && !st; ++dim) {
     const TuneChoice base = best;
-    for (int k = 0; k < (dim <= 1 ? 2 : 3) && !st; ++k) {
+    for (int k = 0; k < (dim <= 1 ? 2 : 3); ++k) {
       TuneChoice c = base;
       if (dim == 0) c.emit_threads = k == 0 ? 128 : 256;
       if (dim == 1) c.chunk_px = k == 0 ? kChunkPx : kChunkPx / 2;
@@ -1697,7 +1738,7 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
       if (dim == 4) c.comp = mults[k];
       if (std::memcmp(&c, &base, sizeof(c)) == 0) continue;
       float ms = 0.0f;
-      if ((st = trial(c, &ms))) break;
+      if ((st = trial(c, &ms, EmissionPin::kEvery))) break;
       if (ms < best_ms * 0.97f) {  // a change of launch parameter has to win clearly (3%:
         // smaller gains on the one-iteration graph do not carry to the whole step)
         best_ms = ms;
@@ -1705,13 +1746,11 @@ extern "C" collage_status collage_autotune(collage_t h, void* stream, float* h_b
       }
     }
   }
+  if (!st) st = apply_search(h, best);
   if (st) {  // leave the handle as it was
-    apply_choice(h, before);
-    h->tuned = was_tuned;
+    before.restore(h);
     return st;
   }
-  st = apply_choice(h, best);
-  if (st) return st;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune_cache[key] = best;
@@ -1751,14 +1790,11 @@ extern "C" collage_status collage_set_tuning(collage_t h, void* stream, const co
       !grid_ok(c->bwd_grid) || !grid_ok(c->comp_grid))
     return fail(h, COLLAGE_ERR_INVALID_ARG, "tuning outside the searched values");
   CK(h, cudaDeviceSynchronize());
-  const TuneChoice before{h->d.tile, h->d.emit_threads, h->d.chunk_tiles * h->d.tile, h->fwd_mult,
-                          h->bwd_mult, h->comp_mult};
-  const bool was_tuned = h->tuned;
+  const TuneBefore before(h);
   const TuneChoice want{c->tile, c->emit_threads, c->chunk_px, c->fwd_grid, c->bwd_grid, c->comp_grid};
-  collage_status st = apply_choice(h, want);
+  collage_status st = apply_choice(h, want, EmissionPin::kEvery);
   if (st) {
-    apply_choice(h, before);
-    h->tuned = was_tuned;
+    before.restore(h);
     return st;
   }
   h->tuning = collage_tuning{};
