@@ -1011,7 +1011,7 @@ extern "C" collage_status collage_create(const collage_problem* probs, int n_pro
   CKC(dmalloc(h->owned, h->grad_out, 4 * (size_t)h->N));
   CKC(dmalloc(h->owned, d.loss_terms, 5 * h->P));
   CKC(cudaMemset(d.loss_terms, 0, sizeof(float) * 5 * h->P));
-  CKC(dmalloc(h->owned, d.loss_part, (size_t)h->P * kLossParts));
+  CKC(dmalloc(h->owned, d.loss_part, 4 * (size_t)h->P * kLossParts));
   CKC(dmalloc(h->owned, d.loss_done, h->P));
   CKC(cudaMemset(d.loss_done, 0, sizeof(int) * h->P));
   CKC(dmalloc(h->owned, d.paths, 4));

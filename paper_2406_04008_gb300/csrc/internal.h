@@ -144,7 +144,7 @@ struct Dev {
                                 //   they end, which FP32 sums showed in their last bits
   float4* partial;              // [cap * units per tile] deterministic gradient partials, by slot
   float* loss_terms;            // [P*5]
-  float4* loss_part;            // [P * kLossParts] the sums over each part of a problem's loss partials
+  float2* loss_part;            // [P * kLossParts * 4] the four sums over each part of a problem's loss partials, (hi, lo)
   int* loss_done;               // [P] parts summed so far (the last one zeroes it)
   int* status;                  // [1]
   int* step;                    // [1] Adam step count (the last gradient kernel advances it)

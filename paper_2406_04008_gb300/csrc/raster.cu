@@ -772,9 +772,8 @@ __device__ __forceinline__ float warp_sum_f(float x) {
 }
 // Loss of one problem (Eq. 8) in parts of kLossUnits units or more, by its own size alone, so that it has the
 // same bits in any batch: fixed-order float sums of a part's partials (eight strided accumulators per thread,
-// then a shuffle tree within and across warps), and the block that ends last adds the parts in order.  Float
-// throughout: FP64 arithmetic is slow on this part and 1e-7 relative is ample for a sum of non-negative
-// partials.  A block reads 1024 units in a round trip, and one block for the 16384 of a 1024^2 image ended 4 to 7
+// then a shuffle tree within a warp; the sums over warps and parts, the means and the weighted total in float
+// pairs), and the block that ends last adds the parts in order.  No FP64, which is slow on this part.  A block reads 1024 units in a round trip, and one block for the 16384 of a 1024^2 image ended 4 to 7
 // us after the adjoint's others; in parts, summed before the predecessor has completed where that is the
 // distribution term's adjoint, an iteration of 100 outlines at 1000^2 takes 56.4 us instead of 61.9, of 64
 // outline fits at 256^2 96.5 instead of 99.3, of 5000 elements at 2048^2 370 instead of 373.
@@ -785,6 +784,9 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
   const int units = d.tile * d.tile / 64;
   int t0 = d.prob_tile_base[p] * units, t1 = d.prob_tile_base[p + 1] * units;
   const int parts = min(max((t1 - t0) / kLossUnits, 1), kLossParts);
+  const float side = (float)d.prob_res[p];
+  float np_lo;  // pixels: np + np_lo
+  const float np = two_prod(side, side, np_lo), inv_np = div_normal(1.0f, np);
   if (wait) pdl_enter();  // the place is the level's: read before the predecessor has completed
   if (part >= parts) return false;
   if (parts > 1) {
@@ -824,33 +826,44 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
     s_red[3][w] = su;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float r[4];
-    for (int k = 0; k < 4; ++k) r[k] = (s_red[k][0] + s_red[k][1]) + (s_red[k][2] + s_red[k][3]);
+  if (w == 0) {  // from here on in float pairs, a sum on each of lanes 0..3, so that each term is rounded once
+    const int lane = threadIdx.x & 31, k = lane & 3;
+    FloatPair r{s_red[k][0], 0.0f};
+    for (int i = 1; i < kPairWarps; ++i) r.add(s_red[k][i]);
     if (parts > 1) {
-      float4* sums = d.loss_part + (size_t)p * kLossParts;
-      __stcg(&sums[part], make_float4(r[0], r[1], r[2], r[3]));
+      float2* sums = d.loss_part + 4 * (size_t)p * kLossParts;
+      if (lane < 4) __stcg(&sums[4 * part + k], make_float2(r.hi, r.lo));
       __threadfence();
-      if (atomicAdd(&d.loss_done[p], 1) != parts - 1) return true;
+      __syncwarp();
+      int done = 0;
+      if (lane == 0) done = atomicAdd(&d.loss_done[p], 1);
+      if (__shfl_sync(0xffffffffu, done, 0) != parts - 1) return true;
       __threadfence();
-      d.loss_done[p] = 0;
-      r[0] = r[1] = r[2] = r[3] = 0.0f;
-      for (int k = 0; k < parts; ++k) {
-        const float4 v = __ldcg(&sums[k]);
-        r[0] += v.x;
-        r[1] += v.y;
-        r[2] += v.z;
-        r[3] += v.w;
+      if (lane == 0) d.loss_done[p] = 0;
+      r = {0.0f, 0.0f};
+#pragma unroll 1  // (the kernel's code, fetched anew by each block, is what a small problem waits for)
+      for (int i = 0; i < parts; ++i) {
+        const float2 v = __ldcg(&sums[4 * i + k]);
+        r.add(v.x);
+        r.lo += v.y;
       }
     }
-    const float np = (float)d.prob_res[p] * (float)d.prob_res[p];
-    const float Lc = r[0] / np, Lo = r[1] / np, Ld = r[2] / np;
+    FloatPair m = r;
+    if (k != 3) {  // the mean over the pixels
+      m.hi = r.hi * inv_np;
+      m.lo = (fmaf(-m.hi, np, r.hi) + fmaf(-m.hi, np_lo, r.lo)) * inv_np;
+    }
+    FloatPair L{0.0f, 0.0f};  // the weighted total
+    L.add_product(k == 0 ? d.L.alpha : k == 1 ? d.L.beta : k == 2 ? d.L.delta : d.L.gamma, m);
+#pragma unroll
+    for (int o = 1; o <= 2; o *= 2) {
+      const float hi = __shfl_xor_sync(0xffffffffu, L.hi, o), lo = __shfl_xor_sync(0xffffffffu, L.lo, o);
+      L.add(hi);
+      L.lo += lo;
+    }
     float* out = d.loss_terms + 5 * p;
-    out[0] = Lc;
-    out[1] = Lo;
-    out[2] = r[3];
-    out[3] = Ld;
-    out[4] = d.L.alpha * Lc + d.L.beta * Lo + d.L.gamma * r[3] + d.L.delta * Ld;
+    if (lane < 4) out[k ^ (k >> 1)] = m.value();  // containment, overlap, distribution, force
+    if (lane == 0) out[4] = L.value();
   }
   return parts > 1;
 }

@@ -8,27 +8,10 @@
 #pragma once
 #include <cmath>
 
+#include "arith.h"
 #include "internal.h"
 
 namespace collage {
-
-// Sum a + b as hi + lo, exactly (Knuth); the second form needs |a| >= |b| or a = 0 (Dekker).
-__device__ __forceinline__ float two_sum(float a, float b, float& lo) {
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  lo = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return s;
-}
-__device__ __forceinline__ float fast_two_sum(float a, float b, float& lo) {
-  const float s = __fadd_rn(a, b);
-  lo = __fsub_rn(b, __fsub_rn(s, a));
-  return s;
-}
-// Product a b as hi + lo, exactly (FMA).
-__device__ __forceinline__ float two_prod(float a, float b, float& lo) {
-  const float p = __fmul_rn(a, b);
-  lo = __fmaf_rn(a, b, -p);
-  return p;
-}
 
 // |z| <= kTrigMax: z = k step + x with the step 2 pi / 4096 in three floats (Cody & Waite 1980), then
 // sin(k + x) = S cos x + C sin x with the tabled S, C of k (three floats each, one quadrant of them),
