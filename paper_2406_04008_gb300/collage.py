@@ -188,7 +188,8 @@ class Collage:
         return {f: getattr(t, f) for f, _ in L.collage_tuning._fields_}
 
     def set_tuning(self, **choice):
-        """Applies a launch configuration (the keys of tuning(); missing ones keep their values)."""
+        """Applies a launch configuration (the keys of tuning(); missing ones keep the values that the
+        current level has), for every level."""
         cur = self.tuning()
         cur.update(choice)
         t = L.collage_tuning(**{f: cur[f] for f, _ in L.collage_tuning._fields_})

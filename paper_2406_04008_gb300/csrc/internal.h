@@ -3,14 +3,15 @@
 // HBM layout, all problems of a handle concatenated:
 //   per element g (SoA):   prob, vertex offset, closed flag, stroke half-width, bin radius,
 //                          params q / Adam m, v (float4), world translation in pixels (hi, lo),
-//                          outline box, tile rectangle, gradient dq
+//                          tile rectangle, first pair slot, gradient dq
 //   per flattened vertex:  local position (unit coords), per-iteration segment record relative to
-//                          the element translation in pixels (float, rounded from double)
-//   per (tile, element) pair, capacity `cap`: element of each pair in emission order and in
-//                          element order, deterministic gradient partials, and per pixel of the
-//                          tile the signed distance + closest segment saved by the forward pass
+//                          the element translation in pixels (float, within an ulp of the exact value)
+//   per (tile, element) pair, capacity `cap`: per pixel of the tile the signed distance + closest
+//                          segment saved by the forward pass, per 64 pixels a deterministic gradient
+//                          partial; the work lists of the emission and the adjoint
 //   per pixel (level):     container coverage, Ihat, prod(1 - tau c^pad), uniform-loss scratch
-//   per tile:              counting-sort count, [begin, end) into the pairs, loss partials
+//   per tile:              its list of pairs (slot, class, element) and its length; per 64 pixels of
+//                          it the loss partials
 #pragma once
 #include <cstdint>
 #include <cstdio>
@@ -84,7 +85,6 @@ struct Dev {
   int tile;                     // raster tile side
   int emit_threads;             // threads per block of the emission / distance kernel (128, 256)
   int chunk_tiles;              // side of the emission's chunks, in tiles (<= kChunkPx / tile)
-  int n_sort_passes;
   // ---- params / optimiser ----
   float4* q;
   float4* m;
@@ -206,9 +206,9 @@ __device__ __forceinline__ bool in_bounds(const Dev& d, bool ok) {
 
 // Adam (bias-corrected, the update torch.optim.Adam performs; it stands in for the plain descent
 // step of Eq. 4) of element g at step t >= 1 with gradient gr, then the clamp of s.
-// An iteration's step is applied lazily: the loss assembly marks it pending, and the next
-// iteration's transform kernel (one block per element, which reads the params first anyway)
-// applies it before forming the geometry; API calls that read or replace params flush it.
+// An iteration's step is applied lazily: the last block of the kernel that completes the gradient marks
+// it pending (mark_step_if_last), and the next iteration's transform kernel (which reads the params
+// first anyway) applies it before forming the geometry; API calls that read or replace params flush it.
 struct AdamScale {
   float step, root2;  // lr / (1 - b1^t), sqrt(1 - b2^t)
 };
