@@ -1810,6 +1810,7 @@ extern "C" collage_status collage_mat_init(collage_t h, void* stream, int* d_axi
   // each), the elements' placed marks, candidate counts
   const size_t need = 4 * up(4 * np) + up(sizeof(int) * (size_t)h->N) + up(sizeof(int) * (size_t)h->P);
   if (need > h->mat_bytes) {
+    CK(h, prepare_mat_init());
     CK(h, cudaDeviceSynchronize());
     if (h->mat_buf) cudaFree(h->mat_buf);
     h->mat_buf = nullptr;

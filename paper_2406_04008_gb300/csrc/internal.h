@@ -364,7 +364,9 @@ cudaError_t launch_adam_flush(const Dev& d, cudaStream_t s, float* out = nullptr
 // takes an Adam step on ctrl at step *d.step and flattens again (vertices and bin radii); mode 2
 // only flattens
 cudaError_t launch_ctrl_step(const Dev& d, cudaStream_t s, int mode);
-// skeleton-based initialisation: distance transform, medial axis, greedy placement into d.q
+// skeleton-based initialisation: distance transform, medial axis, greedy placement into d.q (after
+// prepare_mat_init, once per handle: the placement's shared-memory limits)
+cudaError_t prepare_mat_init();
 cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
                             unsigned* cand, int* n_cand, float* clear, int* placed, int* axis_out,
                             float* width_out);

@@ -332,7 +332,7 @@ __device__ void place_steps(const Dev& d, int p, int nc, int ne, unsigned long l
 }
 
 // Whether the keys and nc candidates of a problem of ne elements fit one block's shared memory and lanes.
-__device__ __forceinline__ bool place_fits(int nc, int ne, int smem, int* n_keys) {
+__host__ __device__ __forceinline__ bool place_fits(int nc, int ne, int smem, int* n_keys) {
   int nk = 0;  // keys, padded to a power of two
   if (ne <= kPlaceRankMax)
     for (nk = 1; nk < ne;) nk <<= 1;
@@ -492,6 +492,12 @@ __global__ void __cluster_dims__(kPlaceBlocks) __launch_bounds__(kPlaceThreads)
   place<kPlaceBlocks>(d, p, cand, nc, d2, gxy, clear, placed);
 }
 
+cudaError_t prepare_mat_init() {
+  cudaError_t e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(1));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_mat_place_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(kPlaceBlocks));
+}
+
 cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned* g, unsigned* d2,
                             unsigned* cand, int* n_cand, float* clear, int* placed, int* axis_out,
                             float* width_out) {
@@ -499,9 +505,6 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
   const size_t cs = edt_col_smem(max_res), rs = edt_row_smem(max_res);
   if (e == cudaSuccess) e = edt_smem_limit(k_edt_cols<OutsideSite>, cs, edt_col_smem(kEdtMaxRes));
   if (e == cudaSuccess) e = edt_smem_limit(k_mat_rows, rs, edt_row_smem(kEdtMaxRes));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mat_place, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(1));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_mat_place_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, place_smem(kPlaceBlocks));
   if (e != cudaSuccess) return e;
   unsigned short* gcol = reinterpret_cast<unsigned short*>(g);
   k_edt_cols<<<dim3((max_res + kEdtCols - 1) / kEdtCols, d.n_probs), kEdtThreads, cs, s>>>(
@@ -512,7 +515,10 @@ cudaError_t launch_mat_init(const Dev& d, cudaStream_t s, int max_res, unsigned*
   // g is free after the row pass: it holds the candidates' coordinates when they do not fit in
   // shared memory
   k_mat_place<<<d.n_probs, kPlaceThreads, place_smem(1), s>>>(d, cand, n_cand, d2, placed);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  int nk;  // (one block holds every problem's candidates, were all of its pixels on the axis)
+  if ((e = cudaGetLastError()) != cudaSuccess ||
+      (max_res <= 1024 && place_fits(max_res * max_res, kPlaceRankMax, place_smem(1), &nk)))
+    return e;
   return klaunch(d.pdl, k_mat_place_wide, d.n_probs * kPlaceBlocks, kPlaceThreads, place_smem(kPlaceBlocks), s, d, cand,
                  n_cand, d2, g, clear, placed);
 }
