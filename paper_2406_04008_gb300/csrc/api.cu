@@ -656,7 +656,7 @@ static cudaError_t enqueue_iter(collage_t h, cudaStream_t s, int mode, float* ou
   // in step mode the last block of the last gradient kernel marks this iteration's Adam step
   // pending; the next transform (or a flush before params are read) applies it
   const bool mark = mode == kStep;
-  if (bwd) LAUNCH_("k_raster_bwd", launch_raster_bwd(d, s, h->bwd_grid, mark && !d.deterministic));
+  if (bwd) LAUNCH_("k_raster_bwd", launch_raster_bwd(d, s, h->bwd_grid, h->opt.persistent != 0, mark && !d.deterministic));
   MARK_(6);
   if (bwd && d.deterministic) LAUNCH_("k_grad_reduce", launch_grad_reduce(d, s, mark));
   MARK_(7);

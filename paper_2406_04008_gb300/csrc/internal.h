@@ -351,9 +351,9 @@ cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int t
 cudaError_t prepare_dilate(int n_dil);  // sets dynamic shared memory limits (not capturable)
 cudaError_t launch_dilate(const Dev& d, cudaStream_t s, bool backward);
 cudaError_t launch_dtile_flags(const Dev& d, cudaStream_t s);  // once per level, after the container
-// the adjoint and the loss assembly; mark_step: the kernel's last block marks the iteration's Adam step
-// (step mode)
-cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step);
+// the adjoint and the loss assembly; resident: unit_grid is a persistent one, not a block per unit; mark_step:
+// the kernel's last block marks the iteration's Adam step (step mode)
+cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool resident, bool mark_step);
 cudaError_t launch_grad_reduce(const Dev& d, cudaStream_t s, bool mark_step);
 // applies a pending Adam step to all elements and clears the flag (before params are read); then, where
 // given, replaces the params by q_in, copies them to q_out (both 16-byte aligned, [4n]) and gathers them

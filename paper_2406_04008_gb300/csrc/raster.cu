@@ -16,6 +16,7 @@
 // loop, so only one pass over the pixel-segment pairs happens per iteration.  Pixels farther than
 // the coverage margin from the outline carry sd = +-1e30 (saturated coverage, no gradient).
 #include <cfloat>
+#include <type_traits>
 
 #include "arith.h"
 #include "internal.h"
@@ -868,7 +869,8 @@ __device__ bool assemble_loss(const Dev& d, int p, int part, bool wait) {
   return parts > 1;
 }
 
-template <int T, bool FIT>  // FIT: also dL/d(vertex) for outline fitting (d.fit)
+// FIT: also dL/d(vertex) for outline fitting (d.fit).  RES: a grid of resident blocks (else a block per unit slot).
+template <int T, bool FIT, bool RES>
 __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev d, int mark, int early, int n_loss) {
   constexpr int NP = T * T, UNITS = NP / 64, DY = 32 / T;
   if ((int)blockIdx.x < n_loss) {
@@ -893,12 +895,29 @@ __global__ void __launch_bounds__(kPairWarps * 32, FIT ? 7 : 8) k_raster_bwd(Dev
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int stride = ((int)gridDim.x - n_loss) * kPairWarps;
   int i = ((int)blockIdx.x - n_loss) * kPairWarps + wid;
-  if (__ldcg(d.status) & kStatusNoBins) {
+  // the status and the number of listed units (those without a gradient-carrying pixel are not listed): before
+  // the wait from L2, by one thread of a block, and only in a grid of resident blocks.  (The words are the same
+  // for all blocks: read from L2 by every warp of a block per unit slot, 1000 elements at 1024^2 took 148 us an
+  // iteration, 113 after the wait through L1; 30 elements at 64^2 by every warp of 1216 blocks 36.0, 34.9 by one of
+  // each.)
+  int status, live;
+  bool waited = !RES;
+  if (RES) {
+    __shared__ int2 s_head;
+    if (threadIdx.x == 0) s_head = make_int2(__ldcg(d.status), __ldcg(&d.work[1]));
+    __syncthreads();
+    status = s_head.x;
+    live = s_head.y;
+  } else {
     pdl_enter();
+    status = *d.status;
+    live = d.work[1];
+  }
+  if (status & kStatusNoBins) {
+    if (!waited) pdl_enter();
     return;
   }
-  const int n_live = min(__ldcg(&d.work[1]), d.cap * UNITS);  // units without a gradient-carrying pixel are not listed
-  bool waited = false;
+  const int n_live = min(live, d.cap * UNITS);
   auto wait = [&]() {
     if (!waited) pdl_enter();
     waited = true;
@@ -1169,7 +1188,7 @@ cudaError_t launch_raster_fwd(const Dev& d, cudaStream_t s, int pair_grid, int t
   }
 }
 
-cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool mark_step) {
+cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool resident, bool mark_step) {
   // the loss blocks take the place of as many resident ones (at most half of them), so that none waits
   const int units = (int)min((long long)d.max_tiles * (d.tile * d.tile / 64), (long long)kLossUnits * kLossParts);
   // a block for each part of the largest problem, in a sixteenth of the resident blocks: more of them leave
@@ -1178,15 +1197,19 @@ cudaError_t launch_raster_bwd(const Dev& d, cudaStream_t s, int unit_grid, bool 
   const int n_loss = d.n_probs * lb;
   const int grid = max(unit_grid - n_loss, (unit_grid + 1) / 2) + n_loss, mk = mark_step ? 1 : 0;
   const int early = d.L.gamma != 0.0f && d.L.n_dil > 0 ? 1 : 0;  // the predecessor is the distribution adjoint
-  switch (d.tile) {
-    case 8:
-      return klaunch(d.pdl, d.fit ? k_raster_bwd<8, true> : k_raster_bwd<8, false>, grid, kPairWarps * 32, 0, s, d, mk,
-                     early, n_loss);
-    case 16:
-      return klaunch(d.pdl, d.fit ? k_raster_bwd<16, true> : k_raster_bwd<16, false>, grid, kPairWarps * 32, 0, s, d,
-                     mk, early, n_loss);
-    default: return cudaErrorInvalidValue;
-  }
+  if (d.tile != 8 && d.tile != 16) return cudaErrorInvalidValue;
+  auto kernel = [&](auto t, auto fit) {
+    constexpr int T = decltype(t)::value;
+    constexpr bool FIT = decltype(fit)::value;
+    return resident ? k_raster_bwd<T, FIT, true> : k_raster_bwd<T, FIT, false>;
+  };
+  using std::false_type;
+  using std::integral_constant;
+  using std::true_type;
+  const auto k = d.tile == 8 ? d.fit ? kernel(integral_constant<int, 8>{}, true_type{}) : kernel(integral_constant<int, 8>{}, false_type{})
+                 : d.fit     ? kernel(integral_constant<int, 16>{}, true_type{})
+                             : kernel(integral_constant<int, 16>{}, false_type{});
+  return klaunch(d.pdl, k, grid, kPairWarps * 32, 0, s, d, mk, early, n_loss);
 }
 
 cudaError_t launch_container(const Dev& d, cudaStream_t s) {
@@ -1206,7 +1229,7 @@ static void per_sm_t(int emit_threads, RasterOcc* o) {
   int a = 1, b = 1, c = 1;
   if (emit_threads == 256) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_raster_chunks<T, 256>, 256, 0);
   else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_raster_chunks<T, 128>, 128, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_raster_bwd<T, false>, kPairWarps * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_raster_bwd<T, false, true>, kPairWarps * 32, 0);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, k_composite<T, 2>, kCompWarps * 32, 0);
   o->fwd_per_sm = a > 0 ? a : 1;
   o->bwd_per_sm = b > 0 ? b : 1;
